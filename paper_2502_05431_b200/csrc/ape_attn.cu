@@ -151,6 +151,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_smem;
+    pdl_wait();
+    pdl_trigger();
 
     const int n_sib = p.n_sib;
     const int group = blockIdx.x / n_sib, sib = blockIdx.x - group * n_sib;
@@ -822,25 +824,23 @@ cudaError_t attn_set_smem_attr(int D, int mode, size_t smem_bytes) {
 }
 
 template <int D>
-static void launch_mode(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
+static cudaError_t launch_mode(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
                         const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, cudaStream_t stream) {
     switch (p.mode) {
-        case kAttnPrefill: ape_attn_kernel<D, kAttnPrefill><<<n_cta, kThreads, smem_bytes, stream>>>(tm_q, tm_k, tm_v, tm_o, split, p); break;
-        case kAttnEncode:  ape_attn_kernel<D, kAttnEncode><<<n_cta, kThreads, smem_bytes, stream>>>(tm_q, tm_k, tm_v, tm_o, split, p); break;
-        case kAttnAlt:     ape_attn_kernel<D, kAttnAlt><<<n_cta, kThreads, smem_bytes, stream>>>(tm_q, tm_k, tm_v, tm_o, split, p); break;
-        case kAttnStats:   ape_attn_kernel<D, kAttnStats><<<n_cta, kThreads, smem_bytes, stream>>>(tm_q, tm_k, tm_v, tm_o, split, p); break;
-        case kAttnBias:    ape_attn_kernel<D, kAttnBias><<<n_cta, kThreads, smem_bytes, stream>>>(tm_q, tm_k, tm_v, tm_o, split, p); break;
-        default: break;
+        case kAttnPrefill: return launch_pdl(ape_attn_kernel<D, kAttnPrefill>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnEncode:  return launch_pdl(ape_attn_kernel<D, kAttnEncode>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnAlt:     return launch_pdl(ape_attn_kernel<D, kAttnAlt>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnStats:   return launch_pdl(ape_attn_kernel<D, kAttnStats>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnBias:    return launch_pdl(ape_attn_kernel<D, kAttnBias>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
     }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_attn(int D, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
                         const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, cudaStream_t stream)
 {
-    if (p.mode < kAttnPrefill || p.mode > kAttnBias) return cudaErrorInvalidValue;
-    if (D == 128) launch_mode<128>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream);
-    else launch_mode<64>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream);
-    return cudaGetLastError();
+    return D == 128 ? launch_mode<128>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream)
+                    : launch_mode<64>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream);
 }
 
 }  // namespace ape

@@ -68,6 +68,8 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
         mbar_fence_init();
     }
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
 
     const int item_begin = p.cta_item_begin[blockIdx.x], item_end = p.cta_item_begin[blockIdx.x + 1];
 
@@ -292,12 +294,7 @@ int decode_pick_stages(int D, int G, size_t smem_limit) {
 cudaError_t launch_decode(int D, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const DecodeParams& p,
                           int n_cta, size_t smem_bytes, cudaStream_t stream)
 {
-    if (D == 128) {
-        ape_decode_kernel<128><<<n_cta, kThreads, smem_bytes, stream>>>(tm_k, tm_v, p);
-    } else {
-        ape_decode_kernel<64><<<n_cta, kThreads, smem_bytes, stream>>>(tm_k, tm_v, p);
-    }
-    return cudaGetLastError();
+    return launch_pdl(D == 128 ? ape_decode_kernel<128> : ape_decode_kernel<64>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
 }
 
 cudaError_t decode_set_smem_attr(int D, size_t smem_bytes) {

@@ -4,7 +4,7 @@
 //      LSE = logsumexp_s(m_s + log2 l_s),  O = sum_s 2^(LSE_s - LSE) O_s;
 //   2. the context log-sum-exp is multiplied by the scaling factor S and the two segments are merged by a
 //      softmax over [S * LSE_C, LSE_other] (Eq. 5; appendix "Efficient Implementation").
-// One warp per output row (query token, query head); lanes cover the head dimension.
+// One or eight warps per output row (query token, query head); lanes cover the head dimension.
 #include "ape_common.cuh"
 #include "ape_kernels.h"
 
@@ -181,62 +181,22 @@ __device__ __forceinline__ void combine_tree(const MergeParams& p, const DevMerg
     lse = (Z[0] > 0.f) ? top[0] + fast_log2(Z[0]) : -INFINITY;
 }
 
+// The end of Eq. 5 for one row, in base-2 units: lse_c already carries S; the segments' sums of weights (norm_*) and of weighted
+// values (ac, ao) still carry their own normalisers.
 template <int VEC>
-__global__ void __launch_bounds__(256) ape_merge_kernel(const MergeParams p)
+__device__ __forceinline__ void write_row(const MergeParams& p, int64_t out_row, int h, int lane, float lse_c, float norm_c,
+                                          const float (&ac)[VEC], float lse_o, float norm_o, const float (&ao)[VEC])
 {
-    const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int group = warp_global / p.rows_per_slot;
-    const int row = warp_global - group * p.rows_per_slot;
-    if (group >= p.n_groups) return;
-    const DevMerge g = p.groups[group];
-    const DevReq rq = p.reqs[g.req];
-    const int tok = g.row_block * p.tokens_per_block + row / p.G;     // query row inside the request
-    const int hg = row % p.G;
-    if (tok >= rq.q_len) return;
-
-    float Mc, Lc, Mo, Lo, ac[VEC], ao[VEC];
-    float lse_c;
-    if (p.per_context == 2) {
-        combine_tree<VEC>(p, g, row, lane, lse_c, Lc, ac);             // Lc: the normaliser of ac
-    } else if (p.per_context == 1) {
-        combine_per_context<VEC>(p, g, row, lane, lse_c, Lc, ac);      // Lc: the normaliser of ac
-    } else {
-        combine_segment<VEC>(p.ws_o_ctx, p.ws_ml_ctx, g.ctx_slot0, g.ctx_n, g.ctx_stride, p.rows_per_slot_ctx, row + g.ctx_row_off,
-                             p.D, lane, Mc, Lc, ac);
-        // base-2 log-sum-exp of the context segment, multiplied by S (Eq. 5: Z_C^S)
-        lse_c = (Lc > 0.f) ? p.S * (Mc + fast_log2(Lc)) : -INFINITY;
-    }
-    combine_segment<VEC>(p.ws_o, p.ws_ml, g.oth_slot0, g.oth_n, g.slot_stride, p.rows_per_slot, row, p.D, lane, Mo, Lo, ao);
-
-    const int h = g.kv_head * p.G + hg;
-    if (p.part_o_ctx != nullptr) {
-        // one shard of a context-sharded attend: hand out the two segments as they are (Eq. 5 form only)
-        const int64_t rh = static_cast<int64_t>(rq.q_row0 + tok) * p.H_q + h;
-        const float ic = (Lc > 0.f) ? 1.f / Lc : 0.f, io = (Lo > 0.f) ? 1.f / Lo : 0.f;
-        #pragma unroll
-        for (int v = 0; v < VEC; ++v) {
-            p.part_o_ctx[rh * p.D + lane * VEC + v] = ac[v] * ic;
-            p.part_o_oth[rh * p.D + lane * VEC + v] = ao[v] * io;
-        }
-        if (lane == 0) {
-            p.part_lse_ctx[rh] = (Lc > 0.f) ? (Mc + fast_log2(Lc)) * kLn2 : -INFINITY;
-            p.part_lse_oth[rh] = (Lo > 0.f) ? (Mo + fast_log2(Lo)) * kLn2 : -INFINITY;
-        }
-        return;
-    }
-    const float lse_o = (Lo > 0.f) ? (Mo + fast_log2(Lo)) : -INFINITY;
     const float top = fmaxf(lse_c, lse_o);
     float wc = 0.f, wo = 0.f, lam = -INFINITY;
     if (top > -INFINITY) {
         const float ec = fast_exp2(lse_c - top), eo = fast_exp2(lse_o - top);
         const float inv = 1.f / (ec + eo);
-        wc = (Lc > 0.f) ? ec * inv / Lc : 0.f;        // weight of the context segment over its own normaliser
-        wo = (Lo > 0.f) ? eo * inv / Lo : 0.f;
+        wc = (norm_c > 0.f) ? ec * inv / norm_c : 0.f;        // weight of the context segment over its own normaliser
+        wo = (norm_o > 0.f) ? eo * inv / norm_o : 0.f;
         lam = (top + fast_log2(ec + eo)) * kLn2;
     }
-    __nv_bfloat16* dst = p.out.data + static_cast<int64_t>(rq.q_row0 + tok) * p.out.token_stride
-                         + static_cast<int64_t>(h) * p.out.head_stride + lane * VEC;
+    __nv_bfloat16* dst = p.out.data + out_row * p.out.token_stride + static_cast<int64_t>(h) * p.out.head_stride + lane * VEC;
     float r[VEC];
     #pragma unroll
     for (int v = 0; v < VEC; ++v) r[v] = wc * ac[v] + wo * ao[v];
@@ -246,8 +206,168 @@ __global__ void __launch_bounds__(256) ape_merge_kernel(const MergeParams p)
     } else {
         *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(r[0], r[1]);
     }
-    if (p.lse_out != nullptr && lane == 0)
-        p.lse_out[static_cast<int64_t>(rq.q_row0 + tok) * p.H_q + h] = lam;
+    if (p.lse_out != nullptr && lane == 0) p.lse_out[out_row * p.H_q + h] = lam;
+}
+
+// Eq. 5 form.  W warps (1 or 8) of a block share a row's partials and meet in shared memory.  The kernel is bound by the latency of its
+// loads (records -> (m, l) -> rows of O~), so it is built to have many of them in flight: a lane per partial fetches all (m, l)
+// of a row at once, the rows of the first kBatch partials are requested together with them, and few registers per thread
+// leave room for many warps (127 before, which left 16 warps per SM: 4 x 128 rows over 20K tokens, 27 MB of partials, 30 us).
+// The weights 2^(m - M) are then one exponential per lane, and folding a partial is VEC multiply-adds.
+template <int VEC, int W>
+__global__ void __launch_bounds__(256, 4) ape_merge_kernel(const MergeParams p)
+{
+    constexpr int kBatch = 4;
+    constexpr int D = VEC * 32;
+    __shared__ float s_acc[W > 1 ? 8 : 1][2][W > 1 ? D : 1];
+    __shared__ float s_ml[8][2][2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int part = warp % W;
+    const int row_global = blockIdx.x * (8 / W) + warp / W;
+    const int group = row_global / p.rows_per_slot;
+    const int row = row_global - group * p.rows_per_slot;
+    bool live = group < p.n_groups;
+    DevMerge g{};
+    DevReq rq{};
+    if (live) { g = p.groups[group]; rq = p.reqs[g.req]; }
+    const int tok = g.row_block * p.tokens_per_block + row / p.G;     // query row inside the request
+    live = live && tok < rq.q_len;
+    pdl_wait();
+    pdl_trigger();
+
+    float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f}, acc[2][VEC];      // context, other
+    #pragma unroll
+    for (int v = 0; v < VEC; ++v) acc[0][v] = acc[1][v] = 0.f;
+    if (live) {
+        #pragma unroll
+        for (int seg = 0; seg < 2; ++seg) {
+            const float* ws_o = seg ? p.ws_o : p.ws_o_ctx;
+            const float* ws_ml = seg ? p.ws_ml : p.ws_ml_ctx;
+            const int n = seg ? g.oth_n : g.ctx_n, stride = seg ? g.slot_stride : g.ctx_stride;
+            const int per_slot = seg ? p.rows_per_slot : p.rows_per_slot_ctx;
+            const size_t row0 = static_cast<size_t>(seg ? g.oth_slot0 : g.ctx_slot0) * per_slot + row + (seg ? 0 : g.ctx_row_off);
+            const size_t step = static_cast<size_t>(stride) * per_slot;        // rows between consecutive partials
+            #pragma unroll 1
+            for (int i0 = part; i0 < n; i0 += 32 * W) {
+                const int mine = i0 + lane * W;                                // this lane's partial
+                float2 ml = make_float2(-INFINITY, 0.f);
+                if (mine < n) ml = *reinterpret_cast<const float2*>(ws_ml + (row0 + mine * step) * 2);
+                const int cnt = min(32, (n - i0 + W - 1) / W);
+                const float* src = ws_o + (row0 + i0 * step) * D + lane * VEC;
+                const size_t src_step = static_cast<size_t>(W) * step * D;
+                auto load = [&](int j, float (&x)[VEC]) {
+                    const float* a = src + j * src_step;
+                    if constexpr (VEC == 4) { const float4 t = *reinterpret_cast<const float4*>(a); x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w; }
+                    else { const float2 t = *reinterpret_cast<const float2*>(a); x[0] = t.x; x[1] = t.y; }
+                };
+                float x[kBatch][VEC];
+                // Requested together with (m, l): the row of an empty partial was never written, but it lies inside the
+                // workspace, and the fold below never looks at what was read from it.
+                #pragma unroll
+                for (int u = 0; u < kBatch; ++u) if (u < cnt) load(u, x[u]);
+                if (!(ml.y > 0.f)) ml = make_float2(-INFINITY, 0.f);           // empty partial
+                float top = fmaxf(M[seg], ml.x);
+                #pragma unroll
+                for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+                const float base = (top == -INFINITY) ? 0.f : top;
+                const float f = (ml.y > 0.f) ? fast_exp2(ml.x - base) : 0.f, f_old = fast_exp2(M[seg] - base);
+                float sum = ml.y * f;
+                #pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                L[seg] = L[seg] * f_old + sum;
+                M[seg] = top;
+                #pragma unroll
+                for (int v = 0; v < VEC; ++v) acc[seg][v] *= f_old;
+                #pragma unroll 1
+                for (int j0 = 0; j0 < cnt; j0 += kBatch) {
+                    if (j0 > 0) {
+                        #pragma unroll
+                        for (int u = 0; u < kBatch; ++u) if (j0 + u < cnt) load(j0 + u, x[u]);
+                    }
+                    #pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const float fj = __shfl_sync(0xffffffffu, f, (j0 + u) & 31);
+                        if (j0 + u >= cnt || fj == 0.f) continue;
+                        #pragma unroll
+                        for (int v = 0; v < VEC; ++v) acc[seg][v] += x[u][v] * fj;
+                    }
+                }
+            }
+        }
+    }
+    if constexpr (W > 1) {
+        #pragma unroll
+        for (int seg = 0; seg < 2; ++seg) {
+            #pragma unroll
+            for (int v = 0; v < VEC; ++v) s_acc[warp][seg][lane * VEC + v] = acc[seg][v];
+            if (lane == 0) { s_ml[warp][seg][0] = M[seg]; s_ml[warp][seg][1] = L[seg]; }
+        }
+        __syncthreads();
+        if (part != 0) return;
+        #pragma unroll
+        for (int seg = 0; seg < 2; ++seg) {
+            float top = -INFINITY;
+            #pragma unroll
+            for (int k = 0; k < W; ++k) top = fmaxf(top, s_ml[warp + k][seg][0]);
+            const float base = (top == -INFINITY) ? 0.f : top;
+            float sum = 0.f;
+            #pragma unroll
+            for (int v = 0; v < VEC; ++v) acc[seg][v] = 0.f;
+            #pragma unroll
+            for (int k = 0; k < W; ++k) {
+                const float f = fast_exp2(s_ml[warp + k][seg][0] - base);
+                sum += s_ml[warp + k][seg][1] * f;
+                #pragma unroll
+                for (int v = 0; v < VEC; ++v) acc[seg][v] += s_acc[warp + k][seg][lane * VEC + v] * f;
+            }
+            M[seg] = top; L[seg] = sum;
+        }
+    }
+    if (!live) return;
+    const int h = g.kv_head * p.G + row % p.G;
+    if (p.part_o_ctx != nullptr) {
+        // one shard of a context-sharded attend: hand out the two segments as they are
+        const int64_t rh = static_cast<int64_t>(rq.q_row0 + tok) * p.H_q + h;
+        const float ic = (L[0] > 0.f) ? 1.f / L[0] : 0.f, io = (L[1] > 0.f) ? 1.f / L[1] : 0.f;
+        #pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            p.part_o_ctx[rh * D + lane * VEC + v] = acc[0][v] * ic;
+            p.part_o_oth[rh * D + lane * VEC + v] = acc[1][v] * io;
+        }
+        if (lane == 0) {
+            p.part_lse_ctx[rh] = (L[0] > 0.f) ? (M[0] + fast_log2(L[0])) * kLn2 : -INFINITY;
+            p.part_lse_oth[rh] = (L[1] > 0.f) ? (M[1] + fast_log2(L[1])) * kLn2 : -INFINITY;
+        }
+        return;
+    }
+    // base-2 log-sum-exp of the context segment, multiplied by S (Eq. 5: Z_C^S)
+    const float lse_c = (L[0] > 0.f) ? p.S * (M[0] + fast_log2(L[0])) : -INFINITY;
+    const float lse_o = (L[1] > 0.f) ? (M[1] + fast_log2(L[1])) : -INFINITY;
+    write_row<VEC>(p, rq.q_row0 + tok, h, lane, lse_c, L[0], acc[0], lse_o, L[1], acc[1]);
+}
+
+// Decode plans of the per-context form and of context trees: one warp per output row walks the partials in order.
+template <int VEC, bool TREE>
+__global__ void __launch_bounds__(256) ape_merge_nodes_kernel(const MergeParams p)
+{
+    const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int group = warp_global / p.rows_per_slot;
+    const int row = warp_global - group * p.rows_per_slot;
+    pdl_wait();
+    pdl_trigger();
+    if (group >= p.n_groups) return;
+    const DevMerge g = p.groups[group];
+    const DevReq rq = p.reqs[g.req];
+    const int tok = g.row_block * p.tokens_per_block + row / p.G;     // query row inside the request
+    if (tok >= rq.q_len) return;
+
+    float lse_c, norm_c, ac[VEC], Mo, Lo, ao[VEC];
+    if constexpr (TREE) combine_tree<VEC>(p, g, row, lane, lse_c, norm_c, ac);
+    else combine_per_context<VEC>(p, g, row, lane, lse_c, norm_c, ac);
+    combine_segment<VEC>(p.ws_o, p.ws_ml, g.oth_slot0, g.oth_n, g.slot_stride, p.rows_per_slot, row, p.D, lane, Mo, Lo, ao);
+    const float lse_o = (Lo > 0.f) ? (Mo + fast_log2(Lo)) : -INFINITY;
+    write_row<VEC>(p, rq.q_row0 + tok, g.kv_head * p.G + row % p.G, lane, lse_c, norm_c, ac, lse_o, Lo, ao);
 }
 
 // Shards of a context-sharded attend (each holds a subset of the contexts): LSE_C = log sum_s e^{LSE_s},
@@ -328,6 +448,8 @@ ape_node_bias_kernel(const NodeBiasParams p)
 {
     const int r = blockIdx.y;
     const DevReq rq = p.reqs[r];
+    pdl_wait();
+    pdl_trigger();
     const int64_t local = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (local >= static_cast<int64_t>(rq.q_len) * p.H_q) return;
     const int64_t row = static_cast<int64_t>(rq.pad) * p.H_q + local;
@@ -385,6 +507,8 @@ ape_node_bias_smem_kernel(const NodeBiasParams p)
         const DevNode nd = p.nodes[n0 + i];
         rec[i] = make_int2(nd.parent >= 0 ? nd.parent - n0 : -1, (nd.scaled ? 1 : 0) | (nd.pad ? 2 : 0));
     }
+    pdl_wait();
+    pdl_trigger();
     __syncthreads();
     #pragma unroll 4
     for (int i = warp; i < n_nodes; i += 8) {                // independent loads: several in flight per warp
@@ -426,23 +550,34 @@ cudaError_t launch_node_bias(const NodeBiasParams& p, cudaStream_t stream)
             cudaFuncSetAttribute(ape_node_bias_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
             return cudaGetLastError();
         const dim3 grid(static_cast<unsigned>((p.max_rows + kBiasRows - 1) / kBiasRows), static_cast<unsigned>(p.n_req));
-        ape_node_bias_smem_kernel<<<grid, 256, smem, stream>>>(p);
-        return cudaGetLastError();
+        return launch_pdl(ape_node_bias_smem_kernel, grid, 256, smem, stream, p);
     }
     // too many nodes for shared memory: the per-node arrays stay in global memory
     const dim3 grid(static_cast<unsigned>((p.max_rows + 255) / 256), static_cast<unsigned>(p.n_req));
-    ape_node_bias_kernel<<<grid, 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(ape_node_bias_kernel, grid, 256, 0, stream, p);
 }
+
+namespace {
+template <int VEC>
+cudaError_t launch_merge_vec(const MergeParams& p, long long rows, cudaStream_t stream) {
+    if (p.per_context != 0)
+        return launch_pdl(p.per_context == 2 ? ape_merge_nodes_kernel<VEC, true> : ape_merge_nodes_kernel<VEC, false>,
+                          static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
+    // Eight warps per row while all rows' blocks are resident at once (148 SMs x 4 blocks): with few rows, as in a decode step,
+    // it is the latency of a row's partials that counts (4 requests over 20K tokens each: 62.1 us per step with one warp per row,
+    // 60.5 with eight; 16 requests over shared 128K tokens: 129.0 and 124.4).  With more rows the warps of other rows hide it,
+    // and sharing a row only adds the meeting in shared memory (64 rows over 10 x 256 tokens, 2048 rows to merge: 19.4 us with
+    // one, 24.4 with eight; 4 x 128 rows over 20K tokens: 212 and 254).
+    if (rows <= 4 * 148) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
+    return launch_pdl(ape_merge_kernel<VEC, 1>, static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
+}
+}  // namespace
 
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
 {
-    const long long warps = static_cast<long long>(p.n_groups) * p.rows_per_slot;
-    if (warps == 0) return cudaSuccess;
-    const int blocks = static_cast<int>((warps * 32 + 255) / 256);
-    if (p.D == 128) ape_merge_kernel<4><<<blocks, 256, 0, stream>>>(p);
-    else ape_merge_kernel<2><<<blocks, 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    const long long rows = static_cast<long long>(p.n_groups) * p.rows_per_slot;
+    if (rows == 0) return cudaSuccess;
+    return p.D == 128 ? launch_merge_vec<4>(p, rows, stream) : launch_merge_vec<2>(p, rows, stream);
 }
 
 }  // namespace ape

@@ -1,0 +1,38 @@
+"""Merge of the partials: rows whose partials are shared by eight warps and rows with one, and rows with more partials than one round of
+lanes covers.  The number of partials per row follows the SM budget (one KV head: every thread block leaves one or two)."""
+import pytest
+
+from paper_2502_05431_b200 import libape
+from paper_2502_05431_b200 import workloads as wl
+from tests.gpu_util import compare, gpu_attend, handle, oracle_attend
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(b, mode, **kw):
+    out, lse, _ = gpu_attend(b, mode, **kw)
+    for r, rq in enumerate(b.requests):
+        ref = oracle_attend(b, r)
+        sl = slice(rq.q_start, rq.q_start + rq.q_len)
+        compare(out[sl], ref.out.float(), f"{b.name} req {r}")
+        assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("n_sm", [1, 6, 7, 8, 14, 15, 16, 33, 0])
+@pytest.mark.parametrize("mode,d,l_q", [(libape.APE_DECODE, 128, 1), (libape.APE_PREFILL, 64, 19), (libape.APE_PREFILL, 128, 150)])
+def test_partials_per_row(n_sm, mode, d, l_q):
+    """(4 rows, 256 slot rows: eight warps a row; 768 slot rows: one)"""
+    b = wl.make_batch(H_q=4, H_kv=1, d=d, l_P=70, ctx_lens=[[3000, 1, 2999]], l_q=l_q, l_k=l_q + 40, seed=31, T=0.8, S=0.9,
+                      name=f"merge_sm{n_sm}")
+    handle().set_sm_budget(n_sm)
+    try:
+        _check(b, mode)
+    finally:
+        handle().set_sm_budget(0)
+
+
+def test_more_partials_than_one_round_of_lanes():
+    """One KV head and a shared-context batch of at most 128 rows: two partials per thread block, 296 per row."""
+    b = wl.share_contexts(wl.make_batch(H_q=4, H_kv=1, d=128, l_P=5, ctx_lens=[[40000]] + [[1]] * 2, l_q=1, l_k=9, seed=32,
+                                        T=0.9, S=0.8, name="merge_296"))
+    _check(b, libape.APE_DECODE, shared=True)
