@@ -97,6 +97,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     constexpr int kSlabs = D / 64;
     constexpr int kTileBytes = kSlabs * kSlabBytes;            // one K or V tile, also one Q half
     constexpr int QBUF = (MODE == kAttnEncode) ? 2 : 1;
+    constexpr bool TURNS = MODE != kAttnAlt && MODE != kAttnEncode;   // the halves take turns in the exponential phase
     constexpr bool ALT = MODE == kAttnAlt, STATS = MODE == kAttnStats, BIAS = MODE == kAttnBias;
     constexpr int kQBytes = (ALT ? 1 : 2) * kTileBytes;        // both halves of a row block (ALT: the one half both read)
     constexpr int kNK = ALT ? 3 : 2;                           // K stages
@@ -151,8 +152,6 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_smem;
-    pdl_wait();
-    pdl_trigger();
 
     const int n_sib = p.n_sib;
     const int group = blockIdx.x / n_sib, sib = blockIdx.x - group * n_sib;
@@ -198,6 +197,9 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
         if (lane == 0) {
             tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
+            if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
+            pdl_wait();
+            pdl_trigger();
             uint32_t kcnt = 0, vcnt = 0, q_loads = 0;
             int last_req = -1, last_head = -1, last_rb = -1;
             bool ok = true;
@@ -465,6 +467,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const uint32_t tS = tmem_base + lane_base + (w ? kColS1 : kColS0);
         const uint32_t tO = tmem_base + lane_base + (w ? kColO1 : kColO0);
         const uint32_t my_s_full = bar_s_full + 8 * w, my_p_full = bar_p_full + 32 * w, my_o_full = bar_o_full + 8 * w;
+        if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
+        pdl_wait();                                                 // in front of the first bias read and the first store
         uint32_t scnt = 0, ocnt = 0, q_loads = 0, tcnt = 0;         // tcnt: visible tiles of the CTA so far (either half's)
         int last_req = -1, last_head = -1, last_rb = -1;
         bool ok = true;
@@ -568,8 +572,10 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // The two halves take turns in the exponential phase: the special-function unit is the scarcest pipe, and
                 // alternating keeps one half in its exponentials while the other half's MMAs run.  Phase n of half 0 follows
                 // phase n-1 of half 1; phase n of half 1 follows phase n of half 0 (both halves see the same tiles).
-                // (Alternating halves work on different tiles, with different numbers of them: no turns there.)
-                if (!alt) {
+                // (Alternating halves work on different tiles, with different numbers of them: no turns there.  Encode's items have
+                // one to three tiles, and a turn mostly makes a half wait whose partner is at the end of an item: 500 x 256
+                // tokens 897 us with turns, 865 without; the long items of prefill lose 11% without.)
+                if (TURNS) {
                     const uint32_t n = scnt - 1;
                     bool turn = true;
                     if (w == 0) { if (n > 0) turn = mbar_wait(bar_tok, (n - 1) & 1, &abort_flag, p.status); }
@@ -605,7 +611,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                             sum2[i & 1] = add2(sum2[i & 1], pack2(p0, p1));
                             pk[i] = pack_bf16x2(p0, p1);
                         }
-                        if (qq == 3 && !alt) {                             // exponentials issued: the other half's turn
+                        if (qq == 3 && TURNS) {                             // exponentials issued: the other half's turn
                             __syncwarp();
                             if (lane == 0) mbar_arrive(bar_tok + 8 * (1 - w));
                         }
@@ -718,6 +724,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (QBUF == 2 && lane == 0) {
             tma_prefetch_desc(&tm_q);
             if (o_via_tma) tma_prefetch_desc(&tm_o);
+            if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
+            pdl_wait();
             uint32_t q_loads = 0, staged[2] = {0, 0};
             int last_req = -1, last_head = -1, last_rb = -1;
             bool ok = true;
