@@ -141,8 +141,8 @@ def _pool(k: torch.Tensor, v: torch.Tensor) -> ape_kv_pool_t:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    # (the raw handle of the current stream: building a torch.cuda.Stream object for it costs 3 us of a 10 us call)
+    return int(stream.cuda_stream) if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _request_array(requests: Sequence):
