@@ -34,6 +34,8 @@ constexpr int kRegsSoftmax = 216;            // registers per thread after the h
 constexpr int kRegsOther = 72;               // producer / MMA warpgroup
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
+constexpr int kBarBytes = 512;                // barriers, behind the tiles
+constexpr int kStageBytes = 8 * 4096;         // transposition buffers of the softmax warps, behind the barriers
 constexpr int kSlabBytes = 128 * 128;         // 128 rows x 64 bf16
 constexpr float kRescaleThreshold = 8.0f;     // base-2 units: O is rescaled only when the row maximum grew by more
 constexpr float kLn2 = 0.6931471805599453f;
@@ -79,6 +81,36 @@ __device__ __forceinline__ bool tile_visible(const DevTile& t, const ItemGeom& g
     return true;
 }
 
+// O of a warp's 32 rows, tensor memory -> workspace.  A thread holds a row, so its own stores would touch 32 lines per
+// instruction: the warp turns 32 x 32 blocks in shared memory (16-byte chunk j of row r at j ^ (r mod 8)) and stores whole 128-byte
+// lines (prefill of 64 rows over 10 x 256 tokens, two tiles per block: 18.4 us with stores by row, 17.2 this way).  A function of its
+// own: inlined, its registers disturbed the tile loop (500 x 256 tokens 545 -> 592 us).
+template <int D>
+__device__ __noinline__ void store_rows_f32(uint32_t tO, uint32_t stage, float* dst, int n_rows) {
+    const int lane = threadIdx.x & 31;
+    dst += (lane & 7) * 4;
+    #pragma unroll 1
+    for (int c = 0; c < D / 32; ++c) {
+        uint32_t o[32];
+        tmem_ld32(tO + c * 32, o);
+        tmem_ld_wait();
+        #pragma unroll
+        for (int j = 0; j < 8; ++j)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage + lane * 128 + ((j ^ (lane & 7)) << 4)),
+                         "r"(o[4 * j]), "r"(o[4 * j + 1]), "r"(o[4 * j + 2]), "r"(o[4 * j + 3]) : "memory");
+        __syncwarp();
+        #pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = i * 4 + (lane >> 3);
+            uint4 v;
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                         : "r"(stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) : "memory");
+            if (r < n_rows) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * D + c * 32) = v;
+        }
+        __syncwarp();
+    }
+}
+
 }  // namespace
 
 // QBUF: number of Q buffers.  Plans with long items (prefill) use one Q buffer and two stages each of K and V; plans
@@ -99,6 +131,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     constexpr int QBUF = (MODE == kAttnEncode) ? 2 : 1;
     constexpr bool TURNS = MODE != kAttnAlt && MODE != kAttnEncode;   // the halves take turns in the exponential phase
     constexpr bool ALT = MODE == kAttnAlt, STATS = MODE == kAttnStats, BIAS = MODE == kAttnBias;
+    constexpr bool STAGED = MODE == kAttnPrefill || MODE == kAttnBias;   // partials leave through shared memory (there is room for it)
     constexpr int kQBytes = (ALT ? 1 : 2) * kTileBytes;        // both halves of a row block (ALT: the one half both read)
     constexpr int kNK = ALT ? 3 : 2;                           // K stages
     constexpr int kNV = ALT ? 3 : (QBUF == 2) ? 1 : 2;         // V stages
@@ -113,6 +146,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint8_t* k_smem = q_smem + QBUF * kQBytes;                 // kNK stages
     uint8_t* v_smem = k_smem + kNK * kTileBytes;               // kNV stages
     uint64_t* bars = reinterpret_cast<uint64_t*>(v_smem + kNV * kTileBytes);
+    uint8_t* stage_smem = v_smem + kNV * kTileBytes + kBarBytes;   // STAGED: 4 KB per softmax warp
     // barrier map
     const uint32_t bar0 = smem_u32(bars);
     const uint32_t bar_q_full = bar0, bar_q_empty = bar0 + 16;             // [QBUF] each
@@ -698,6 +732,10 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const size_t row = static_cast<size_t>(item.slot + sib) * kAttnRows + R;
                 if (n_local > 0) {
                     float* dst = p.ws_o + row * D;
+                    if constexpr (STAGED) {
+                        const int n_rows = min(32, (rq.q_len - g.rb * TB) * G - (R - lane));      // live rows of the warp (may be <= 0)
+                        store_rows_f32<D>(tO, smem_u32(stage_smem + warp * 4096), p.ws_o + (row - lane) * D, n_rows);
+                    } else
                     #pragma unroll
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t o[32];
@@ -792,7 +830,7 @@ size_t attn_smem_bytes(int D, int mode) {
     const size_t tile = static_cast<size_t>(D / 64) * kSlabBytes;
     // Q halves + K stages + V stages
     const int tiles = (mode == kAttnAlt) ? (1 + 3 + 3) : (mode == kAttnEncode) ? (4 + 2 + 1) : (2 + 2 + 2);
-    return 1024 + tiles * tile + 512;
+    return 1024 + tiles * tile + kBarBytes + (tiles == 6 ? kStageBytes : 0);
 }
 
 // The register hand-over only works if the registers that the third warpgroup gives up cover what the two softmax
