@@ -64,6 +64,8 @@ struct ape_plan_s {
     // the prefill with per-row, per-node biases): their per-node arrays live behind the partials in the workspace.
     bool two_pass = false;
     int32_t* d_req_node0 = nullptr;  // [n_req + 1]
+    DevBfsNode* d_bfs = nullptr;
+    int32_t* d_levels = nullptr;
     int n_nodes = 0, max_rows = 0, max_nodes = 0;
     int64_t stat_rows = 0;
     size_t off_stats = 0, off_mass = 0, off_bias = 0;
@@ -214,6 +216,8 @@ struct HostMeta {
     std::vector<DevMerge> merge;
     std::vector<DevNode> nodes;      // tree plans; two-pass plans
     std::vector<int32_t> req_node0;  // two-pass plans: first node of every request, and the total
+    std::vector<DevBfsNode> bfs;     // two-pass plans: the nodes of every request, breadth first
+    std::vector<int32_t> levels;     // two-pass plans: kLevelStride entries per request
 };
 
 struct Run {   // a run of tiles of one segment for one (request, kv head, row-block group)
@@ -257,6 +261,33 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, Host
     while (static_cast<int>(m.cta_begin.size()) < n_bins + 1) m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
 }
 
+// Nodes [n0, n1) of one request in breadth-first order: level by level, the children of a node next to each other.
+void add_bfs_nodes(HostMeta& m, int n0, int n1) {
+    std::vector<std::vector<int>> children(n1 - n0);
+    std::vector<int> order, up;                        // node (from n0) and position of its parent, by position
+    for (int n = n0; n < n1; ++n) {
+        if (m.nodes[n].parent < 0) { order.push_back(n - n0); up.push_back(-1); }
+        else children[m.nodes[n].parent - n0].push_back(n - n0);
+    }
+    std::vector<int32_t> level(kLevelStride, n1 - n0);
+    int n_levels = 0;
+    for (size_t begin = 0; begin < order.size();) {
+        const size_t end = order.size();
+        level[1 + n_levels++] = static_cast<int32_t>(begin);
+        for (size_t i = begin; i < end; ++i) {
+            const DevNode& nd = m.nodes[n0 + order[i]];
+            const uint32_t first = static_cast<uint32_t>(order.size());
+            for (int c : children[order[i]]) { order.push_back(c); up.push_back(static_cast<int>(i)); }
+            m.bfs.push_back(DevBfsNode{(static_cast<uint32_t>(order[i]) & BFS_MASK) | ((static_cast<uint32_t>(up[i] + 1) & BFS_MASK) << 12)
+                                           | (nd.scaled ? BFS_SCALED : 0u) | (nd.pad ? BFS_TOKENS : 0u),
+                                       (first & BFS_MASK) | ((static_cast<uint32_t>(order.size()) & BFS_MASK) << 12)});
+        }
+        begin = end;
+    }
+    level[0] = n_levels;
+    m.levels.insert(m.levels.end(), level.begin(), level.end());
+}
+
 // Every item carries a copy of its request's geometry and of its first tile record.
 void finish_items(HostMeta& m) {
     for (auto& it : m.items) {
@@ -272,8 +303,8 @@ int upload(ape_plan_t p, const HostMeta& m) {
     const size_t b_tiles = rnd(m.tiles.size() * sizeof(DevTile) + 16), b_items = rnd(m.items.size() * sizeof(DevItem) + 16),
                  b_cta = rnd(m.cta_begin.size() * 4 + 16), b_reqs = rnd(m.reqs.size() * sizeof(DevReq) + 16),
                  b_merge = rnd(m.merge.size() * sizeof(DevMerge) + 16), b_nodes = rnd(m.nodes.size() * sizeof(DevNode) + 16),
-                 b_rn = rnd(m.req_node0.size() * 4 + 16);
-    const size_t total = b_tiles + b_items + b_cta + b_reqs + b_merge + b_nodes + b_rn;
+                 b_rn = rnd(m.req_node0.size() * 4 + 16), b_bfs = rnd(m.bfs.size() * sizeof(DevBfsNode) + 16), b_lv = rnd(m.levels.size() * 4 + 16);
+    const size_t total = b_tiles + b_items + b_cta + b_reqs + b_merge + b_nodes + b_rn + b_bfs + b_lv;
     std::vector<uint8_t> host(total, 0);
     size_t o = 0;
     auto put = [&](const void* src, size_t n, size_t padded) { if (n) std::memcpy(host.data() + o, src, n); size_t at = o; o += padded; return at; };
@@ -284,6 +315,8 @@ int upload(ape_plan_t p, const HostMeta& m) {
     const size_t o_merge = put(m.merge.data(), m.merge.size() * sizeof(DevMerge), b_merge);
     const size_t o_nodes = put(m.nodes.data(), m.nodes.size() * sizeof(DevNode), b_nodes);
     const size_t o_rn = put(m.req_node0.data(), m.req_node0.size() * 4, b_rn);
+    const size_t o_bfs = put(m.bfs.data(), m.bfs.size() * sizeof(DevBfsNode), b_bfs);
+    const size_t o_lv = put(m.levels.data(), m.levels.size() * 4, b_lv);
     if (cudaMalloc(&p->d_blob, total) != cudaSuccess) { p->d_blob = nullptr; return APE_ERR_NOMEM; }
     if (cudaMemcpy(p->d_blob, host.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) return APE_ERR_CUDA;
     uint8_t* b = static_cast<uint8_t*>(p->d_blob);
@@ -294,6 +327,8 @@ int upload(ape_plan_t p, const HostMeta& m) {
     p->d_merge = reinterpret_cast<DevMerge*>(b + o_merge);
     p->d_nodes = reinterpret_cast<DevNode*>(b + o_nodes);
     p->d_req_node0 = reinterpret_cast<int32_t*>(b + o_rn);
+    p->d_bfs = reinterpret_cast<DevBfsNode*>(b + o_bfs);
+    p->d_levels = reinterpret_cast<int32_t*>(b + o_lv);
     p->n_items = static_cast<int>(m.items.size());
     p->n_merge = static_cast<int>(m.merge.size());
     return APE_OK;
@@ -557,6 +592,7 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             p->ws_bytes = ((rows * D * 4 + 255) & ~size_t(255)) + ((rows * 2 * 4 + 255) & ~size_t(255));
             m.req_node0.push_back(static_cast<int32_t>(m.nodes.size()));
             if (per_context != 0 && any_node_tiles) {
+                for (int r = 0; r < n_req; ++r) add_bfs_nodes(m, m.req_node0[r], m.req_node0[r + 1]);
                 if (row_base * shape->n_q_heads >= (1ll << 31)) { delete p; return APE_ERR_LAYOUT; }
                 p->two_pass = true;
                 p->n_nodes = static_cast<int>(m.nodes.size());
@@ -1060,7 +1096,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             ap.mode = kAttnStats; ap.stats = reinterpret_cast<float2*>(base + p->off_stats);
             if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
             NodeBiasParams nb;
-            nb.nodes = p->d_nodes; nb.reqs = p->d_reqs; nb.req_node0 = p->d_req_node0; nb.n_req = static_cast<int32_t>(p->n_req);
+            nb.nodes = p->d_nodes; nb.reqs = p->d_reqs; nb.req_node0 = p->d_req_node0; nb.bfs = p->d_bfs; nb.levels = p->d_levels; nb.n_req = static_cast<int32_t>(p->n_req);
             nb.stats = ap.stats; nb.mass = reinterpret_cast<float*>(base + p->off_mass); nb.bias = reinterpret_cast<float*>(base + p->off_bias);
             nb.stat_rows = p->stat_rows; nb.S = S; nb.H_q = p->shape.n_q_heads; nb.max_rows = p->max_rows;
             nb.max_nodes = p->max_nodes; nb.smem_limit = p->h->smem_optin;

@@ -78,6 +78,16 @@ struct DevNode {
 };
 constexpr int kMaxTreeDepth = 16;   // levels of nodes below the final merge
 
+// The nodes of a request once more, in breadth-first order (two-pass plans): a level is a range, a node's children are a range.
+// Indices and positions count from the request's first node and have 12 bits each: such a walk only runs for as many nodes as
+// fit into shared memory (a few more than 1,600), and eight bytes per record let the most of them fit.
+struct DevBfsNode {
+    uint32_t a;           // node index | (position of the parent + 1) << 12 | BFS_ flags
+    uint32_t b;           // position of the first child | position behind the last child << 12
+};
+enum : uint32_t { BFS_SCALED = 1u << 24, BFS_TOKENS = 1u << 25, BFS_MASK = 0xfffu };
+constexpr int kLevelStride = kMaxTreeDepth + 2;   // per request: number of levels, first position of every level, number of nodes
+
 struct RowsDesc {        // Q or O rows: element (r, h, e) at data[r*token_stride + h*head_stride + e]
     __nv_bfloat16* data;
     int64_t token_stride;

@@ -117,6 +117,8 @@ struct NodeBiasParams {
     const DevNode* nodes;            // all requests' nodes; pad != 0: the node has tokens of its own
     const DevReq* reqs;              // pad: the request's row base (rows before it in the plan)
     const int32_t* req_node0;        // [n_req + 1]: the nodes of request r are req_node0[r] .. req_node0[r + 1] - 1
+    const DevBfsNode* bfs;           // the same nodes, breadth first inside every request
+    const int32_t* levels;           // [n_req][kLevelStride]
     int32_t n_req;
     const float2* stats;             // [n_nodes][stat_rows] from the statistics pass (base-2 units)
     float* mass;                     // [n_nodes][stat_rows] scratch: A_n
