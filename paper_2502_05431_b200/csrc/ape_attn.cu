@@ -129,7 +129,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     constexpr int kSlabs = D / 64;
     constexpr int kTileBytes = kSlabs * kSlabBytes;            // one K or V tile, also one Q half
     constexpr int QBUF = (MODE == kAttnEncode) ? 2 : 1;
-    constexpr bool TURNS = MODE != kAttnAlt && MODE != kAttnEncode;   // the halves take turns in the exponential phase
+    constexpr bool TURNS = MODE == kAttnPrefill || MODE == kAttnBias;   // the halves take turns in the exponential phase
     constexpr bool ALT = MODE == kAttnAlt, STATS = MODE == kAttnStats, BIAS = MODE == kAttnBias;
     constexpr bool STAGED = MODE == kAttnPrefill || MODE == kAttnBias;   // partials leave through shared memory (there is room for it)
     constexpr int kQBytes = (ALT ? 1 : 2) * kTileBytes;        // both halves of a row block (ALT: the one half both read)
@@ -608,7 +608,9 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // phase n-1 of half 1; phase n of half 1 follows phase n of half 0 (both halves see the same tiles).
                 // (Alternating halves work on different tiles, with different numbers of them: no turns there.  Encode's items have
                 // one to three tiles, and a turn mostly makes a half wait whose partner is at the end of an item: 500 x 256
-                // tokens 897 us with turns, 865 without; the long items of prefill lose 11% without.)
+                // tokens 897 us with turns, 865 without; the long items of prefill lose 11% without.  In the statistics pass nothing but the
+                // exponentials is on a half's chain, and without turns the two halves fill each other's gaps: 386 us, now 339, for 256
+                // rows over 128K tokens.)
                 if (TURNS) {
                     const uint32_t n = scnt - 1;
                     bool turn = true;
@@ -630,10 +632,6 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                             float x0, x1;
                             unpack2(fma2(pack2(s[qq * 32 + 2 * i], s[qq * 32 + 2 * i + 1]), scale2, negm2), x0, x1);
                             sum2[i & 1] = add2(sum2[i & 1], pack2(fast_exp2(x0), fast_exp2(x1)));
-                        }
-                        if (qq == 3) {
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(bar_tok + 8 * (1 - w));
                         }
                     } else {
                         uint32_t pk[16];
