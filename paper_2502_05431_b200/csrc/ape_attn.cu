@@ -329,13 +329,14 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // Descriptors differ from their tile's base descriptor only in the 14-bit start-address field (units of 16 B),
         // so every MMA costs one add per operand instead of a descriptor build: the issuing lane shares its scheduler
         // with two softmax warps and must stay lean.
+        uint32_t idesc_qk = kIdescQK;
         uint64_t q_desc0 = smem_desc_sw128(smem_u32(q_smem + (ALT ? 0 : w) * kTileBytes), 16, 1024);
         auto issue_qk = [&](uint32_t k_base) {
             const uint64_t k_desc0 = smem_desc_sw128(k_base, 16, 1024);
             #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
                 const uint64_t o = static_cast<uint64_t>(((ks >> 2) * kSlabBytes + (ks & 3) * 32) >> 4);
-                mma_ss_elect(leader, tS, q_desc0 + o, k_desc0 + o, kIdescQK, ks > 0);
+                mma_ss_elect(leader, tS, q_desc0 + o, k_desc0 + o, idesc_qk, ks > 0);
             }
         };
         // P is zero past the last key that any row of the block may see, so the product stops there (rounded up to 16).
@@ -464,17 +465,19 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     o_started = true;
                 }
                 tc_fence_after();
+                int n_keys = tile.n_valid;                         // keys any row of the block may see
+                if (tile.flags & TILE_CAUSAL) n_keys = min(n_keys, g.last_tok + g.off - tile.key_base + 1);
+                // Encode, where every second or third tile is cut by the causal rule, computes S up to the last visible key only
+                // (the columns behind it are masked anyway).  A narrower product takes as long but less power, which is what
+                // bounds a large encode: 500 x 256 tokens 847 -> 840 us.
+                if (MODE == kAttnEncode) idesc_qk = idesc_bf16_f32(128, 0, 0, 0) | (static_cast<uint32_t>(max((n_keys + 15) >> 4, 1)) << 18);
                 issue_qk(k_base);
                 mma_commit_elect(leader, my_s_full);               // first: the softmax threads wait on this one
                 mma_commit_elect(leader, bar_k_empty + 8 * ksn);
                 if (prev_v_release) mma_commit_elect(leader, prev_v_release);
                 if (pending_q_release) mma_commit_elect(leader, pending_q_release);
                 prev_v_release = 0; pending_q_release = 0;
-                {
-                    int n_keys = tile.n_valid;                     // keys any row of the block may see
-                    if (tile.flags & TILE_CAUSAL) n_keys = min(n_keys, g.last_tok + g.off - tile.key_base + 1);
-                    prev_n16 = (n_keys + 15) & ~15;
-                }
+                prev_n16 = (n_keys + 15) & ~15;
                 have_prev = true; prev_valid = min(tile.n_valid, prev_n16); prev_vs = vs; prev_vphase = vphase;
             }
             if (ok && have_prev) {
@@ -560,8 +563,15 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 int limit = tile.n_valid;
                 if (tile.flags & TILE_CAUSAL) limit = min(limit, tok + g.off - tile.key_base + 1);
                 if (limit < kTileN) {
+                    // by mask bits, which reach the selects as predicates, several per instruction (a comparison each cost a
+                    // masked tile 1,000 cycles of its 3,800: encode 500 x 256 tokens 855 us, now 847; 10 x 256 26.2, now 25.6)
                     #pragma unroll
-                    for (int i = 0; i < kTileN; ++i) s[i] = (i < limit) ? s[i] : -INFINITY;
+                    for (int q = 0; q < kTileN / 32; ++q) {
+                        const int lq = min(max(limit - 32 * q, 0), 32);
+                        const uint32_t mask = static_cast<uint32_t>((1ull << lq) - 1);
+                        #pragma unroll
+                        for (int i = 0; i < 32; ++i) s[32 * q + i] = (mask & (1u << i)) ? s[32 * q + i] : -INFINITY;
+                    }
                 }
                 // eight independent running maxima (3-input max) keep the dependency chain short
                 float mxa[8];
