@@ -1,6 +1,7 @@
 """Merge of the partials: rows whose partials are shared by eight warps and rows with one, and rows with more partials than one round of
 lanes covers.  The number of partials per row follows the SM budget (one KV head: every thread block leaves one or two)."""
 import pytest
+import torch
 
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
@@ -36,3 +37,16 @@ def test_more_partials_than_one_round_of_lanes():
     b = wl.share_contexts(wl.make_batch(H_q=4, H_kv=1, d=128, l_P=5, ctx_lens=[[40000]] + [[1]] * 2, l_q=1, l_k=9, seed=32,
                                         T=0.9, S=0.8, name="merge_296"))
     _check(b, libape.APE_DECODE, shared=True)
+
+
+@pytest.mark.parametrize("n_sm", [16, 15, 17, 40, 148])
+def test_runs_with_thread_blocks_of_their_own(n_sm):
+    """Eight heads, a long and a short segment each: budgets at which every (head, segment) gets its own thread blocks (16: one
+    each), the one below at which that does not fit, and budgets with tiles to spare."""
+    b = wl.make_batch(H_q=8, H_kv=8, d=128, l_P=70, ctx_lens=[[60, 1, 130, 64]], l_q=1, l_k=9, gap=3, seed=33, T=0.8, S=0.9,
+                      name=f"own_blocks_sm{n_sm}")
+    handle().set_sm_budget(min(n_sm, torch.cuda.get_device_properties(0).multi_processor_count))
+    try:
+        _check(b, libape.APE_DECODE)
+    finally:
+        handle().set_sm_budget(0)
