@@ -65,10 +65,6 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return r;
 }
 
-__device__ __forceinline__ void prefetch_l1(const void* ptr) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr));
-}
-
 struct ItemGeom {
     int rb;          // row block of this CTA for the item
     int last_tok;    // last live query token of the row block
