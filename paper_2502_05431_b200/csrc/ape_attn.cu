@@ -153,7 +153,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const uint32_t bar_o_full = bar_p_full + 64;               // [2]
     const uint32_t bar_done = bar_o_full + 16;
     const uint32_t bar_tok = bar_done + 8;                     // [2]: turn-taking of the two halves' exponential phases
-    const uint32_t bar_o_staged = bar_tok + 16;                // [2]: a half's O tile sits in shared memory, ready for its bulk store
+    const uint32_t bar_o_staged = bar_tok + 16;                // [QBUF][2]: a half's O tile sits in its Q buffer, ready for its bulk store
     __shared__ uint32_t tmem_base_smem;
     __shared__ int abort_flag;
 
@@ -171,7 +171,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
         mbar_init(bar_done, 2);
         mbar_init(bar_tok, 4); mbar_init(bar_tok + 8, 4);          // one arrival per softmax warp of the other half
-        mbar_init(bar_o_staged, 4); mbar_init(bar_o_staged + 8, 4);  // one arrival per softmax warp of the half
+        for (int b = 0; b < 2 * QBUF; ++b) mbar_init(bar_o_staged + 8 * b, 4);       // one arrival per softmax warp of the half
         mbar_fence_init();
     }
     if (warp == kMmaWarp) {
@@ -689,7 +689,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (o_via_tma && half_is_full(rq, g, w)) {
                     // The item's Q buffer is free (O is final, so every S = Q K^T that read it is done) and has the layout
                     // the bulk store wants: row r of the half, 16-byte chunk j of a 128-byte line at chunk j ^ (r mod 8).
-                    uint8_t* stage = q_smem + ((q_loads - 1) % QBUF) * kQBytes + w * kTileBytes + r_local * 128;
+                    const uint32_t qb = (q_loads - 1) % QBUF;
+                    uint8_t* stage = q_smem + qb * kQBytes + w * kTileBytes + r_local * 128;
                     #pragma unroll
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t o[32];
@@ -708,7 +709,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_o_staged + 8 * w);
+                    if (lane == 0) mbar_arrive(bar_o_staged + 16 * qb + 8 * w);
                 } else
                 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
@@ -768,20 +769,23 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (o_via_tma) tma_prefetch_desc(&tm_o);
             if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
             pdl_wait();
-            uint32_t q_loads = 0, staged[2] = {0, 0};
+            uint32_t q_loads = 0, staged = 0;                        // staged: phase parity of each of the four barriers
             int last_req = -1, last_head = -1, last_rb = -1;
             bool ok = true;
             // what the bulk store of a row block needs, kept for the two row blocks whose buffers are in use
             struct Pending { int head0, tok0; bool full[2]; } pend[2] = {{0, 0, {false, false}}, {0, 0, {false, false}}};
             // O of the row block that used buffer qb: wait for each staged half, send it, and return once the copies have
-            // read the buffer (it is about to be refilled with the next Q).
+            // read the buffer (it is about to be refilled with the next Q).  A half may be a whole row block ahead of this
+            // look (nothing holds it to the other half's epilogue), so the two row blocks in flight have barriers of their
+            // own: the next arrival on this one belongs to the row block whose Q is only loaded after the look.
             auto drain = [&](uint32_t qb) {
                 bool any = false;
                 #pragma unroll
                 for (int w = 0; w < 2; ++w) {
                     if (!pend[qb].full[w]) continue;
-                    if (!mbar_wait(bar_o_staged + 8 * w, staged[w] & 1, &abort_flag, p.status)) return false;
-                    ++staged[w];
+                    const uint32_t b = 2 * qb + w;
+                    if (!mbar_wait(bar_o_staged + 8 * b, (staged >> b) & 1, &abort_flag, p.status)) return false;
+                    staged ^= 1u << b;
                     #pragma unroll
                     for (int sl = 0; sl < kSlabs; ++sl)
                         tma_store_3d(&tm_o, smem_u32(q_smem + qb * kQBytes + w * kTileBytes + sl * kSlabBytes),
