@@ -312,6 +312,9 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // walk the loop and take part in the waits; lane 0 issues the tensor-core instructions.
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
         const int w = warp - kMmaWarp;
+        // Nothing here touches memory in front of the first Q tile, but the waits are bounded: their time must not run while the
+        // kernel before this one still does.
+        pdl_wait();
         uint32_t kcnt = 0, vcnt = 0, q_loads = 0, pcnt = 0;
         int last_req = -1, last_head = -1, last_rb = -1;
         bool ok = true;

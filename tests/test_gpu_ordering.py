@@ -2,6 +2,7 @@
 import pytest
 import torch
 
+from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
 from tests.gpu_util import handle
 from tests.test_gpu_parity import _check_encode
@@ -28,3 +29,40 @@ def test_encode_stages_two_row_blocks_at_a_time(l_P, heads, lens):
         plans[1].encode_contexts()
         assert torch.equal(outs[0], outs[1])
     assert handle().get_status() == 0
+
+
+EARLY_AND_LONG = """
+extern "C" __global__ void early_and_long() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2800000000ll) {}
+}
+"""
+
+
+@pytest.mark.parametrize("op", ["prefill", "per_context", "decode", "encode"])
+def test_time_limit_of_waits_starts_after_the_kernel_before(op):
+    """A kernel (any library's) that lets the next one in early and then runs for longer than the limit of a bounded wait (2^31
+    cycles): what a call waits for meanwhile is that kernel, and it must not count as a copy or product that never came."""
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=30, ctx_lens=[[256, 70, 1]], l_q=1 if op == "decode" else 70, l_k=75, seed=61, T=0.8, S=0.9,
+                      with_encode_q=True, name="late").to("cuda:0")
+    rq, heads = b.requests[0], dict(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool)
+    q = b.q_enc if op == "encode" else b.q
+    out = torch.zeros_like(q)
+    if op == "encode":
+        plan = handle().encode_plan(**heads, q=q, out=out, prefix=rq.prefix, ctx=rq.ctx)
+        launch = plan.encode_contexts
+    else:
+        plan = handle().attend_plan(**heads, q=q, out=out, requests=b.requests, per_context=op == "per_context",
+                                    mode=libape.APE_DECODE if op == "decode" else libape.APE_PREFILL)
+        ws = plan.alloc_workspace()
+        launch = lambda: plan.attend(b.T, b.S, ws)  # noqa: E731
+    launch()
+    first = out.clone()
+    out.zero_()
+    before = torch.cuda._compile_kernel(EARLY_AND_LONG, "early_and_long")
+    before(grid=(1, 1, 1), block=(32, 1, 1), args=[])
+    launch()
+    torch.cuda.synchronize()
+    assert handle().get_status() == 0
+    assert torch.equal(out, first)
