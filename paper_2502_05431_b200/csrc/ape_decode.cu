@@ -127,7 +127,8 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
             const float scale = (item.seg == SEG_CTX) ? p.scale_ctx_log2 : p.scale_oth_log2;
             const int l_k_now = rq.l_k + p.kv_extra;
 
-            // Q fragments (A operand, 16 x D, rows >= G are zero)
+            // Q fragments (A operand, 16 x D, rows >= G are zero).  Plain loads: this grid exists while the kernel before it, which
+            // may be writing Q, still runs, and the read-only path is for data that nobody writes in a grid's lifetime.
             uint32_t qa[kKSteps][4];
             {
                 const __nv_bfloat16* qbase = p.q.data + static_cast<int64_t>(rq.q_row0) * p.q.token_stride
@@ -137,10 +138,10 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
                     const int col = ks * 16 + 2 * qc;
                     const uint32_t* r_lo = reinterpret_cast<const uint32_t*>(qbase + static_cast<int64_t>(qr) * p.q.head_stride + col);
                     const uint32_t* r_hi = reinterpret_cast<const uint32_t*>(qbase + static_cast<int64_t>(qr + 8) * p.q.head_stride + col);
-                    qa[ks][0] = (qr < G) ? __ldg(r_lo) : 0u;
-                    qa[ks][1] = (qr + 8 < G) ? __ldg(r_hi) : 0u;
-                    qa[ks][2] = (qr < G) ? __ldg(r_lo + 4) : 0u;
-                    qa[ks][3] = (qr + 8 < G) ? __ldg(r_hi + 4) : 0u;
+                    qa[ks][0] = (qr < G) ? *r_lo : 0u;
+                    qa[ks][1] = (qr + 8 < G) ? *r_hi : 0u;
+                    qa[ks][2] = (qr < G) ? r_lo[4] : 0u;
+                    qa[ks][3] = (qr + 8 < G) ? r_hi[4] : 0u;
                 }
             }
 

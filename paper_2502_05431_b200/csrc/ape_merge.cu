@@ -15,7 +15,7 @@ namespace {
 constexpr float kLn2 = 0.6931471805599453f;
 
 template <int VEC>
-__device__ __forceinline__ void combine_segment(const float* __restrict__ ws_o, const float* __restrict__ ws_ml,
+__device__ __forceinline__ void combine_segment(const float* ws_o, const float* ws_ml,
                                                 int slot0, int n, int stride, int rows_per_slot, int row, int D,
                                                 int lane, float& M, float& L, float (&acc)[VEC])
 {

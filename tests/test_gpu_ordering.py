@@ -66,3 +66,66 @@ def test_time_limit_of_waits_starts_after_the_kernel_before(op):
     torch.cuda.synchronize()
     assert handle().get_status() == 0
     assert torch.equal(out, first)
+
+
+def _same_with_and_without_waits(launches, bufs):
+    """Chains of 1, 2, ... calls, each reading the buffer that the one before it wrote: the same bits with a synchronisation behind
+    every call and with nothing at all between two calls."""
+    start = bufs[0].clone()
+    for n in range(1, len(launches) + 1):
+        ends = []
+        for wait in (True, False):
+            bufs[0].copy_(start)
+            bufs[1].zero_()
+            torch.cuda.synchronize()
+            for launch in launches[:n]:
+                launch()
+                if wait:
+                    torch.cuda.synchronize()
+            torch.cuda.synchronize()
+            ends.append([x.clone() for x in bufs])
+        assert not torch.isnan(ends[0][n % 2].float()).any()
+        assert torch.equal(ends[0][0], ends[1][0]) and torch.equal(ends[0][1], ends[1][1]), f"{n} calls"
+        assert not torch.equal(ends[0][0], ends[0][1])
+    assert handle().get_status() == 0
+
+
+@pytest.mark.parametrize("mode,l_q,n_req", [(libape.APE_DECODE, 1, 4), (libape.APE_PREFILL, 64, 1), (libape.APE_PREFILL, 200, 1)])
+def test_calls_that_feed_each_other(mode, l_q, n_req):
+    """The output of a call is the query of the next, all calls share one workspace, and no kernel of another library stands between
+    them: what a kernel reads too early is an older query, partial or bias.  All plan kinds, each call over contexts of its own."""
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=30, ctx_lens=[[256, 70, 130, 64] * 12] * n_req, l_q=l_q, l_k=l_q + 5, seed=62, T=0.7, S=0.8,
+                      name="chain").to("cuda:0")
+    b.v_pool *= 8                              # (large outputs, a high logit scale: a call's query decides its result)
+    bufs = [b.q, torch.zeros_like(b.q)]
+    forms = [dict(), dict(per_context=True), dict(tree=([[-1, 0, 0, 0]] * n_req, None))]
+    if mode == libape.APE_DECODE:
+        forms.append(dict(shared=True))
+    plans = []
+    for i in range(12):
+        form = forms[i % len(forms)]
+        ctx = [r.ctx[4 * i:4 * i + 4] for r in b.requests]
+        reqs = [wl.Request(r.q_start, r.q_len, r.prefix, ctx[0 if form.get("shared") else j], r.query_kv, r.query_kv_capacity)
+                for j, r in enumerate(b.requests)]
+        plans.append(handle().attend_plan(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool, q=bufs[i % 2], out=bufs[(i + 1) % 2],
+                                          requests=reqs, mode=mode, softmax_scale=0.5, **form))
+    ws = torch.empty(max(p.workspace_bytes for p in plans), dtype=torch.uint8, device="cuda:0")
+    _same_with_and_without_waits([lambda p=p: p.attend(b.T, b.S, ws) for p in plans], bufs)
+
+
+def test_encode_and_prefill_that_feed_each_other():
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=64, ctx_lens=[[256] * 8], l_q=1, l_k=9, seed=63, T=0.7, S=0.8, with_encode_q=True,
+                      name="chain_encode").to("cuda:0")
+    b.v_pool *= 8
+    rq, heads = b.requests[0], dict(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool, softmax_scale=0.5)
+    bufs = [torch.nan_to_num(b.q_enc), torch.zeros_like(b.q_enc)]
+    plans = []
+    for i in range(10):
+        io = dict(q=bufs[i % 2], out=bufs[(i + 1) % 2])
+        if i % 2 == 0:
+            plans.append(handle().encode_plan(**heads, **io, prefix=rq.prefix, ctx=rq.ctx))
+        else:                                  # the rows of every context, over all the contexts but that one
+            reqs = [wl.Request(s, n, rq.prefix, [c for c in rq.ctx if c[0] != s], (s, n), n) for s, n in rq.ctx]
+            plans.append(handle().attend_plan(**heads, **io, requests=reqs, mode=libape.APE_PREFILL))
+    ws = torch.empty(max(p.workspace_bytes for p in plans), dtype=torch.uint8, device="cuda:0")
+    _same_with_and_without_waits([p.encode_contexts if i % 2 == 0 else lambda p=p: p.attend(b.T, b.S, ws) for i, p in enumerate(plans)], bufs)
