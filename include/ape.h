@@ -95,6 +95,9 @@ int ape_destroy(ape_handle_t handle);
  * key/value stream over thread blocks (the split-KV of the appendix "Hierarchical Formula for Softmax Attention")
  * follows the budget, the result does not depend on it beyond rounding.  1 <= n_sm <= SMs of the device, else
  * APE_ERR_INVALID_ARG.  Plans that already exist keep their split.
+ * While an attention or decode kernel of such a plan runs, no later kernel of its stream takes SMs (plans without a budget let
+ * the next kernel's thread blocks in early, where they wait).  The short kernels between and behind them (merge, node biases) use
+ * the whole GPU.
  */
 int ape_set_sm_budget(ape_handle_t handle, int32_t n_sm);
 

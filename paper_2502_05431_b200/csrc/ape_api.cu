@@ -56,6 +56,7 @@ struct ape_plan_s {
     SplitMaps tm_split{};           // encode plans with split_r > 0
     int split_r = 0;
     bool o_via_tma = false;         // encode plans: tm_o describes the output rows
+    bool budget = false;            // made under an SM budget: the SMs that it leaves stay free while its kernels run
     bool alt_halves = false;        // context pass of a shared plan with at most 128 rows: the halves take alternate tiles
     int32_t last_launches = 0;
     int per_context = 0;             // merge form: 0 Eq. 5, 1 Eq. 11-12 (per context), 2 context trees
@@ -500,7 +501,7 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
 
     ape_plan_t p = new (std::nothrow) ape_plan_s();
     if (!p) return APE_ERR_NOMEM;
-    p->h = h; p->kind = (mode == APE_DECODE) ? PLAN_DECODE : PLAN_PREFILL;
+    p->h = h; p->budget = h->n_sm < h->n_sm_device; p->kind = (mode == APE_DECODE) ? PLAN_DECODE : PLAN_PREFILL;
     p->shape = *shape; p->c = c; p->G = G; p->pool = *pool; p->q = *q; p->out = *out; p->lse = lse; p->per_context = per_context;
     p->max_kv_extra = (mode == APE_DECODE) ? max_extra : 0;
     p->n_req = n_req;
@@ -695,7 +696,7 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
 
     auto new_plan = [&](PlanKind kind) {
         ape_plan_t p = new (std::nothrow) ape_plan_s();
-        if (p) { p->h = h; p->kind = kind; p->shape = *shape; p->c = c; p->G = G; p->pool = *pool; p->q = *q; p->out = *out; p->lse = lse; }
+        if (p) { p->h = h; p->budget = h->n_sm < h->n_sm_device; p->kind = kind; p->shape = *shape; p->c = c; p->G = G; p->pool = *pool; p->q = *q; p->out = *out; p->lse = lse; }
         return p;
     };
     ape_plan_t p = new_plan(PLAN_SHARED);
@@ -826,7 +827,7 @@ int ape_encode_plan(ape_handle_t h, const ape_shape_t* shape, const ape_kv_pool_
 
     ape_plan_t p = new (std::nothrow) ape_plan_s();
     if (!p) return APE_ERR_NOMEM;
-    p->h = h; p->kind = PLAN_ENCODE; p->shape = *shape; p->c = c; p->G = G; p->pool = *pool; p->q = *q; p->out = *out; p->lse = lse;
+    p->h = h; p->budget = h->n_sm < h->n_sm_device; p->kind = PLAN_ENCODE; p->shape = *shape; p->c = c; p->G = G; p->pool = *pool; p->q = *q; p->out = *out; p->lse = lse;
     p->n_sib = 1;
     const int D = shape->head_dim, H_kv = shape->n_kv_heads, tile = kAttnTileN, TB = kAttnRows / G;
 
@@ -1061,7 +1062,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             ap.out = rows_desc(p->out); ap.lse_out = nullptr; ap.ws_o = a_o; ap.ws_ml = a_ml;
             ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
             ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = a->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
-            ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; if (a->alt_halves) ap.mode = kAttnAlt;
+            ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1; if (a->alt_halves) ap.mode = kAttnAlt;
             if (launch_attn(D, a->tm_q, a->tm_k, a->tm_v, a->tm_q, a->tm_split, ap, a->n_cta, a->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
             p->last_launches++;
         }
@@ -1070,6 +1071,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         dp.q = rows_desc(p->q); dp.ws_o = b_o; dp.ws_ml = b_ml;
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = b->n_stages; dp.status = p->h->d_status;
+        dp.let_next_in = p->budget ? 0 : 1;
         if (launch_decode(D, b->tm_k, b->tm_v, dp, b->n_cta, b->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
         p->last_launches++;
         MergeParams mp;
@@ -1095,6 +1097,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         dp.q = rows_desc(p->q); dp.ws_o = ws_o; dp.ws_ml = ws_ml;
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = p->n_stages; dp.status = p->h->d_status;
+        dp.let_next_in = p->budget ? 0 : 1;
         if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
     } else {
         AttnParams ap;
@@ -1102,7 +1105,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         ap.out = rows_desc(p->out); ap.lse_out = nullptr; ap.ws_o = ws_o; ap.ws_ml = ws_ml;
         ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
         ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = p->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
-        ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0;
+        ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1;
         if (p->two_pass) {
             // per-context form / context trees: (1) every node's own (maximum, sum) per row, (2) per-row, per-node biases
             // from them and S, (3) the prefill with the biases on the context logits; the merge below then sees an
@@ -1196,7 +1199,7 @@ int ape_encode_contexts(ape_plan_t p, void* workspace, size_t ws_bytes, void* st
     ap.out = rows_desc(p->out); ap.lse_out = p->lse; ap.ws_o = nullptr; ap.ws_ml = nullptr;
     ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c * kLog2e;
     ap.G = p->G; ap.H_q = p->shape.n_q_heads; ap.n_sib = 1; ap.mode = kAttnEncode; ap.q_rows_are_pool = 1; ap.status = p->h->d_status;
-    ap.o_via_tma = p->o_via_tma ? 1 : 0; ap.split_r = p->split_r; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0;
+    ap.o_via_tma = p->o_via_tma ? 1 : 0; ap.split_r = p->split_r; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1;
     if (launch_attn(p->shape.head_dim, p->tm_q, p->tm_k, p->tm_v, p->tm_o, p->tm_split, ap, p->n_cta, p->smem_bytes,
                     static_cast<cudaStream_t>(stream_v)) != cudaSuccess) return APE_ERR_CUDA;
     p->last_launches = 1;
@@ -1528,7 +1531,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     dp.cta_item_begin = reinterpret_cast<const int32_t*>(base + o_cta); dp.reqs = reinterpret_cast<const DevReq*>(base + o_reqs);
     dp.q = rows_desc(*q); dp.ws_o = ws_o; dp.ws_ml = ws_ml;
     dp.scale_oth_log2 = c * kLog2e; dp.scale_ctx_log2 = c / T * kLog2e;
-    dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = n_stages; dp.status = reinterpret_cast<int*>(base);
+    dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = n_stages; dp.status = reinterpret_cast<int*>(base); dp.let_next_in = 1;
     if (launch_decode(D, tm_k, tm_v, dp, n_cta, smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
     MergeParams mp;
     mp.groups = reinterpret_cast<const DevMerge*>(base + o_merge); mp.reqs = dp.reqs; mp.items = dp.items; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = static_cast<int32_t>(m.merge.size());

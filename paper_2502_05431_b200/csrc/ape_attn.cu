@@ -229,7 +229,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
             if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
             pdl_wait();
-            pdl_trigger();
+            if (p.let_next_in != 0) pdl_trigger();
             uint32_t kcnt = 0, vcnt = 0, q_loads = 0;
             int last_req = -1, last_head = -1, last_rb = -1;
             bool ok = true;

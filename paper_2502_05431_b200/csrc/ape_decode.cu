@@ -77,7 +77,7 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
     }
     __syncthreads();
     pdl_wait();
-    pdl_trigger();
+    if (p.let_next_in != 0) pdl_trigger();
 
     if (warp == kConsumerWarps) {
         // ---------------- producer: one lane feeds the ring --------------------------------------------------------

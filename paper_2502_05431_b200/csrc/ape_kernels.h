@@ -22,6 +22,7 @@ struct DecodeParams {
     int32_t kv_extra;
     int32_t G;
     int32_t n_stages;
+    int32_t let_next_in;             // 0: no block of the next kernel is placed before this one ends (plans under an SM budget)
     int* status;
 };
 
@@ -64,6 +65,7 @@ struct AttnParams {
     float2* stats;                   // kAttnStats writes (running maximum, sum) in base-2 units
     const float* bias;               // kAttnBias reads the bias (base-2 units) of the node's tokens
     int64_t stat_rows;
+    int32_t let_next_in;             // as in DecodeParams
     int* status;
 };
 

@@ -129,3 +129,45 @@ def test_encode_and_prefill_that_feed_each_other():
             plans.append(handle().attend_plan(**heads, **io, requests=reqs, mode=libape.APE_PREFILL))
     ws = torch.empty(max(p.workspace_bytes for p in plans), dtype=torch.uint8, device="cuda:0")
     _same_with_and_without_waits([p.encode_contexts if i % 2 == 0 else lambda p=p: p.attend(b.T, b.S, ws) for i, p in enumerate(plans)], bufs)
+
+
+@pytest.mark.parametrize("op", ["encode", "decode", "prefill", "per_context", "shared"])
+def test_budget_leaves_the_other_sms_free(op):
+    """A long call on one SM with another call queued behind it: a call on a second stream, which needs whole SMs, runs meanwhile on
+    the ones that the budget leaves.  (None of the calls waits for another one's result.)"""
+    n = 4000 if op == "encode" else 60000
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=64, ctx_lens=[[n], [64]], l_q=1, l_k=9, seed=64, T=0.8, S=0.9, with_encode_q=True,
+                      name="budget", device="cuda:0")
+    reqs = b.requests[:1]
+    heads = dict(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool)
+    rq = reqs[0]
+    form = dict(per_context=op == "per_context", shared=op == "shared")
+    handle().set_sm_budget(1)
+    try:
+        if op == "encode":
+            long = handle().encode_plan(**heads, q=b.q_enc, out=torch.zeros_like(b.q_enc), prefix=rq.prefix, ctx=rq.ctx)
+        else:
+            mode = libape.APE_DECODE if op in ("decode", "shared") else libape.APE_PREFILL
+            long = handle().attend_plan(**heads, q=b.q, out=torch.zeros_like(b.q), requests=reqs, mode=mode, **form)
+    finally:
+        handle().set_sm_budget(0)
+    ws = [long.alloc_workspace()]
+    run_long = long.encode_contexts if op == "encode" else lambda: long.attend(b.T, b.S, ws[0])
+    other = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=64, ctx_lens=[[64] * 40], l_q=64, l_k=64, seed=65, T=0.8, S=0.9, name="beside",
+                          device="cuda:0")
+    after, beside = [handle().attend_plan(H_q=32, H_kv=8, d=128, k_pool=other.k_pool, v_pool=other.v_pool, q=other.q,
+                                          out=torch.zeros_like(other.q), requests=other.requests, mode=libape.APE_PREFILL) for _ in range(2)]
+    ws += [after.alloc_workspace(), beside.alloc_workspace()]
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    run_long(), after.attend(0.8, 0.9, ws[1]), beside.attend(0.8, 0.9, ws[2])       # (first launches load code)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        run_long()
+        after.attend(0.8, 0.9, ws[1])
+        done = s1.record_event()
+    with torch.cuda.stream(s2):
+        beside.attend(0.8, 0.9, ws[2])
+    s2.synchronize()
+    assert not done.query(), "the call beside it only ran once the long call had ended"
+    torch.cuda.synchronize()
+    assert handle().get_status() == 0
