@@ -225,6 +225,9 @@ struct HostMeta {
 // kernel).
 constexpr int kDecodeItemTiles = 1, kAttnItemTiles = 2;
 
+// The decode kernel's static shared memory, which counts against the same limit (1,024 bytes, and as much to spare).
+constexpr size_t kDecodeStaticSmem = 2048;
+
 struct Run {   // a run of tiles of one segment for one (request, kv head, row-block group)
     int req, kv_head, row_block, n_sib, seg, t0, t1, merge0;
     int ctx_id = 0;   // per-context plans: ordinal of the context of a SEG_CTX run
@@ -535,14 +538,14 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             p->n_cta = h->n_sm;
             assign_stream(runs, p->n_cta, 1, kDecodeItemTiles, m);
             p->n_slots = static_cast<int>(m.items.size());
-            p->n_stages = decode_pick_stages(D, G, h->smem_optin - 2048);
+            p->n_stages = decode_pick_stages(D, G, h->smem_optin - kDecodeStaticSmem);
             if (p->n_stages < 2) { delete p; return APE_ERR_SHAPE; }
             p->smem_bytes = decode_smem_bytes(D, G, p->n_stages);
             const size_t rows = static_cast<size_t>(p->n_slots) * G;
             p->ws_bytes = ((rows * D * 4 + 255) & ~size_t(255)) + ((rows * 2 * 4 + 255) & ~size_t(255));
             rc = make_map(h, &p->tm_k, pool->k, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, tile);
             if (!rc) rc = make_map(h, &p->tm_v, pool->v, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, tile);
-            if (!rc && decode_set_smem_attr(D, p->smem_bytes) != cudaSuccess) rc = APE_ERR_CUDA;
+            if (!rc && decode_set_smem_attr(D, h->smem_optin - kDecodeStaticSmem) != cudaSuccess) rc = APE_ERR_CUDA;
             if (!rc) rc = setup_decode_step(p, reqs, n_req);
         } else {
             const int tile = kAttnTileN;
@@ -759,14 +762,14 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
             b->n_sib = 1; b->n_cta = h->n_sm;
             assign_stream(runs_b, b->n_cta, 1, kDecodeItemTiles, mb);
             b->n_slots = static_cast<int>(mb.items.size());
-            b->n_stages = decode_pick_stages(D, G, h->smem_optin - 2048);
+            b->n_stages = decode_pick_stages(D, G, h->smem_optin - kDecodeStaticSmem);
             if (b->n_stages < 2) rc = APE_ERR_SHAPE;
         }
         if (!rc) {
             b->smem_bytes = decode_smem_bytes(D, G, b->n_stages);
             rc = make_map(h, &b->tm_k, pool->k, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, kDecodeTile);
             if (!rc) rc = make_map(h, &b->tm_v, pool->v, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, kDecodeTile);
-            if (!rc && decode_set_smem_attr(D, b->smem_bytes) != cudaSuccess) rc = APE_ERR_CUDA;
+            if (!rc && decode_set_smem_attr(D, h->smem_optin - kDecodeStaticSmem) != cudaSuccess) rc = APE_ERR_CUDA;
             if (!rc) { finish_items(mb); rc = upload(b, mb); }
         }
 
@@ -1503,10 +1506,10 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
         return APE_ERR_NOMEM;
     }
 
-    const int n_stages = decode_pick_stages(D, G, dv->h.smem_optin - 2048);
+    const int n_stages = decode_pick_stages(D, G, dv->h.smem_optin - kDecodeStaticSmem);
     if (n_stages < 2) return APE_ERR_SHAPE;
     const size_t smem_bytes = decode_smem_bytes(D, G, n_stages);
-    if (decode_set_smem_attr(D, smem_bytes) != cudaSuccess) return APE_ERR_CUDA;
+    if (decode_set_smem_attr(D, dv->h.smem_optin - kDecodeStaticSmem) != cudaSuccess) return APE_ERR_CUDA;
     CUtensorMap tm_k, tm_v;
     rc = make_map(&dv->h, &tm_k, pool->k, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, tile);
     if (!rc) rc = make_map(&dv->h, &tm_v, pool->v, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, tile);

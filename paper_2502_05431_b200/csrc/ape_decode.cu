@@ -304,10 +304,9 @@ cudaError_t launch_decode(int D, const CUtensorMap& tm_k, const CUtensorMap& tm_
     return launch_pdl(D == 128 ? ape_decode_kernel<128> : ape_decode_kernel<64>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
 }
 
-cudaError_t decode_set_smem_attr(int D, size_t smem_bytes) {
-    if (D == 128)
-        return cudaFuncSetAttribute(ape_decode_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
-    return cudaFuncSetAttribute(ape_decode_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+cudaError_t decode_set_smem_attr(int D, size_t smem_limit) {
+    return cudaFuncSetAttribute(D == 128 ? ape_decode_kernel<128> : ape_decode_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem_limit));
 }
 
 }  // namespace ape

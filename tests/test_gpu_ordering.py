@@ -4,7 +4,7 @@ import torch
 
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
-from tests.gpu_util import handle
+from tests.gpu_util import compare, handle, oracle_attend
 from tests.test_gpu_parity import _check_encode
 
 pytestmark = pytest.mark.gpu
@@ -171,3 +171,25 @@ def test_budget_leaves_the_other_sms_free(op):
     assert not done.query(), "the call beside it only ran once the long call had ended"
     torch.cuda.synchronize()
     assert handle().get_status() == 0
+
+
+def test_decode_plans_of_other_head_layouts_leave_a_plan_usable():
+    """The shared memory that a decode launch asks for depends on G; the kernel's limit is one per process and must not follow the plan
+    made last (nor an allocation-free call)."""
+    plans = []
+    for H_q, H_kv in ((32, 8), (16, 1), (8, 8), (16, 8)):
+        b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=128, l_P=20, ctx_lens=[[300, 5]], l_q=1, l_k=9, seed=66, T=0.8, S=0.9, name=f"G{H_q // H_kv}")
+        dev = b.to("cuda:0")
+        out = torch.zeros_like(dev.q)
+        plan = handle().attend_plan(H_q=H_q, H_kv=H_kv, d=128, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=out, requests=b.requests,
+                                    mode=libape.APE_DECODE)
+        plans.append((b, dev, plan, out, plan.alloc_workspace()))
+    for b, dev, plan, out, ws in plans + plans[:1]:
+        plan.attend(b.T, b.S, ws)
+        compare(out.cpu(), oracle_attend(b, 0).out.float(), b.name)
+    b, dev, _, out, _ = plans[1]
+    libape.decode_noalloc(H_q=16, H_kv=1, d=128, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=out, requests=b.requests, T=b.T, S=b.S,
+                          want_status=True)
+    b, dev, plan, out, ws = plans[0]
+    plan.attend(b.T, b.S, ws)
+    compare(out.cpu(), oracle_attend(b, 0).out.float(), b.name)
