@@ -553,8 +553,9 @@ cudaError_t launch_node_bias(const NodeBiasParams& p, cudaStream_t stream)
     if (p.n_req <= 0 || p.max_rows <= 0) return cudaSuccess;
     const size_t smem = static_cast<size_t>(p.max_nodes) * (kBiasRows * sizeof(float) + sizeof(DevBfsNode));
     if (p.max_nodes > 0 && smem <= p.smem_limit) {
+        // (the device's limit, not this launch's size: another thread may be between its own two steps)
         if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(ape_node_bias_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+            cudaFuncSetAttribute(ape_node_bias_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(p.smem_limit)) != cudaSuccess)
             return cudaGetLastError();
         const dim3 grid(static_cast<unsigned>((p.max_rows + kBiasRows - 1) / kBiasRows), static_cast<unsigned>(p.n_req));
         return launch_pdl(ape_node_bias_smem_kernel, grid, kBiasWarps * 32, smem, stream, p);

@@ -1,11 +1,14 @@
 """The walk between the two passes of a prefill over context trees: levels of very different widths, children whose breadth-first
 order differs from their index order, the deepest tree, and as many nodes as the shared-memory form of the walk takes."""
 import random
+import threading
 
 import pytest
+import torch
 
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
+from tests.gpu_util import handle
 from tests.test_gpu_tree import _check
 
 pytestmark = pytest.mark.gpu
@@ -38,3 +41,33 @@ def test_deepest_tree_and_a_request_without_contexts():
 def test_as_many_nodes_as_fit_and_more(n, parents):
     """(1,709 nodes x 136 bytes is what a block's shared memory holds)"""
     _run([[1 + i % 3 for i in range(n)]], [parents], None, l_q=3)
+
+
+def test_two_threads_with_trees_of_different_sizes():
+    """The walk's launch asks for shared memory by the number of nodes: one thread's small tree must not lower the limit between the two
+    steps (limit, launch) of another thread's large one."""
+    errors = []
+
+    def work(n):
+        try:
+            torch.cuda.set_device(0)
+            b = wl.make_batch(**HEADS, l_P=9, ctx_lens=[[1] * n], l_q=1, seed=81, T=0.8, S=0.7, name="threads").to("cuda:0")
+            out = torch.zeros_like(b.q)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                plan = handle().attend_plan(**HEADS, k_pool=b.k_pool, v_pool=b.v_pool, q=b.q, out=out, requests=b.requests,
+                                            mode=libape.APE_PREFILL, tree=([[-1] * n], None))
+                ws = plan.alloc_workspace()
+                plan.attend(b.T, b.S, ws)
+                torch.cuda.current_stream().synchronize()
+                first = out.clone()
+                for i in range(4000):
+                    plan.attend(b.T, b.S, ws)
+                torch.cuda.current_stream().synchronize()
+                assert torch.equal(out, first)
+        except Exception as e:                                        # noqa: BLE001
+            errors.append(f"{n} nodes: {e!r}")
+
+    threads = [threading.Thread(target=work, args=(n,)) for n in (1600, 400)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not errors, errors
