@@ -1341,8 +1341,8 @@ int ape_selftest_timeout(ape_handle_t h, void* stream_v) {
     if (!h) return APE_ERR_INVALID_ARG;
     DeviceGuard guard(h->device);
     if (!guard.ok) return APE_ERR_CUDA;
-    ape_wait_probe_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream_v)>>>(h->d_status);
-    return cudaGetLastError() == cudaSuccess ? APE_OK : APE_ERR_CUDA;
+    return launch_kernel(false, ape_wait_probe_kernel, 1, 32, 0, static_cast<cudaStream_t>(stream_v), h->d_status) == cudaSuccess
+               ? APE_OK : APE_ERR_CUDA;
 }
 
 const char* ape_status_string(int s) {
@@ -1559,8 +1559,8 @@ int ape_selftest_timeout_noalloc(int device, void* stream_v) {
     int rc = noalloc_setup(device, &dv);              if (rc) return rc;
     DeviceGuard guard(device);
     if (!guard.ok) return APE_ERR_CUDA;
-    ape_wait_probe_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream_v)>>>(reinterpret_cast<int*>(dv->scratch));
-    return cudaGetLastError() == cudaSuccess ? APE_OK : APE_ERR_CUDA;
+    return launch_kernel(false, ape_wait_probe_kernel, 1, 32, 0, static_cast<cudaStream_t>(stream_v), reinterpret_cast<int*>(dv->scratch))
+                   == cudaSuccess ? APE_OK : APE_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -188,17 +188,23 @@ __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Launch with the programmatic attribute, so that the set-up of this kernel (block scheduling, barriers, tensor memory, first
-// records) overlaps the end of the one before it.  Every kernel launched through here calls pdl_wait first.
+// Launch a kernel and return the launch's own result.  (cudaGetLastError would also return, and so blame on this launch, what any
+// earlier call has left behind.)
+// early: with the programmatic attribute, so that the set-up of this kernel (block scheduling, barriers, tensor memory, first
+// records) overlaps the end of the one before it.  Every kernel launched this way calls pdl_wait first.
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t stream, const A&... args) {
+inline cudaError_t launch_kernel(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t stream, const A&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem_bytes; cfg.stream = stream;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = &attr; cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t stream, const A&... args) {
+    return launch_kernel(true, kernel, grid, block, smem_bytes, stream, args...);
 }
 
 __device__ __forceinline__ void prefetch_l1(const void* ptr) {

@@ -428,9 +428,7 @@ cudaError_t launch_shard_merge(const ShardMergeParams& p, cudaStream_t stream)
     const long long warps = static_cast<long long>(p.n_rows) * p.H_q;
     if (warps == 0) return cudaSuccess;
     const int blocks = static_cast<int>((warps * 32 + 255) / 256);
-    if (p.D == 128) ape_shard_merge_kernel<4><<<blocks, 256, 0, stream>>>(p);
-    else ape_shard_merge_kernel<2><<<blocks, 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_kernel(false, p.D == 128 ? ape_shard_merge_kernel<4> : ape_shard_merge_kernel<2>, blocks, 256, 0, stream, p);
 }
 
 namespace {
@@ -554,9 +552,11 @@ cudaError_t launch_node_bias(const NodeBiasParams& p, cudaStream_t stream)
     const size_t smem = static_cast<size_t>(p.max_nodes) * (kBiasRows * sizeof(float) + sizeof(DevBfsNode));
     if (p.max_nodes > 0 && smem <= p.smem_limit) {
         // (the device's limit, not this launch's size: another thread may be between its own two steps)
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(ape_node_bias_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(p.smem_limit)) != cudaSuccess)
-            return cudaGetLastError();
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(ape_node_bias_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(p.smem_limit));
+            if (e != cudaSuccess) return e;
+        }
         const dim3 grid(static_cast<unsigned>((p.max_rows + kBiasRows - 1) / kBiasRows), static_cast<unsigned>(p.n_req));
         return launch_pdl(ape_node_bias_smem_kernel, grid, kBiasWarps * 32, smem, stream, p);
     }

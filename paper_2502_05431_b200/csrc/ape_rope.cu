@@ -114,14 +114,11 @@ __global__ void __launch_bounds__(128) ape_append_kernel(const AppendParams p)
 
 cudaError_t launch_append(const AppendParams& p, cudaStream_t stream) {
     if (p.n_req <= 0) return cudaSuccess;
-    ape_append_kernel<<<p.n_req, 128, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_kernel(false, ape_append_kernel, p.n_req, 128, 0, stream, p);
 }
 
 cudaError_t launch_rope(int D, const RopeParams& p, int n_cta, cudaStream_t stream) {
-    if (D == 128) ape_rope_kernel<128><<<n_cta, kRopeThreads, 0, stream>>>(p);
-    else ape_rope_kernel<64><<<n_cta, kRopeThreads, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_kernel(false, D == 128 ? ape_rope_kernel<128> : ape_rope_kernel<64>, n_cta, kRopeThreads, 0, stream, p);
 }
 
 }  // namespace ape

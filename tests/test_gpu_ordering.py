@@ -1,4 +1,6 @@
 """What orders the parts of the library that run side by side: the warps of a block, the kernels of a call, calls on one stream."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -193,3 +195,35 @@ def test_decode_plans_of_other_head_layouts_leave_a_plan_usable():
     b, dev, plan, out, ws = plans[0]
     plan.attend(b.T, b.S, ws)
     compare(out.cpu(), oracle_attend(b, 0).out.float(), b.name)
+
+
+def test_a_failed_launch_is_not_blamed_on_a_later_call():
+    """Calls that fail on the host (here: on a stream whose capture has been invalidated, where every launch is refused) leave nothing
+    behind that makes a later, good call report an error."""
+    rt = C.CDLL("libcudart.so.12")
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=20, ctx_lens=[[64]], l_q=4, l_k=9, seed=67, T=0.8, S=0.9, name="blame").to("cuda:0")
+    out = torch.zeros_like(b.q)
+    make = lambda: handle().attend_plan(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool, q=b.q, out=out, requests=b.requests,  # noqa: E731
+                                        mode=libape.APE_PREFILL)
+    plan, rope = make(), libape.RopePlan(handle(), 128, 500000.0, [(0, 0, 20, 0)])
+    ws, dst = plan.alloc_workspace(), torch.zeros_like(b.k_pool)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert rt.cudaStreamBeginCapture(C.c_void_p(s.cuda_stream), 0) == 0
+    try:
+        with pytest.raises(libape.ApeError):
+            make()                                                 # allocates: not allowed, and ends the capture's validity
+        with pytest.raises(libape.ApeError) as e:
+            plan.attend(b.T, b.S, ws, stream=s)
+        assert e.value.code == -7
+    finally:
+        graph = C.c_void_p()
+        assert rt.cudaStreamEndCapture(C.c_void_p(s.cuda_stream), C.byref(graph)) != 0 and not graph.value
+        rt.cudaGetLastError()
+    rope.write(b.k_pool, dst, False)
+    part = [torch.zeros(1, 4, 32, 128, device="cuda:0"), torch.zeros(1, 4, 32, device="cuda:0")]
+    libape.merge_shards(handle(), H_q=32, H_kv=8, d=128, o_ctx_all=part[0], lse_ctx_all=part[1], o_oth=part[0][0], lse_oth=part[1][0], S=1.0,
+                        out=out)
+    plan.attend(b.T, b.S, ws)
+    torch.cuda.synchronize()
+    assert torch.equal(dst[:20], b.k_pool[:20]) and handle().get_status() == 0
