@@ -1075,7 +1075,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = b->n_stages; dp.status = p->h->d_status;
         dp.let_next_in = p->budget ? 0 : 1;
-        if (launch_decode(D, b->tm_k, b->tm_v, dp, b->n_cta, b->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+        if (launch_decode(D, b->tm_k, b->tm_v, dp, b->n_cta, b->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
         p->last_launches++;
         MergeParams mp;
         mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = nullptr; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = p->n_merge;
@@ -1101,7 +1101,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = p->n_stages; dp.status = p->h->d_status;
         dp.let_next_in = p->budget ? 0 : 1;
-        if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+        if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
     } else {
         AttnParams ap;
         ap.tiles = p->d_tiles; ap.items = p->d_items; ap.cta_item_begin = p->d_cta_begin; ap.reqs = p->d_reqs;
@@ -1535,7 +1535,8 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     dp.q = rows_desc(*q); dp.ws_o = ws_o; dp.ws_ml = ws_ml;
     dp.scale_oth_log2 = c * kLog2e; dp.scale_ctx_log2 = c / T * kLog2e;
     dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = n_stages; dp.status = reinterpret_cast<int*>(base); dp.let_next_in = 1;
-    if (launch_decode(D, tm_k, tm_v, dp, n_cta, smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+    // Not early: the records that the kernel reads in front of its dependency wait are those of the copy above, on this stream.
+    if (launch_decode(D, tm_k, tm_v, dp, n_cta, smem_bytes, false, stream) != cudaSuccess) return APE_ERR_CUDA;
     MergeParams mp;
     mp.groups = reinterpret_cast<const DevMerge*>(base + o_merge); mp.reqs = dp.reqs; mp.items = dp.items; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = static_cast<int32_t>(m.merge.size());
     mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = ws_o; mp.ws_ml = ws_ml; mp.out = rows_desc(*out); mp.lse_out = lse;

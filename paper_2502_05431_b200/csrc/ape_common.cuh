@@ -182,7 +182,8 @@ __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
 
 // Programmatic dependent launch: pdl_wait returns once every kernel launched before this one on the stream has completed
 // and its writes are visible; pdl_trigger lets the next kernel of the stream be set up on the SMs (its own pdl_wait
-// still holds it).  Only plan metadata, which is uploaded before any launch, may be read in front of pdl_wait.
+// still holds it).  Only plan metadata, which is uploaded before any launch, may be read in front of pdl_wait
+// (a kernel whose metadata was copied on the stream is launched without the attribute).
 // The attention and decode kernels of a plan made under an SM budget do not trigger: blocks of the next kernel, which wait with
 // their registers and shared memory taken, would sit on the SMs that the budget leaves to others for as long as the kernel runs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

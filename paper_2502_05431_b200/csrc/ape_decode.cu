@@ -299,9 +299,9 @@ int decode_pick_stages(int D, int G, size_t smem_limit) {
 }
 
 cudaError_t launch_decode(int D, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const DecodeParams& p,
-                          int n_cta, size_t smem_bytes, cudaStream_t stream)
+                          int n_cta, size_t smem_bytes, bool early, cudaStream_t stream)
 {
-    return launch_pdl(D == 128 ? ape_decode_kernel<128> : ape_decode_kernel<64>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
+    return launch_kernel(early, D == 128 ? ape_decode_kernel<128> : ape_decode_kernel<64>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
 }
 
 cudaError_t decode_set_smem_attr(int D, size_t smem_limit) {

@@ -30,8 +30,9 @@ size_t decode_smem_bytes(int D, int G, int n_stages);
 int decode_pick_stages(int D, int G, size_t smem_limit);
 // The limit of the kernel, not of a plan: launches of all head layouts share it, so it is always what decode_pick_stages was given.
 cudaError_t decode_set_smem_attr(int D, size_t smem_limit);
+// early: the blocks may be placed, and read their records, while the kernel before this one still runs
 cudaError_t launch_decode(int D, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const DecodeParams& p,
-                          int n_cta, size_t smem_bytes, cudaStream_t stream);
+                          int n_cta, size_t smem_bytes, bool early, cudaStream_t stream);
 
 // Tensor-core attention kernel shared by query prefill and context encoding.
 enum : int32_t {

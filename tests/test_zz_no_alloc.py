@@ -146,3 +146,27 @@ def test_noalloc_size_gate_counts_fused_spans():
     assert libape.decode_noalloc(out=out_a, requests=[many], want_status=True, **kw) == 0
     assert libape.decode_noalloc(out=out_b, requests=b.requests, want_status=True, **kw) == 0
     assert torch.equal(out_a, out_b) and not torch.isnan(out_a.float()).any()
+
+
+def test_noalloc_calls_of_different_batches_back_to_back():
+    """Every call copies its own tile lists and records over those of the call before, on the stream and with nothing to wait for in
+    between; each output must still be that of its own batch."""
+    runs = []
+    for i, (heads, lens) in enumerate([(LLAMA, [[256] * 10]), (dict(H_q=4, H_kv=1, d=64), [[70, 1, 129], [5]]), (LLAMA, [[2000], [64, 3], [700]]),
+                                       (dict(H_q=8, H_kv=8, d=128), [[33]])]):
+        b = wl.make_batch(**heads, l_P=10 * i, ctx_lens=lens, l_q=1, l_k=4, seed=90 + i, T=0.8, S=0.9, name=f"noalloc_{i}").to("cuda:0")
+        out = torch.full_like(b.q, float("nan"))
+        call = lambda b=b, heads=heads, out=out: libape.decode_noalloc(**heads, k_pool=b.k_pool, v_pool=b.v_pool, q=b.q, out=out,  # noqa: E731
+                                                                       requests=b.requests, T=b.T, S=b.S)
+        call()
+        torch.cuda.synchronize()
+        runs.append((call, out, out.clone()))
+    for _, out, _ in runs:
+        out.fill_(float("nan"))
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for call, _, _ in runs:
+            call()
+    torch.cuda.synchronize()
+    for _, out, first in runs:
+        assert not torch.isnan(first.float()).any() and torch.equal(out, first)
