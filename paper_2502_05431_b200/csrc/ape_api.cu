@@ -56,6 +56,7 @@ struct ape_plan_s {
     SplitMaps tm_split{};           // encode plans with split_r > 0
     int split_r = 0;
     bool o_via_tma = false;         // encode plans: tm_o describes the output rows
+    bool early = true;              // the attention kernel's blocks may be placed before the kernel in front of it has ended
     bool budget = false;            // made under an SM budget: the SMs that it leaves stay free while its kernels run
     bool alt_halves = false;        // context pass of a shared plan with at most 128 rows: the halves take alternate tiles
     int32_t last_launches = 0;
@@ -279,6 +280,20 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int 
         }
     }
     while (static_cast<int>(m.cta_begin.size()) < n_bins + 1) m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
+}
+
+// Whether an attention kernel's blocks may be placed while the kernel before it ends.  That saves a call 1 to 3 us, but the blocks
+// then go wherever an SM falls free instead of in order, and siblings, which stream the same tiles, cost more energy that way (the
+// likely reason: their tiles reach them through both halves of the L2).  A long call at the power limit pays for it in time.
+// Placed early / in order, 32 heads of 128, contexts of 256 tokens, back to back for 0.4 s:
+//   one block per group     200 contexts 0.966, 500 contexts 0.987
+//   two siblings            40 contexts (9 tiles a group) 0.941, 160 (35) 0.992, 500 (108) 1.007; 4 x 20 documents (71) 1.009
+//   four siblings           20 contexts (9) 0.980, 40 (18) 1.001, 160 (70) 1.008, 500 (217) 1.013; 512 rows, 30 contexts (26) 1.024
+// Heads of 64 stay below the power limit (four siblings, 54 tiles: 0.992).
+bool place_early(const std::vector<Run>& runs, int n_groups, int n_sib, int D) {
+    long long total = 0;
+    for (const auto& r : runs) total += r.t1 - r.t0;
+    return D < 128 || n_sib == 1 || total * n_sib < 96ll * n_groups;
 }
 
 // Nodes [n0, n1) of one request in breadth-first order: level by level, the children of a node next to each other.
@@ -605,6 +620,7 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                 }
             }
             assign_stream(runs, n_groups, p->n_sib, kAttnItemTiles, m, per_context != 0);
+            p->early = place_early(runs, n_groups, p->n_sib, D);
             p->n_cta = n_groups * p->n_sib;
             p->n_slots = static_cast<int>(m.items.size()) * p->n_sib;
             p->smem_bytes = attn_smem_bytes(D, kAttnPrefill);
@@ -732,6 +748,7 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
                 if (t1 > t0) runs_a.push_back(Run{0, hh, rb0, live, SEG_CTX, t0, t1, mi});
             }
         assign_stream(runs_a, n_groups, a->n_sib, kAttnItemTiles, ma);
+        a->early = place_early(runs_a, n_groups, a->n_sib, D);
         a->n_cta = n_groups * a->n_sib;
         a->n_slots = static_cast<int>(ma.items.size()) * a->n_sib;
         a->smem_bytes = attn_smem_bytes(D, a->alt_halves ? kAttnAlt : kAttnPrefill);
@@ -1066,7 +1083,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
             ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = a->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
             ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1; if (a->alt_halves) ap.mode = kAttnAlt;
-            if (launch_attn(D, a->tm_q, a->tm_k, a->tm_v, a->tm_q, a->tm_split, ap, a->n_cta, a->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+            if (launch_attn(D, a->tm_q, a->tm_k, a->tm_v, a->tm_q, a->tm_split, ap, a->n_cta, a->smem_bytes, a->early, stream) != cudaSuccess) return APE_ERR_CUDA;
             p->last_launches++;
         }
         DecodeParams dp;
@@ -1116,7 +1133,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             uint8_t* base = static_cast<uint8_t*>(workspace);
             ap.stat_rows = p->stat_rows;
             ap.mode = kAttnStats; ap.stats = reinterpret_cast<float2*>(base + p->off_stats);
-            if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+            if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, p->early, stream) != cudaSuccess) return APE_ERR_CUDA;
             NodeBiasParams nb;
             nb.nodes = p->d_nodes; nb.reqs = p->d_reqs; nb.req_node0 = p->d_req_node0; nb.bfs = p->d_bfs; nb.levels = p->d_levels; nb.n_req = static_cast<int32_t>(p->n_req);
             nb.stats = ap.stats; nb.mass = reinterpret_cast<float*>(base + p->off_mass); nb.bias = reinterpret_cast<float*>(base + p->off_bias);
@@ -1126,7 +1143,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             ap.mode = kAttnBias; ap.stats = nullptr; ap.bias = nb.bias;
             p->last_launches += 2;
         }
-        if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, stream) != cudaSuccess) return APE_ERR_CUDA;
+        if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, p->early, stream) != cudaSuccess) return APE_ERR_CUDA;
     }
     p->last_launches++;
 
@@ -1203,7 +1220,7 @@ int ape_encode_contexts(ape_plan_t p, void* workspace, size_t ws_bytes, void* st
     ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c * kLog2e;
     ap.G = p->G; ap.H_q = p->shape.n_q_heads; ap.n_sib = 1; ap.mode = kAttnEncode; ap.q_rows_are_pool = 1; ap.status = p->h->d_status;
     ap.o_via_tma = p->o_via_tma ? 1 : 0; ap.split_r = p->split_r; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1;
-    if (launch_attn(p->shape.head_dim, p->tm_q, p->tm_k, p->tm_v, p->tm_o, p->tm_split, ap, p->n_cta, p->smem_bytes,
+    if (launch_attn(p->shape.head_dim, p->tm_q, p->tm_k, p->tm_v, p->tm_o, p->tm_split, ap, p->n_cta, p->smem_bytes, p->early,
                     static_cast<cudaStream_t>(stream_v)) != cudaSuccess) return APE_ERR_CUDA;
     p->last_launches = 1;
     return APE_OK;

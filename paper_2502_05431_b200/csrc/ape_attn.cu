@@ -882,22 +882,22 @@ cudaError_t attn_set_smem_attr(int D, int mode, size_t smem_bytes) {
 
 template <int D>
 static cudaError_t launch_mode(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
-                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, cudaStream_t stream) {
+                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, bool early, cudaStream_t stream) {
     switch (p.mode) {
-        case kAttnPrefill: return launch_pdl(ape_attn_kernel<D, kAttnPrefill>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
-        case kAttnEncode:  return launch_pdl(ape_attn_kernel<D, kAttnEncode>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
-        case kAttnAlt:     return launch_pdl(ape_attn_kernel<D, kAttnAlt>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
-        case kAttnStats:   return launch_pdl(ape_attn_kernel<D, kAttnStats>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
-        case kAttnBias:    return launch_pdl(ape_attn_kernel<D, kAttnBias>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnPrefill: return launch_kernel(early, ape_attn_kernel<D, kAttnPrefill>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnEncode:  return launch_kernel(early, ape_attn_kernel<D, kAttnEncode>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnAlt:     return launch_kernel(early, ape_attn_kernel<D, kAttnAlt>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnStats:   return launch_kernel(early, ape_attn_kernel<D, kAttnStats>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
+        case kAttnBias:    return launch_kernel(early, ape_attn_kernel<D, kAttnBias>, n_cta, kThreads, smem_bytes, stream, tm_q, tm_k, tm_v, tm_o, split, p);
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_attn(int D, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
-                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, cudaStream_t stream)
+                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, bool early, cudaStream_t stream)
 {
-    return D == 128 ? launch_mode<128>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream)
-                    : launch_mode<64>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, stream);
+    return D == 128 ? launch_mode<128>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, early, stream)
+                    : launch_mode<64>(tm_q, tm_k, tm_v, tm_o, split, p, n_cta, smem_bytes, early, stream);
 }
 
 }  // namespace ape

@@ -76,7 +76,7 @@ cudaError_t attn_set_smem_attr(int D, int mode, size_t smem_bytes);
 // K and V boxes of split_r rows (prefix part) and 128 - split_r rows (context part) for TILE_SPLIT tiles
 struct SplitMaps { CUtensorMap ka, kb, va, vb; };
 cudaError_t launch_attn(int D, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const CUtensorMap& tm_o,
-                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, cudaStream_t stream);
+                        const SplitMaps& split, const AttnParams& p, int n_cta, size_t smem_bytes, bool early, cudaStream_t stream);
 
 // Merge of the partials: hierarchical softmax identity inside each segment, then Eq. 5's scaling factor.
 struct MergeParams {
