@@ -1098,7 +1098,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = nullptr; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = p->n_merge;
         mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = b_o; mp.ws_ml = b_ml;
         mp.ws_o_ctx = a_o; mp.ws_ml_ctx = a_ml; mp.rows_per_slot_ctx = a->alt_halves ? kAttnRows / 2 : kAttnRows;
-        mp.out = rows_desc(p->out); mp.lse_out = p->lse; mp.S = S; mp.G = G; mp.H_q = p->shape.n_q_heads; mp.D = D;
+        mp.out = rows_desc(p->out); mp.lse_out = p->lse; mp.S = S; mp.G = G; mp.H_q = p->shape.n_q_heads; mp.D = D; mp.n_sm = p->h->n_sm_device;
         mp.part_o_ctx = part ? part->o_ctx : nullptr; mp.part_lse_ctx = part ? part->lse_ctx : nullptr;
         mp.part_o_oth = part ? part->o_oth : nullptr; mp.part_lse_oth = part ? part->lse_oth : nullptr;
         if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
@@ -1151,7 +1151,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
     mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = p->d_items; mp.per_context = p->two_pass ? 0 : p->per_context; mp.nodes = p->d_nodes; mp.n_groups = p->n_merge; mp.rows_per_slot = rows_per_slot;
     mp.tokens_per_block = rows_per_slot / G; mp.ws_o = ws_o; mp.ws_ml = ws_ml; mp.out = rows_desc(p->out); mp.lse_out = p->lse;
     mp.ws_o_ctx = ws_o; mp.ws_ml_ctx = ws_ml; mp.rows_per_slot_ctx = rows_per_slot;
-    mp.S = p->two_pass ? 1.f : S; mp.G = G; mp.H_q = p->shape.n_q_heads; mp.D = D;
+    mp.S = p->two_pass ? 1.f : S; mp.G = G; mp.H_q = p->shape.n_q_heads; mp.D = D; mp.n_sm = p->h->n_sm_device;
     mp.part_o_ctx = part ? part->o_ctx : nullptr; mp.part_lse_ctx = part ? part->lse_ctx : nullptr;
     mp.part_o_oth = part ? part->o_oth : nullptr; mp.part_lse_oth = part ? part->lse_oth : nullptr;
     if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
@@ -1559,7 +1559,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = ws_o; mp.ws_ml = ws_ml; mp.out = rows_desc(*out); mp.lse_out = lse;
     mp.ws_o_ctx = ws_o; mp.ws_ml_ctx = ws_ml; mp.rows_per_slot_ctx = G;
     mp.part_o_ctx = nullptr; mp.part_lse_ctx = nullptr; mp.part_o_oth = nullptr; mp.part_lse_oth = nullptr;
-    mp.S = S; mp.G = G; mp.H_q = shape->n_q_heads; mp.D = D;
+    mp.S = S; mp.G = G; mp.H_q = shape->n_q_heads; mp.D = D; mp.n_sm = dv->h.n_sm;
     if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
     if (device_status != nullptr) {
         // the caller asked for the status word: this makes the call synchronous; a word that was set is cleared once read

@@ -108,6 +108,7 @@ struct MergeParams {
     int32_t G;
     int32_t H_q;
     int32_t D;
+    int32_t n_sm;                    // SMs of the device (an SM budget does not limit the merge)
 };
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
 

@@ -571,12 +571,12 @@ cudaError_t launch_merge_vec(const MergeParams& p, long long rows, cudaStream_t 
     if (p.per_context != 0)
         return launch_pdl(p.per_context == 2 ? ape_merge_nodes_kernel<VEC, true> : ape_merge_nodes_kernel<VEC, false>,
                           static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
-    // Eight warps per row while all rows' blocks are resident at once (148 SMs x 4 blocks): with few rows, as in a decode step,
+    // Eight warps per row while all rows' blocks are resident at once (four to an SM): with few rows, as in a decode step,
     // it is the latency of a row's partials that counts (4 requests over 20K tokens each: 62.1 us per step with one warp per row,
     // 60.5 with eight; 16 requests over shared 128K tokens: 129.0 and 124.4).  With more rows the warps of other rows hide it,
     // and sharing a row only adds the meeting in shared memory (64 rows over 10 x 256 tokens, 2048 rows to merge: 19.4 us with
     // one, 24.4 with eight; 4 x 128 rows over 20K tokens: 212 and 254).
-    if (rows <= 4 * 148) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
+    if (rows <= 4ll * p.n_sm) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
     return launch_pdl(ape_merge_kernel<VEC, 1>, static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
 }
 }  // namespace
