@@ -33,9 +33,16 @@ def test_partials_per_row(n_sm, mode, d, l_q):
 
 
 def test_more_partials_than_one_round_of_lanes():
-    """One KV head and a shared-context batch of at most 128 rows: two partials per thread block, 296 per row."""
-    b = wl.share_contexts(wl.make_batch(H_q=4, H_kv=1, d=128, l_P=5, ctx_lens=[[40000]] + [[1]] * 2, l_q=1, l_k=9, seed=32,
+    """One KV head and a shared-context batch of at most 128 rows, two tiles per thread block: two partials per block, 296 per row on
+    148 SMs, of which the eight warps of a row take 256 in one round."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    b = wl.share_contexts(wl.make_batch(H_q=4, H_kv=1, d=128, l_P=5, ctx_lens=[[2 * n_sm * 128]] + [[1]] * 2, l_q=1, l_k=9, seed=32,
                                         T=0.9, S=0.8, name="merge_296"))
+    dev = b.to("cuda:0")
+    plan = handle().attend_plan(H_q=4, H_kv=1, d=128, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=torch.zeros_like(dev.q),
+                                requests=b.requests, mode=libape.APE_DECODE, shared=True)
+    # a slot holds two partials of 128 rows; what the requests' own segments add is less than three slots
+    assert 2 * (plan.workspace_bytes // (256 * (128 + 2) * 4) - 3) > 256
     _check(b, libape.APE_DECODE, shared=True)
 
 
