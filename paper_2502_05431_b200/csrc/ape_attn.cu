@@ -617,7 +617,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // phase n-1 of half 1; phase n of half 1 follows phase n of half 0 (both halves see the same tiles).
                 // (Alternating halves work on different tiles, with different numbers of them: no turns there.  Encode's items have
                 // one to three tiles, and a turn mostly makes a half wait whose partner is at the end of an item: 500 x 256
-                // tokens 897 us with turns, 865 without; the long items of prefill lose 11% without.  In the statistics pass nothing but the
+                // tokens 871 us with turns, 837 without, back to back at the power limit (861 and 793 in bursts of 20 ms; ten
+                // contexts, two or three items per block, 22.3 and 22.9); the long items of prefill lose 11% without.  In the statistics pass nothing but the
                 // exponentials is on a half's chain, and without turns the two halves fill each other's gaps: 386 us, now 339, for 256
                 // rows over 128K tokens.)
                 if (TURNS) {
