@@ -92,12 +92,15 @@ def _same_with_and_without_waits(launches, bufs):
     assert handle().get_status() == 0
 
 
-@pytest.mark.parametrize("mode,l_q,n_req", [(libape.APE_DECODE, 1, 4), (libape.APE_PREFILL, 64, 1), (libape.APE_PREFILL, 200, 1)])
-def test_calls_that_feed_each_other(mode, l_q, n_req):
+@pytest.mark.parametrize("mode,l_q,n_req,longest", [
+    (libape.APE_DECODE, 1, 4, 256), (libape.APE_PREFILL, 64, 1, 256), (libape.APE_PREFILL, 200, 1, 256),
+    (libape.APE_PREFILL, 200, 1, 18000),       # siblings and 30 tiles a group: the attention kernel is launched in order
+])
+def test_calls_that_feed_each_other(mode, l_q, n_req, longest):
     """The output of a call is the query of the next, all calls share one workspace, and no kernel of another library stands between
     them: what a kernel reads too early is an older query, partial or bias.  All plan kinds, each call over contexts of its own."""
-    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=30, ctx_lens=[[256, 70, 130, 64] * 12] * n_req, l_q=l_q, l_k=l_q + 5, seed=62, T=0.7, S=0.8,
-                      name="chain").to("cuda:0")
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=30, ctx_lens=[[longest, 70, 130, 64] * 12] * n_req, l_q=l_q, l_k=l_q + 5, seed=62, T=0.7, S=0.8,
+                      name="chain", device="cuda:0")
     b.v_pool *= 8                              # (large outputs, a high logit scale: a call's query decides its result)
     bufs = [b.q, torch.zeros_like(b.q)]
     forms = [dict(), dict(per_context=True), dict(tree=([[-1, 0, 0, 0]] * n_req, None))]
