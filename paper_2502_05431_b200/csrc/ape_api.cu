@@ -346,16 +346,19 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
 }
 
 // Whether a plan takes the cluster form (limit: tiles of its largest block), and with which size: all clusters must be on the device at once (of 16 blocks seven fit, of 10
-// eleven, of 8 fifteen: a cluster sits inside one part of the chip) and within the SM budget; among the sizes that leave the largest
-// block the fewest tiles the smallest; and that block may have kClusterTiles tiles more than the largest of the ordinary form, whose
-// merge kernel costs about as much.  In us per call, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
+// eleven, of 8 fifteen: a cluster sits inside one part of the chip); among the sizes that leave the largest block the fewest tiles
+// the smallest; and that block may have kClusterTiles tiles more than the largest of the ordinary form, whose merge kernel costs about
+// as much.  Never under an SM budget: the budget leaves SMs to a kernel that runs beside, which takes some of every part, and a
+// cluster waits until it finds as many free SMs in one part as it has blocks; single blocks take the SMs that are left.
+// In us per call, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
 //   1 request   1 x 64 tokens 5.1 / 3.7 (2 / 1)   10 contexts 5.9 / 5.7 (3 / 5)   20: 7.5 / 7.5 (5 / 9: stays ordinary)   40: 9.3 / 11.3 (10 / 18)
 //   2 requests  4 contexts 6.3 / 5.1 (3 / 4)   10: 7.5 / 7.0 (5 / 8)   20: 9.6 / 10.4 (10 / 15)      4 requests  4 contexts 7.4 / 6.2
 constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 12;
-ClusterSplit pick_cluster(const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], int n_sm, long long limit) {
+ClusterSplit pick_cluster(const ape_handle_s* h, const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], long long limit) {
     ClusterSplit best;
+    if (h->n_sm < h->n_sm_device) return best;
     for (int i = 0; i < kClusterSizes; ++i) {
-        if (n_groups > resident[i] || n_groups * kCluster[i] > n_sm) continue;
+        if (n_groups > resident[i] || n_groups * kCluster[i] > h->n_sm) continue;
         const long long u = cluster_largest(runs, kCluster[i]);
         if (u > 0 && (best.size == 0 || u <= best.largest)) best = ClusterSplit{kCluster[i], u};
     }
@@ -641,7 +644,7 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             p->n_slots = static_cast<int>(m.items.size());
             if (per_context == 0) {
                 const int n_groups = n_req * H_kv;
-                const ClusterSplit cs = pick_cluster(runs, n_groups, h->decode_clusters, h->n_sm, largest_bin(m) + kClusterTiles);
+                const ClusterSplit cs = pick_cluster(h, runs, n_groups, h->decode_clusters, largest_bin(m) + kClusterTiles);
                 if (cs.size > 0) {
                     // (the workspace that the ordinary form needs is still asked for: a call is refused for the same reasons in both)
                     m.items.clear();
@@ -756,7 +759,7 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                 }
                 const int n_blocks = static_cast<int>(ms.merge.size());
                 const long long most = largest_bin(m);
-                const ClusterSplit cs = pick_cluster(runs_s, n_blocks, h->attn_clusters, h->n_sm, 2 * most - most / 4);
+                const ClusterSplit cs = pick_cluster(h, runs_s, n_blocks, h->attn_clusters, 2 * most - most / 4);
                 if (cs.size > 0) {
                     m.items.clear(); m.merge = std::move(ms.merge);
                     assign_clusters(runs_s, cs, m);

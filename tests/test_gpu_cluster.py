@@ -19,10 +19,10 @@ def _ordinary(b, mode, **kw):
         handle().set_sm_budget(0)
 
 
-def _kernels(b, mode):
+def _kernels(b, mode, **how):
     dev = b.to("cuda:0")
     plan = handle().attend_plan(H_q=b.H_q, H_kv=b.H_kv, d=b.d, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=torch.zeros_like(dev.q),
-                                requests=b.requests, mode=mode)
+                                requests=b.requests, mode=mode, **how)
     plan.attend(b.T, b.S, plan.alloc_workspace())
     torch.cuda.synchronize()
     return plan.last_kernels()
@@ -79,3 +79,20 @@ def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
         sl = slice(rq.q_start, rq.q_start + rq.q_len)
         compare(out[sl], ref.out.float(), f"req {r}")
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("budget", [2, 40, 147])
+@pytest.mark.parametrize("mode,l_q,shared", [(libape.APE_DECODE, 1, False), (libape.APE_DECODE, 1, True), (libape.APE_PREFILL, 16, False)])
+def test_no_clusters_under_a_budget(budget, mode, l_q, shared):
+    """A cluster waits for free SMs in one part of the chip, and the kernel that the budget is for takes some of every part."""
+    b = wl.make_batch(H_q=4, H_kv=1, d=128, l_P=8, ctx_lens=[[64] * 4], l_q=l_q, seed=45, T=0.8, S=0.7, name="budget")
+    assert _kernels(b, mode, shared=shared) == 1
+    handle().set_sm_budget(budget)
+    try:
+        assert _kernels(b, mode, shared=shared) == 2
+        out, lse, _ = gpu_attend(b, mode, shared=shared)
+    finally:
+        handle().set_sm_budget(0)
+    ref = oracle_attend(b, 0)
+    compare(out, ref.out.float(), f"budget {budget}")
+    assert (lse.double() - ref.lse).abs().max().item() < 2e-3
