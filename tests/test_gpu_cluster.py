@@ -65,6 +65,19 @@ def test_shared_contexts_read_by_every_request_or_once(n_req, lens, budget):
         assert (lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("n_req,n_ctx,length,gap,kernels", [(8, 120, 8, 3, 3), (8, 120, 8, 0, 2), (2, 120, 8, 3, 2), (4, 60, 129, 1, 3), (4, 30, 128, 0, 2)])
+def test_shared_contexts_of_short_spans(n_req, n_ctx, length, gap, kernels):
+    """Spans that touch are one span; with gaps between them each is a tile of its own, for every request that reads it itself."""
+    b = wl.share_contexts(wl.make_batch(H_q=32, H_kv=8, d=128, l_P=7, ctx_lens=[[length] * n_ctx] * n_req, l_q=1, l_k=3, gap=gap, seed=46, T=0.8,
+                                        S=0.7, name="spans"))
+    assert _kernels(b, libape.APE_DECODE, shared=True) == kernels
+    out, lse, _ = gpu_attend(b, libape.APE_DECODE, shared=True)
+    for r in (0, n_req - 1):
+        ref = oracle_attend(b, r)
+        compare(out[r:r + 1], ref.out.float(), f"req {r}")
+        assert (lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
+
+
 @pytest.mark.parametrize("H_q,H_kv,d", [(32, 8, 128), (4, 1, 64), (16, 1, 128), (8, 8, 64)])
 @pytest.mark.parametrize("n_req,ctx,l_P,l_q,l_k,gap", [(1, [], 0, 1, 1, 0), (1, [64] * 4, 16, 16, 16, 0), (2, [1, 130, 200], 70, 9, 140, 2),
                                                        (1, [900], 128, 33, 33, 0), (1, [129] * 3, 5, 129, 129, 1)])
