@@ -671,16 +671,31 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             const int n_groups = std::max(1, h->n_sm / p->n_sib);
             // Few nodes, and sibling groups enough that every run gets one of its own: one pass with a partial per node (a node's end costs
             // nothing then) and the merge that walks the nodes, instead of statistics, biases, pass and merge.
-            // In us, two passes / one: 2 requests x 6 contexts of 59 tokens 19.0 / 14.4, 6 contexts of 1,500 tokens and 64 rows 65 / 27, a tree of
-            // 5 x 256 tokens 22.8 / 24.5 (its walk is longer).  A row's walk grows with its nodes: no more than six.
+            // In us, two passes / one: 2 requests x 6 contexts of 59 tokens 19.0 / 14.4, 6 contexts of 1,500 tokens and 64 rows 65 / 27.
+            // A row's walk grows with its nodes: no more than six.
+            // A tree's walk is longer: 0.65 per node, 0.75 more per wave of 16 rows per SM that walk (1.75 from the third wave on), 0.05 per
+            // partial of a row (half of each for heads of 64), against 3.4 for the two kernels saved and 1 per tile of the longest node, which no
+            // block of the statistics pass shares with another.  The weights are fitted to 411 trees of one to six nodes: six of those that
+            // this line sends through one pass were more than 1% slower there (at most 5.7%), and six that it does not would have gained more
+            // than 5% (at most 10%).  In us, two passes / one: 64 rows, three nodes of 256 tokens 22.1 / 19.4, six 23.5 / 26.0, five of 2,000
+            // 78 / 39; 128 rows, five of 256 25.3 / 32.1, of 2,000 79.6 / 68.8.
             bool one_pass = per_context != 0;
-            long long run_groups = 0;
+            long long run_groups = 0, rows_all = 0, most_nodes = 0, most_tiles = 0, longest = 0, row_groups = 0;
             for (int r = 0; r < n_req && one_pass; ++r) {
-                long long n = 0;
-                for (int i = 0; i < reqs[r].n_ctx; ++i) n += reqs[r].ctx[i].len > 0 ? 1 : 0;
+                long long n = 0, tiles = 0;
+                for (int i = 0; i < reqs[r].n_ctx; ++i) {
+                    const long long t = (reqs[r].ctx[i].len + kAttnTileN - 1) / kAttnTileN;
+                    n += t > 0 ? 1 : 0; tiles += t; longest = std::max(longest, t);
+                }
                 if (n > 0) p->one_pass = true;
-                run_groups += (n + 1) * H_kv * (((reqs[r].q_len + TB - 1) / TB + p->n_sib - 1) / p->n_sib);
+                const long long mine = H_kv * (((reqs[r].q_len + TB - 1) / TB + p->n_sib - 1) / p->n_sib);
+                row_groups += mine; run_groups += (n + 1) * mine;
+                rows_all += reqs[r].q_len * shape->n_q_heads; most_nodes = std::max(most_nodes, n); most_tiles = std::max(most_tiles, tiles);
                 one_pass = n <= kOnePassNodes && run_groups <= n_groups;
+            }
+            if (per_context == 2) {
+                const double waves = rows_all / (16.0 * h->n_sm_device), partials = static_cast<double>(std::min(most_tiles, std::max(most_nodes, n_groups / std::max(1ll, row_groups))));
+                one_pass = one_pass && (most_nodes * (0.65 + 0.75 * waves + std::max(waves - 2.0, 0.0)) + 0.05 * partials) * D / 128 <= 3.4 + longest;
             }
             p->one_pass = p->one_pass && one_pass;
             int64_t row_base = 0;                          // query rows of the requests before this one

@@ -1,6 +1,7 @@
 """Prefill of the per-context form and of trees with so few nodes that one pass with a partial per node serves: node counts on both sides of
 that line, ragged and empty nodes, against the oracle and against the two-pass form, which an SM budget of one selects."""
 import pytest
+import torch
 
 from oracle import ape_oracle as orc
 from paper_2502_05431_b200 import libape
@@ -34,4 +35,31 @@ def test_few_nodes(form, kw):
         ref = orc.attend(q, p, c, k, b.T, b.S, per_context=True) if form == "per_context" else orc.attend_tree(q, p, c, k, b.T, b.S, parents[r], None)
         sl = slice(rq.q_start, rq.q_start + rq.q_len)
         compare(out[sl], ref.out.float(), f"{form} req {r}")
+        assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("H_q,H_kv,d,n_req,nodes,l_q,kernels", [
+    (32, 8, 128, 1, [256] * 3, 64, 2), (32, 8, 128, 1, [256] * 5, 64, 4),          # 4.2 against 5.4, 7.0 against 5.4
+    (32, 8, 128, 1, [512] * 5, 128, 4), (32, 8, 128, 1, [1100] * 5, 128, 2),       # two waves of rows: 10.2 against 7.4 and 12.4
+    (32, 8, 128, 2, [31] * 3, 37, 2), (32, 8, 128, 2, [31] * 3, 38, 4),            # 4.35 and 4.41 against 4.4
+    (8, 8, 128, 1, [40] * 4, 3, 2),
+    (8, 2, 64, 1, [256] * 6, 64, 2), (8, 2, 64, 1, [100] * 6, 64, 2), (8, 2, 64, 1, [100] * 6, 400, 4),
+])
+def test_trees_whose_walk_is_worth_it(H_q, H_kv, d, n_req, nodes, l_q, kernels):
+    """Where the walk over a tree's nodes costs more than the two kernels and the pass that it saves (148 SMs), the plan keeps them."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the rows of a wave are those of 148 SMs")
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=20, ctx_lens=[nodes] * n_req, l_q=l_q, seed=52, T=0.8, S=0.6, name="walk")
+    parents = [[-1] + [0] * (len(nodes) - 1)] * n_req
+    dev = b.to("cuda:0")
+    plan = handle().attend_plan(H_q=H_q, H_kv=H_kv, d=d, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=torch.zeros_like(dev.q),
+                                requests=b.requests, mode=libape.APE_PREFILL, tree=(parents, None))
+    plan.attend(b.T, b.S, plan.alloc_workspace())
+    torch.cuda.synchronize()
+    assert plan.last_kernels() == kernels
+    out, lse, _ = gpu_attend(b, libape.APE_PREFILL, tree=(parents, None))
+    for r, rq in enumerate(b.requests):
+        ref = orc.attend_tree(*b.views(r), b.T, b.S, parents[r], None)
+        sl = slice(rq.q_start, rq.q_start + rq.q_len)
+        compare(out[sl], ref.out.float(), f"req {r}")
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
