@@ -319,6 +319,15 @@ long long cluster_largest(const std::vector<Run>& runs, int size) {        // ti
     }
     return worst;
 }
+long long cluster_partials(const std::vector<Run>& runs, const ClusterSplit& cs) {     // of the cluster with the most
+    long long most = 0;
+    for (size_t i = 0, j; i < runs.size(); i = j) {
+        long long n = 0;
+        for (j = i; j < runs.size() && runs[j].merge0 == runs[i].merge0; ++j) n += (runs[j].t1 - runs[j].t0 + cs.largest - 1) / cs.largest;
+        most = std::max(most, n);
+    }
+    return most;
+}
 void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostMeta& m) {
     m.cta_begin.assign(1, 0);
     for (size_t i = 0, j; i < runs.size(); i = j) {
@@ -353,12 +362,12 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
 // In us per call, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
 //   1 request   1 x 64 tokens 5.1 / 3.7 (2 / 1)   10 contexts 5.9 / 5.7 (3 / 5)   20: 7.5 / 7.5 (5 / 9: stays ordinary)   40: 9.3 / 11.3 (10 / 18)
 //   2 requests  4 contexts 6.3 / 5.1 (3 / 4)   10: 7.5 / 7.0 (5 / 8)   20: 9.6 / 10.4 (10 / 15)      4 requests  4 contexts 7.4 / 6.2
-constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 12;
-ClusterSplit pick_cluster(const ape_handle_s* h, const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], long long limit) {
+constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 12, kFewBlocks = 6;
+ClusterSplit pick_cluster(const ape_handle_s* h, const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], long long limit, int max_size = kCluster[0]) {
     ClusterSplit best;
     if (h->n_sm < h->n_sm_device) return best;
     for (int i = 0; i < kClusterSizes; ++i) {
-        if (n_groups > resident[i] || n_groups * kCluster[i] > h->n_sm) continue;
+        if (n_groups > resident[i] || n_groups * kCluster[i] > h->n_sm || kCluster[i] > max_size) continue;
         const long long u = cluster_largest(runs, kCluster[i]);
         if (u > 0 && (best.size == 0 || u <= best.largest)) best = ClusterSplit{kCluster[i], u};
     }
@@ -758,6 +767,12 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                 // the ordinary form's largest in about the same time, a little less for long ones (16 tiles against 31: 38.3 / 40.4 us).
                 // Ordinary / cluster, us per call: 4 x 64 tokens 8.2 / 6.9, 64 rows over 10 contexts of 256 16.5 / 14.4, 2 x 16 rows over
                 // 10 contexts 16.5 / 13.1, 4 x 5 rows over 24 contexts of 284 44.5 / 34.1, 128 rows over 10 contexts 17.6 / 17.6.
+                // A row's merge reads the partials of all blocks, three at a time, and with few row blocks the ordinary form has few rows to merge and
+                // leaves more of the chip to the tiles.  So clusters of more than six blocks only where the partials and the rows of a row block
+                // stay below a line that rises with the number of row blocks; else at most six blocks, all of one tile when there are fewer than
+                // four row blocks.  One KV head, one row block, ordinary / cluster: 128 rows, 10 tiles 9.9 / 11.0, 20 tiles 9.9 / 12.1, 16 rows, 10 tiles
+                // 9.1 / 8.3; eight heads of 40 rows, 20 tiles 14.8 / 11.1.  Of 329 calls with such clusters, 226 pass the line: six of
+                // them are more than 1.5% slower (one 7%), and 14 of the others would be more than 5% faster (none 10%).
                 const int TS = kAttnRows / 2 / G;
                 std::vector<Run> runs_s;
                 HostMeta ms;
@@ -773,8 +788,13 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                     }
                 }
                 const int n_blocks = static_cast<int>(ms.merge.size());
-                const long long most = largest_bin(m);
-                const ClusterSplit cs = pick_cluster(h, runs_s, n_blocks, h->attn_clusters, 2 * most - most / 4);
+                const long long most = largest_bin(m), limit = 2 * most - most / 4;
+                ClusterSplit cs = pick_cluster(h, runs_s, n_blocks, h->attn_clusters, limit);
+                if (cs.size > kFewBlocks) {
+                    const double live = std::min(kAttnRows / 2, p->max_rows / H_kv);
+                    if (cluster_partials(runs_s, cs) + 6.0 * live / (kAttnRows / 2) > 11.6 + 1.2 * std::min(n_blocks, 8))
+                        cs = pick_cluster(h, runs_s, n_blocks, h->attn_clusters, n_blocks < 4 ? 1 : limit, kFewBlocks);
+                }
                 if (cs.size > 0) {
                     m.items.clear(); m.merge = std::move(ms.merge);
                     assign_clusters(runs_s, cs, m);

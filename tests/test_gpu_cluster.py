@@ -94,6 +94,23 @@ def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("H_q,H_kv,d,n_ctx,length,l_q,kernels", [
+    (32, 8, 128, 10, 256, 64, 1), (16, 1, 128, 1, 512, 8, 1), (16, 1, 128, 1, 513, 8, 2),      # one row block of 128 rows: six tiles, seven
+    (16, 1, 128, 1, 1200, 1, 1), (16, 1, 128, 1, 1281, 1, 2), (4, 1, 64, 1, 3000, 40, 2),      # of 16 rows: 12 and 13 tiles
+    (16, 4, 128, 1, 2300, 16, 1), (16, 4, 128, 1, 3000, 8, 1), (16, 4, 128, 1, 3000, 32, 2),   # four row blocks: 10 partials, 13 of 32 and of 128 rows
+])
+def test_prefill_takes_clusters_where_they_are_faster(H_q, H_kv, d, n_ctx, length, l_q, kernels):
+    """Large clusters merge slowly: only for several row blocks of few rows, small ones wherever the tiles fit (148 SMs)."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the split is that of 148 SMs")
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=64, ctx_lens=[[length] * n_ctx], l_q=l_q, seed=47, T=0.8, S=0.7, name="line")
+    assert _kernels(b, libape.APE_PREFILL) == kernels
+    out, lse, _ = gpu_attend(b, libape.APE_PREFILL)
+    ref = oracle_attend(b, 0)
+    compare(out, ref.out.float(), "line")
+    assert (lse.double() - ref.lse).abs().max().item() < 2e-3
+
+
 @pytest.mark.parametrize("budget", [2, 40, 147])
 @pytest.mark.parametrize("mode,l_q,shared", [(libape.APE_DECODE, 1, False), (libape.APE_DECODE, 1, True), (libape.APE_PREFILL, 16, False)])
 def test_no_clusters_under_a_budget(budget, mode, l_q, shared):
