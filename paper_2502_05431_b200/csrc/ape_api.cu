@@ -83,6 +83,7 @@ struct ape_plan_s {
     ape_plan_s* child_oth = nullptr;
     bool plain = false;              // shared plan whose requests read the contexts themselves: child_oth is an ordinary decode plan
     int plain_steps = 0;         // ... and the steps that its last_launches counts
+    bool rest_first = false;         // shared plan: the per-request rest goes in front of the context pass
     // decode plans: what the host-buffer step needs (staging for the new token's Q is the plan's Q tensor itself)
     int n_req = 0;
     std::vector<int64_t> q_rows;     // Q / O row of every request
@@ -979,6 +980,9 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
             return APE_OK;
         }
 
+        long long rest_tiles = 0;
+        for (const auto& r : runs_b) rest_tiles += r.t1 - r.t0;
+        p->rest_first = D == 128 && 4 * rest_tiles >= (a->alt_halves ? 7ll : 4ll) * h->n_sm;
         a->smem_bytes = attn_smem_bytes(D, a->alt_halves ? kAttnAlt : kAttnPrefill);
         rc = make_map(h, &a->tm_k, pool->k, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, kAttnTileN);
         if (!rc) rc = make_map(h, &a->tm_v, pool->v, D, H_kv, pool->n_tokens, pool->head_stride, pool->token_stride, 1, kAttnTileN);
@@ -1295,9 +1299,13 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         return rc;
     }
     if (p->kind == PLAN_SHARED) {
-        // the per-request rest, the context pass of all requests at once beside it, then one merge that reads both sets of partials.  The rest
-        // first, so that its short blocks start at once and the context pass's blocks follow one by one as they end, without a launch
-        // between them (16 requests: 40 contexts 21.7 -> 19.5 us, 500 contexts 116.9 -> 115.4; 8 requests over 16 x 23 tokens 12.9 -> 10.4).
+        // The per-request rest and the context pass of all requests at once, then one merge that reads both sets of partials.  With the rest
+        // first, its short blocks start at once and the context pass's blocks follow one by one as they end, without a launch between them
+        // (16 requests: 500 contexts 118.5 -> 116.2; 22 requests over 39 contexts of 48 tokens 24.3 -> 22.6; 24 requests of 8 / 2 heads over 128K
+        // tokens 39.6 -> 38.0).  But the context pass's own start (barriers, tensor memory, records) then comes after the rest instead of
+        // under the merge before it, and a small rest does not make up for that: with alternating halves less than 1.75 tiles per SM (8 requests
+        // of 16 / 1 heads over 69K tokens 23.6 -> 26.6, 4 of 8 / 2 22.1 -> 22.9; 12 of 16 / 4 with 1.95 tiles 16.3 -> 15.6), otherwise less than one
+        // (12 requests of 16 / 1 heads 24.1 -> 25.1, 24 with 1.6 tiles 39.1 -> 38.4); nor any with heads of 64 (32 requests over 100K tokens 26.4 -> 27.1).
         // SMs of its own for the rest, a third more than its share of the bytes, were slower (500 contexts 119.5 -> 123.6, 40 contexts 19.5 -> 21.0):
         // the context pass needs all of them.
         ape_plan_t a = p->child_ctx, b = p->child_oth;
@@ -1315,8 +1323,12 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = b->n_stages; dp.status = p->h->d_status;
         dp.let_next_in = p->budget ? 0 : 1;
-        if (launch_decode(D, b->tm_k, b->tm_v, dp, b->n_cta, b->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
-        p->last_launches++;
+        auto launch_rest = [&] {
+            if (launch_decode(D, b->tm_k, b->tm_v, dp, b->n_cta, b->smem_bytes, true, stream) != cudaSuccess) return false;
+            p->last_launches++;
+            return true;
+        };
+        if (p->rest_first && !launch_rest()) return APE_ERR_CUDA;
         if (a->n_items > 0) {
             AttnParams ap{};
             ap.tiles = a->d_tiles; ap.items = a->d_items; ap.cta_item_begin = a->d_cta_begin; ap.reqs = a->d_reqs;
@@ -1324,10 +1336,11 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
             ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
             ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = a->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
             ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1; if (a->alt_halves) ap.mode = kAttnAlt;
-            ap.wait_late = a->early ? 1 : 0;           // beside the kernel in front of it, where it is placed early at all
+            ap.wait_late = (p->rest_first && a->early) ? 1 : 0;    // beside the kernel in front of it, where it is placed early at all
             if (launch_attn(D, a->tm_q, a->tm_k, a->tm_v, a->tm_q, a->tm_split, ap, a->n_cta, a->smem_bytes, a->early, stream) != cudaSuccess) return APE_ERR_CUDA;
             p->last_launches++;
         }
+        if (!p->rest_first && !launch_rest()) return APE_ERR_CUDA;
         MergeParams mp;
         mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = nullptr; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = p->n_merge;
         mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = b_o; mp.ws_ml = b_ml;

@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests: run the library through its C ABI, run the oracle, compare."""
+import ctypes as C
+import re
 from typing import Optional, Sequence, Tuple
 
 import numpy as np
@@ -58,6 +60,40 @@ def guarded_workspace(plan, device=None):
         lo, hi = buf[:GUARD_BYTES], buf[GUARD_BYTES + n:] if n > 0 else buf[GUARD_BYTES + 256:]
         assert bool((lo == 0xA5).all()) and bool((hi == 0xA5).all()), "a kernel wrote outside its workspace"
     return ws, check
+
+
+class _KernelNode(C.Structure):
+    _fields_ = [("func", C.c_void_p), ("dims", C.c_uint * 6), ("smem", C.c_uint), ("params", C.c_void_p), ("extra", C.c_void_p),
+                ("kern", C.c_void_p), ("ctx", C.c_void_p)]
+
+
+def kernels_in_order(launch):
+    """The kernels that a call launches, in stream order: the nodes of a graph captured from it, each behind the one before."""
+    cu = C.CDLL("libcuda.so.1")
+    launch()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        launch()
+    graph, n = C.c_void_p(g.raw_cuda_graph()), C.c_size_t()
+    assert cu.cuGraphGetNodes(graph, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    before = {}
+    for node in nodes:
+        k = C.c_size_t(4)
+        deps, data = (C.c_void_p * 4)(), (C.c_uint64 * 4)()
+        assert cu.cuGraphNodeGetDependencies_v2(C.c_void_p(node), deps, data, C.byref(k)) == 0 and k.value <= 1
+        before[deps[0] if k.value else None] = node
+    out, node = [], before.get(None)
+    while node is not None:
+        p, name = _KernelNode(), C.c_char_p()
+        assert cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(node), C.byref(p)) == 0
+        assert (cu.cuFuncGetName(C.byref(name), C.c_void_p(p.func)) if p.func else cu.cuKernelGetName(C.byref(name), C.c_void_p(p.kern))) == 0
+        out.append(re.search("ape_([a-z_]+)_kernel", name.value.decode()).group(1))
+        node = before.get(node)
+    assert len(out) == n.value
+    return out
 
 
 def oracle_attend(b: Batch, r: int, *, rows: Optional[Tuple[int, int]] = None, l_k: Optional[int] = None, q_override=None):

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2502_05431_b200 import libape, workloads as wl
-from tests.gpu_util import handle, gpu_attend, oracle_attend, compare
+from tests.gpu_util import handle, gpu_attend, kernels_in_order, oracle_attend, compare
 
 pytestmark = pytest.mark.gpu
 LLAMA = dict(H_q=32, H_kv=8, d=128)
@@ -79,3 +79,24 @@ def test_shared_decode_at_the_benchmark_size_sampled_requests():
             ref = oracle_attend(b, r, l_k=rq.query_kv[1] + t)
             compare(out[r:r + 1], ref.out.float(), f"shared 128K step {t} req {r}")
             assert (lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("H_q,H_kv,d,n_req,n_ctx,capacity,first", [
+    (32, 8, 128, 16, 2000, 64, "attn"), (32, 8, 128, 16, 2000, 65, "decode"),        # alternating halves: 1.73 and 2.6 tiles per SM
+    (16, 1, 128, 24, 6000, 320, "attn"), (16, 1, 128, 24, 6000, 321, "decode"),      # 384 rows: 0.97 and 1.14
+    (8, 2, 64, 32, 2048, 400, "attn"),                                               # heads of 64
+])
+def test_order_of_a_shared_step(H_q, H_kv, d, n_req, n_ctx, capacity, first):
+    """The per-request rest goes in front of the context pass where it is long enough to be worth it (148 SMs)."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the line is drawn in tiles per SM")
+    b = wl.share_contexts(wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=7, ctx_lens=[[n_ctx]] + [[]] * (n_req - 1), l_q=1, l_k=30, capacity=capacity, seed=34,
+                                        T=0.9, S=0.9, name="order"))
+    dev = b.to("cuda:0")
+    out = torch.zeros_like(dev.q)
+    plan = handle().attend_plan(H_q=H_q, H_kv=H_kv, d=d, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=out, requests=b.requests,
+                                mode=libape.APE_DECODE, shared=True)
+    ws = plan.alloc_workspace()
+    assert kernels_in_order(lambda: plan.attend(b.T, b.S, ws, kv_extra=3)) == [first, {"attn": "decode", "decode": "attn"}[first], "merge"]
+    for r in (0, n_req - 1):
+        compare(out[r:r + 1].cpu(), oracle_attend(b, r, l_k=33).out.float(), f"{first} first, req {r}")
