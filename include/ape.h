@@ -121,7 +121,8 @@ int ape_attend_plan(ape_handle_t handle, const ape_shape_t *shape, const ape_kv_
  * APE_PREFILL plans run in two passes (ape_attend then launches four kernels): per query row the log-sum-exp of every
  * context, then the same attention as ape_attend_plan with (S - 1) * LogSumExp_i added to the logits of context i, which
  * gives its tokens exactly the weights of Eq. 11-12; the plan's workspace also holds 16 bytes per (context, query row,
- * query head).  APE_DECODE plans keep one partial per context and cut their work items at every context boundary.
+ * query head).  APE_DECODE plans, and APE_PREFILL plans of so few contexts and rows that it is faster, keep one partial per context, cut
+ * their work items at every context boundary and merge the contexts by their log-sum-exps (one pass, two kernels).
  */
 int ape_attend_plan_per_context(ape_handle_t handle, const ape_shape_t *shape, const ape_kv_pool_t *pool,
                                 const ape_rows_t *q, const ape_rows_t *out, float *lse,
@@ -143,8 +144,8 @@ int ape_attend_plan_per_context(ape_handle_t handle, const ape_shape_t *shape, c
  * branch is this library's reading, made explicit by `scaled`.
  * Launch with ape_attend.  APE_PREFILL plans run in two passes like the per-context form (the bias of a node's tokens is
  * the sum of (S - 1) * A_a over the scaled nodes a on its path to the top, itself included; 16 bytes of workspace per
- * (node, query row, query head)); APE_DECODE plans cut their work items at node boundaries and merge the partials with a
- * stack of accumulators.  APE_ERR_INVALID_ARG for a malformed tree.
+ * (node, query row, query head)); APE_DECODE plans, and APE_PREFILL plans of few nodes and rows, cut their work items at node boundaries and
+ * merge the partials with a stack of accumulators.  APE_ERR_INVALID_ARG for a malformed tree.
  */
 int ape_attend_plan_tree(ape_handle_t handle, const ape_shape_t *shape, const ape_kv_pool_t *pool,
                          const ape_rows_t *q, const ape_rows_t *out, float *lse,
@@ -158,7 +159,9 @@ int ape_attend_plan_tree(ape_handle_t handle, const ape_shape_t *shape, const ap
  * and the context tokens of all requests are the same set (any split into contexts, any order); prefixes and query
  * segments are per request.  The context K/V is then read ONCE for the whole batch: the context pass runs on the tensor
  * cores with the batch's query rows as one block of rows, the rest (prefix + the request's own growing query segment)
- * runs per request, and one merge applies Eq. 5 per request.  Launch with ape_attend (T, S, kv_extra as for APE_DECODE).
+ * runs per request, and one merge applies Eq. 5 per request.  Where the contexts are so short, or the requests so few, that three kernels
+ * cost more than every request reading the contexts itself, the plan takes the ordinary decode step (the workspace asked for
+ * stays that of the shared form).  Launch with ape_attend (T, S, kv_extra as for APE_DECODE).
  * APE_ERR_INVALID_ARG if the requests do not share their contexts or their rows are not consecutive.
  */
 int ape_attend_plan_shared(ape_handle_t handle, const ape_shape_t *shape, const ape_kv_pool_t *pool,
@@ -335,12 +338,11 @@ int ape_rope_plan(ape_handle_t handle, int32_t head_dim, double theta, const ape
 int ape_rope_write(ape_plan_t plan, const ape_rows_t *src, const ape_rows_t *dst, int32_t n_heads, int32_t rotate,
                    void *stream);
 
-/* Steps of the last ape_attend / ape_encode_contexts call on this plan, as its form has them: its passes over the keys, the
- * walk between two passes, the merge (and the append of ape_decode_step_host).  Each is a kernel launch of its own, except
- * that a small plan takes several in one kernel (the merge inside the pass; per-context and tree prefills of few nodes: one
- * pass that needs no statistics and no biases); they are counted here all the same. */
+/* Kernels launched by the last ape_attend / ape_encode_contexts / ape_decode_step_host / ape_rope_write call on this plan.  Small plans
+ * take several steps of their form in one kernel (the merge inside the pass; contexts read by every request of a shared plan
+ * itself), so the number tells which form a plan has. */
 int ape_plan_last_launches(ape_plan_t plan, int32_t *n_launches);
-/* The kernels that the same call really launched. */
+/* The same number. */
 int ape_plan_last_kernels(ape_plan_t plan, int32_t *n_kernels);
 
 /*

@@ -66,12 +66,12 @@ struct ape_plan_s {
     bool budget = false;            // made under an SM budget: the SMs that it leaves stay free while its kernels run
     int cluster = 0;                // blocks per cluster when the kernel merges its partials itself (0: merge kernel)
     bool alt_halves = false;        // context pass of a shared plan with at most 128 rows: the halves take alternate tiles
-    int32_t last_launches = 0, last_fused = 0;   // steps of the last call; those of them that ran inside another step's kernel
+    int32_t last_launches = 0;
     int per_context = 0;             // merge form: 0 Eq. 5, 1 Eq. 11-12 (per context), 2 context trees
     DevNode* d_nodes = nullptr;      // tree plans; two-pass plans
     // Prefill plans of the per-context and tree forms run in two passes (statistics of every node's own tokens, then
     // the prefill with per-row, per-node biases): their per-node arrays live behind the partials in the workspace.
-    bool two_pass = false, one_pass = false;     // (one_pass: few nodes, a partial per node)
+    bool two_pass = false;
     int32_t* d_req_node0 = nullptr;  // [n_req + 1]
     DevBfsNode* d_bfs = nullptr;
     int32_t* d_levels = nullptr;
@@ -82,7 +82,6 @@ struct ape_plan_s {
     ape_plan_s* child_ctx = nullptr;
     ape_plan_s* child_oth = nullptr;
     bool plain = false;              // shared plan whose requests read the contexts themselves: child_oth is an ordinary decode plan
-    int plain_steps = 0;         // ... and the steps that its last_launches counts
     bool rest_first = false;         // shared plan: the per-request rest goes in front of the context pass
     // decode plans: what the host-buffer step needs (staging for the new token's Q is the plan's Q tensor itself)
     int n_req = 0;
@@ -697,7 +696,6 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                     const long long t = (reqs[r].ctx[i].len + kAttnTileN - 1) / kAttnTileN;
                     n += t > 0 ? 1 : 0; tiles += t; longest = std::max(longest, t);
                 }
-                if (n > 0) p->one_pass = true;
                 const long long mine = H_kv * (((reqs[r].q_len + TB - 1) / TB + p->n_sib - 1) / p->n_sib);
                 row_groups += mine; run_groups += (n + 1) * mine;
                 rows_all += reqs[r].q_len * shape->n_q_heads; most_nodes = std::max(most_nodes, n); most_tiles = std::max(most_tiles, tiles);
@@ -707,7 +705,6 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
                 const double waves = rows_all / (16.0 * h->n_sm_device), partials = static_cast<double>(std::min(most_tiles, std::max(most_nodes, n_groups / std::max(1ll, row_groups))));
                 one_pass = one_pass && (most_nodes * (0.65 + 0.75 * waves + std::max(waves - 2.0, 0.0)) + 0.05 * partials) * D / 128 <= 3.4 + longest;
             }
-            p->one_pass = p->one_pass && one_pass;
             int64_t row_base = 0;                          // query rows of the requests before this one
             bool any_node_tiles = false;
             for (int r = 0; r < n_req; ++r) {
@@ -974,7 +971,7 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
             rc = attend_plan_impl(h, shape, pool, q, out, lse, reqs, n_req, APE_DECODE, 0, nullptr, nullptr, &p->child_oth);
             // (the workspace that the shared form needs is still asked for: a call is refused for the same reasons in both)
             if (rc) { ape_plan_destroy(p); return rc; }
-            p->plain = true; p->plain_steps = t1 > t0 ? 3 : 2; p->ws_bytes = std::max(p->ws_bytes, p->child_oth->ws_bytes);
+            p->plain = true; p->ws_bytes = std::max(p->ws_bytes, p->child_oth->ws_bytes);
             p->n_req = n_req; p->q_rows = p->child_oth->q_rows; p->d_step = p->child_oth->d_step; p->child_oth->d_step = nullptr;
             *plan_out = p;
             return APE_OK;
@@ -1271,7 +1268,7 @@ int ape_plan_last_launches(ape_plan_t p, int32_t* n) {
 
 int ape_plan_last_kernels(ape_plan_t p, int32_t* n) {
     if (!p || !n) return APE_ERR_INVALID_ARG;
-    *n = p->last_launches - p->last_fused;
+    *n = p->last_launches;
     return APE_OK;
 }
 
@@ -1295,7 +1292,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
     rows_out.part_o_oth = part ? part->o_oth : nullptr; rows_out.part_lse_oth = part ? part->lse_oth : nullptr;
     if (p->kind == PLAN_SHARED && p->plain) {
         const int rc = attend_impl(p->child_oth, T, S, kv_extra, workspace, ws_bytes, stream_v, part);
-        p->last_launches = rc ? 0 : p->plain_steps; p->last_fused = rc ? 0 : p->last_launches - (p->child_oth->last_launches - p->child_oth->last_fused);
+        p->last_launches = rc ? 0 : p->child_oth->last_launches;
         return rc;
     }
     if (p->kind == PLAN_SHARED) {
@@ -1354,7 +1351,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
     const size_t rows = static_cast<size_t>(p->n_slots) * rows_per_slot;
     float* ws_o = static_cast<float*>(workspace);
     float* ws_ml = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + ((rows * D * 4 + 255) & ~size_t(255)));
-    p->last_launches = 0; p->last_fused = 0;
+    p->last_launches = 0;
 
     if (p->kind == PLAN_DECODE) {
         DecodeParams dp{};
@@ -1366,7 +1363,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         if (p->cluster > 0) {
             dp.cluster = p->cluster; dp.groups = p->d_merge; dp.fin = rows_out;
             if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
-            p->last_launches = 2; p->last_fused = 1;
+            p->last_launches = 1;
             return APE_OK;
         }
         if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
@@ -1396,7 +1393,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         }
         if (p->cluster > 0) { ap.mode = kAttnShort; ap.cluster = p->cluster; ap.groups = p->d_merge; ap.fin = rows_out; ap.n_sib = 1; }
         if (launch_attn(D, p->tm_q, p->tm_k, p->tm_v, p->tm_q, p->tm_split, ap, p->n_cta, p->smem_bytes, p->early, stream) != cudaSuccess) return APE_ERR_CUDA;
-        if (p->cluster > 0) { p->last_launches = 2; p->last_fused = 1; return APE_OK; }
+        if (p->cluster > 0) { p->last_launches = 1; return APE_OK; }
     }
     p->last_launches++;
 
@@ -1407,7 +1404,6 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
     static_cast<RowsOut&>(mp) = rows_out; mp.G = G; mp.D = D; mp.n_sm = p->h->n_sm_device;
     if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
     p->last_launches++;
-    if (p->one_pass) { p->last_launches += 2; p->last_fused = 2; }
     return APE_OK;
 }
 

@@ -403,7 +403,7 @@ class Plan:
         return int(n.value)
 
     def last_kernels(self) -> int:
-        """The kernels that the last call launched (last_launches counts its steps, of which a small plan runs two in one kernel)."""
+        """The same number as last_launches."""
         n = C.c_int32(0)
         _check(load().ape_plan_last_kernels(self._p, C.byref(n)), "ape_plan_last_kernels")
         return int(n.value)

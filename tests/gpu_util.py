@@ -1,4 +1,5 @@
 """Helpers shared by the GPU parity tests: run the library through its C ABI, run the oracle, compare."""
+import contextlib
 import ctypes as C
 import re
 from typing import Optional, Sequence, Tuple
@@ -23,9 +24,19 @@ def handle() -> libape.Handle:
     return _handle
 
 
+@contextlib.contextmanager
+def all_sms_but_one():
+    """Plans made inside are made for one SM less than the device has: nearly the same split, and no thread-block clusters."""
+    handle().set_sm_budget(torch.cuda.get_device_properties(0).multi_processor_count - 1)
+    try:
+        yield
+    finally:
+        handle().set_sm_budget(0)
+
+
 def gpu_attend(b: Batch, mode: int, *, kv_extra: int = 0, want_lse: bool = True, q_override=None, per_context: bool = False,
                shared: bool = False, tree=None):
-    """Copy the batch to cuda:0, plan, launch, return (out bf16 CPU, lse fp32 CPU, plan launches)."""
+    """Copy the batch to cuda:0, plan, launch, return (out bf16 CPU, lse fp32 CPU, kernels launched)."""
     dev = torch.device("cuda:0")
     q = (b.q if q_override is None else q_override).to(dev)
     k, v = b.k_pool.to(dev), b.v_pool.to(dev)

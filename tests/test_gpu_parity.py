@@ -7,7 +7,7 @@ import torch
 from oracle import ape_oracle as orc
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
-from tests.gpu_util import compare, gpu_attend, handle, oracle_attend
+from tests.gpu_util import all_sms_but_one, compare, gpu_attend, handle, oracle_attend
 
 pytestmark = pytest.mark.gpu
 LLAMA = dict(H_q=32, H_kv=8, d=128)
@@ -15,7 +15,15 @@ LLAMA = dict(H_q=32, H_kv=8, d=128)
 
 def _check_batch(b, mode, rows=None, lse_tol=2e-3, **kw):
     out, lse, n = gpu_attend(b, mode, **kw)
+    _check_result(b, out, lse, rows, lse_tol, **kw)
+    if n == 1:                                          # the blocks of a cluster merged; the same call with a merge kernel
+        with all_sms_but_one():
+            out, lse, n = gpu_attend(b, mode, **kw)
+        _check_result(b, out, lse, rows, lse_tol, **kw)
     assert n == 2
+
+
+def _check_result(b, out, lse, rows, lse_tol, **kw):
     for r, rq in enumerate(b.requests):
         ref = oracle_attend(b, r, rows=rows, l_k=(rq.query_kv[1] + kw.get("kv_extra", 0)) if kw.get("kv_extra") else None,
                             q_override=None if kw.get("q_override") is None else kw["q_override"][rq.q_start:rq.q_start + rq.q_len])

@@ -10,10 +10,10 @@ pytestmark = pytest.mark.gpu
 LLAMA = dict(H_q=32, H_kv=8, d=128)
 
 
-def _check(b, kv_extra=0, lse_tol=2e-3):
+def _check(b, once, kv_extra=0, lse_tol=2e-3):
+    """once: the contexts are read once for the batch (rest, context pass, merge); else every request reads them itself."""
     out, lse, n = gpu_attend(b, libape.APE_DECODE, shared=True, kv_extra=kv_extra)
-    has_ctx = any(l > 0 for _, l in b.requests[0].ctx)
-    assert n == (3 if has_ctx else 2)
+    assert n == 3 if once else n < 3
     for r, rq in enumerate(b.requests):
         ref = oracle_attend(b, r, l_k=(rq.query_kv[1] + kv_extra) if kv_extra else None)
         compare(out[rq.q_start:rq.q_start + 1], ref.out.float(), f"{b.name} req {r} O")
@@ -22,28 +22,36 @@ def _check(b, kv_extra=0, lse_tol=2e-3):
     return out
 
 
-@pytest.mark.parametrize("kw,n_req", [
-    (dict(**LLAMA, l_P=16, ctx_lens=[64, 200, 1, 130], l_k=5, T=0.9, S=0.9), 3),
-    (dict(**LLAMA, l_P=7, ctx_lens=[300], l_k=66, T=0.6, S=1.2, gap=2), 16),
-    (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[100, 100], l_k=9, T=0.9, S=0.5), 5),        # G = 1, d = 64
-    (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 3, l_k=65, T=1.1, S=0.9), 20),    # G = 16: two row blocks
-    (dict(**LLAMA, l_P=4, ctx_lens=[], l_k=3, T=0.9, S=0.9), 2),                            # no contexts at all
-    (dict(**LLAMA, l_P=0, ctx_lens=[129], l_k=1, T=0.8, S=0.7), 70),                        # 70 x 4 rows: two row blocks, ragged
-    (dict(**LLAMA, l_P=5, ctx_lens=[100], l_k=2, T=0.9, S=0.9), 32),                        # 128 rows exactly, one tile: one half idle
-    (dict(**LLAMA, l_P=5, ctx_lens=[100, 700], l_k=2, T=0.9, S=0.9), 33),                   # 132 rows: one 256-row block again
-    (dict(**LLAMA, l_P=9, ctx_lens=[128 * 5], l_k=2, T=0.7, S=0.8), 9),                     # an odd number of whole tiles
+@pytest.mark.parametrize("kw,n_req,once", [
+    (dict(**LLAMA, l_P=16, ctx_lens=[64, 200, 1, 130], l_k=5, T=0.9, S=0.9), 3, False),
+    (dict(**LLAMA, l_P=16, ctx_lens=[6000, 200, 1, 1300], l_k=5, T=0.9, S=0.9), 3, True),
+    (dict(**LLAMA, l_P=7, ctx_lens=[300], l_k=66, T=0.6, S=1.2, gap=2), 16, False),
+    (dict(**LLAMA, l_P=7, ctx_lens=[1300], l_k=66, T=0.6, S=1.2, gap=2), 16, True),
+    (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[100, 100], l_k=9, T=0.9, S=0.5), 5, False),        # G = 1, d = 64
+    (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[2000, 1700], l_k=9, T=0.9, S=0.5), 5, True),
+    (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 3, l_k=65, T=1.1, S=0.9), 20, False),    # G = 16: two row blocks
+    (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 24, l_k=65, T=1.1, S=0.9), 20, True),
+    (dict(**LLAMA, l_P=4, ctx_lens=[], l_k=3, T=0.9, S=0.9), 2, False),                            # no contexts at all
+    (dict(**LLAMA, l_P=900, ctx_lens=[], l_k=3, T=0.9, S=0.9), 16, False),                         # (the rest and the merge alone)
+    (dict(**LLAMA, l_P=0, ctx_lens=[129], l_k=1, T=0.8, S=0.7), 70, True),                         # 70 x 4 rows: two row blocks, ragged
+    (dict(**LLAMA, l_P=5, ctx_lens=[100], l_k=2, T=0.9, S=0.9), 32, False),
+    (dict(**LLAMA, l_P=300, ctx_lens=[100], l_k=2, T=0.9, S=0.9), 32, True),                       # 128 rows exactly, one tile: one half idle
+    (dict(**LLAMA, l_P=5, ctx_lens=[100, 700], l_k=2, T=0.9, S=0.9), 33, True),                    # 132 rows: one 256-row block again
+    (dict(**LLAMA, l_P=9, ctx_lens=[128 * 5], l_k=2, T=0.7, S=0.8), 9, False),
+    (dict(**LLAMA, l_P=9, ctx_lens=[128 * 21], l_k=2, T=0.7, S=0.8), 9, True),                     # an odd number of whole tiles
 ])
-def test_shared_context_decode(kw, n_req):
+def test_shared_context_decode(kw, n_req, once):
     lens = kw.pop("ctx_lens")
-    b = wl.share_contexts(wl.make_batch(ctx_lens=[lens] * n_req, l_q=1, seed=21, name="shared", **kw))
-    _check(b)
+    b = wl.share_contexts(wl.make_batch(ctx_lens=[lens] + [lens if not once else []] * (n_req - 1), l_q=1, seed=21, name="shared", **kw))
+    _check(b, once)
 
 
-def test_shared_plan_agrees_with_the_per_request_plan_and_grows():
-    b = wl.share_contexts(wl.make_batch(**LLAMA, l_P=32, ctx_lens=[[256] * 6] * 4, l_q=1, l_k=40, capacity=60, seed=22,
+@pytest.mark.parametrize("length,once", [(256, False), (2048, True)])
+def test_shared_plan_agrees_with_the_per_request_plan_and_grows(length, once):
+    b = wl.share_contexts(wl.make_batch(**LLAMA, l_P=32, ctx_lens=[[length] * 6] + [[]] * 3, l_q=1, l_k=40, capacity=60, seed=22,
                                         T=0.9, S=0.9, name="shared_grow"))
     for t in (0, 1, 20):
-        out = _check(b, kv_extra=t)
+        out = _check(b, once, kv_extra=t)
         ref, _, _ = gpu_attend(b, libape.APE_DECODE, kv_extra=t)                # ordinary decode plan on the same requests
         assert (out.float() - ref.float()).abs().max().item() <= 2e-2
 

@@ -12,9 +12,10 @@ pytestmark = pytest.mark.gpu
 LLAMA = dict(H_q=32, H_kv=8, d=128)
 
 
-def _check(b, mode, parents, scaled=None, kv_extra=0):
+def _check(b, mode, parents, scaled=None, kv_extra=0, one_pass=False):
     out, lse, n = gpu_attend(b, mode, tree=(parents, scaled), kv_extra=kv_extra)
-    assert n == (4 if mode == libape.APE_PREFILL else 2)      # prefill: statistics pass, biases, biased prefill, merge
+    # prefill: statistics pass, biases, biased prefill, merge; or, like decode, one pass and the merge that walks the nodes
+    assert n == (4 if mode == libape.APE_PREFILL and not one_pass else 2)
     for r, rq in enumerate(b.requests):
         q, p, c, k = b.views(r)
         if kv_extra:
@@ -29,6 +30,13 @@ def _check(b, mode, parents, scaled=None, kv_extra=0):
 
 TREES = [
     # node lengths per request, parents per request, scaled per request (None: roots)
+    ([[300, 0, 130, 64, 200, 1, 77, 90]], [[-1, 0, 1, 1, 0, -1, 5, 2]], None),           # seven nodes with tokens: two passes
+    ([[300, 0, 130, 64, 200, 1, 77, 90]], [[-1, 0, 1, 1, 0, -1, 5, 2]], [[0, 1, 0, 1, 1, 1, 0, 1]]),
+    ([[0, 256, 256, 256], [40, 5, 500, 1, 1, 1, 9]], [[-1, 0, 0, 0], [-1, 0, -1, 2, 3, 2, 0]], None),
+    ([[100, 90, 80, 70, 60, 50, 40]], [[-1, 0, 1, 2, 3, 4, 5]], [[1] * 7]),
+    ([[0, 0, 0, 129, 0, 65, 1, 2, 3, 4, 5]], [[-1, 0, 1, 2, 0, 4, 4, 4, 2, 0, -1]], [[1, 0, 1, 0, 0, 1, 1, 0, 1, 0, 1]]),
+]
+FEW = [                                                                                      # one pass in prefill, with 17 rows
     ([[300, 0, 130, 64, 200, 1, 77]], [[-1, 0, 1, 1, 0, -1, 5]], None),
     ([[300, 0, 130, 64, 200, 1, 77]], [[-1, 0, 1, 1, 0, -1, 5]], [[0, 1, 0, 1, 1, 1, 0]]),
     ([[0, 256, 256, 256], [40, 500]], [[-1, 0, 0, 0], [-1, 0]], None),
@@ -38,12 +46,12 @@ TREES = [
 
 
 @pytest.mark.parametrize("mode", [libape.APE_PREFILL, libape.APE_DECODE])
-@pytest.mark.parametrize("tree", range(len(TREES)))
+@pytest.mark.parametrize("tree", range(len(TREES + FEW)))
 def test_tree_form_matches_the_oracle(mode, tree):
-    lens, parents, scaled = TREES[tree]
-    l_q = 1 if mode == libape.APE_DECODE else 33
+    lens, parents, scaled = (TREES + FEW)[tree]
+    l_q = 1 if mode == libape.APE_DECODE else 33 if tree < len(TREES) else 17
     b = wl.make_batch(**LLAMA, l_P=20, ctx_lens=lens, l_q=l_q, l_k=40, capacity=44, gap=2, seed=60 + tree, T=0.8, S=0.7, name=f"tree{tree}")
-    _check(b, mode, parents, scaled, kv_extra=3 if mode == libape.APE_DECODE else 0)
+    _check(b, mode, parents, scaled, kv_extra=3 if mode == libape.APE_DECODE else 0, one_pass=tree >= len(TREES))
 
 
 def test_the_two_ends_of_the_family():
