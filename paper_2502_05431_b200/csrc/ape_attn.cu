@@ -808,7 +808,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             __syncwarp();
             named_bar_sync(2, kThreads);
             tc_fence_after();
-            ml[w * kHalfRows + r] = make_float2(m_end, l_end);
+            ml[w * kHalfRows + r] = (l_end > 0.f) ? make_float2(m_end, l_end) : make_float2(-INFINITY, 0.f);   // empty, as the merge kernel sees it (also: NaN)
             #pragma unroll 1
             for (int c = 0; c < kCols / 32; ++c) {
                 uint32_t o[32];

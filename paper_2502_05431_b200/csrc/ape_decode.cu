@@ -325,6 +325,10 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
                     L += fw * l[w];
                 }
                 if (CLUSTER) {
+                    // a sum that is no positive number: empty, as the merge kernel sees it
+                    const bool live = L > 0.f;
+                    M = live ? M : -INFINITY; L = live ? L : 0.f;
+                    acc.x = live ? acc.x : 0.f; acc.y = live ? acc.y : 0.f; acc.z = live ? acc.z : 0.f; acc.w = live ? acc.w : 0.f;
                     const int2 to = (idx < kConsumerWarps * 32) ? first_to : sent_to(row);
                     cluster_st4(cluster_map(smem_u32(recv + to.y * RS + e), to.x), acc);
                     if (e == 0) cluster_st2(cluster_map(smem_u32(&recv_ml[to.y]), to.x), M, L);

@@ -94,6 +94,25 @@ def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("mode,l_q", [(libape.APE_DECODE, 1), (libape.APE_PREFILL, 20)])
+def test_weights_that_are_no_numbers(mode, l_q, d):
+    """A partial whose sum of weights is no positive number counts as empty, with a merge kernel or without: a head with NaN in its query
+    gets zeros, and NaN in a key leaves no NaN behind."""
+    b = wl.make_batch(H_q=8, H_kv=2, d=d, l_P=40, ctx_lens=[[300, 64, 65]], l_q=l_q, l_k=l_q + 3, seed=48, T=0.8, S=0.7, name="nan")
+    assert _kernels(b, mode) == 1
+    clean = gpu_attend(b, mode)[0]
+    b.q[l_q - 1, 3] = float("nan")
+    (out, lse, _), (ref_o, ref_lse) = gpu_attend(b, mode), _ordinary(b, mode)
+    assert (out[l_q - 1, 3] == 0).all() and (ref_o[l_q - 1, 3] == 0).all()
+    assert lse[l_q - 1, 3] == ref_lse[l_q - 1, 3] == float("-inf")
+    out[l_q - 1, 3] = clean[l_q - 1, 3]
+    assert torch.equal(out, clean)
+    for s in (b.requests[0].ctx[1][0], b.requests[0].prefix[0]):
+        b.k_pool[s, 1] = float("nan")
+        assert torch.isfinite(gpu_attend(b, mode)[0].float()).all() and torch.isfinite(_ordinary(b, mode)[0].float()).all()
+
+
 @pytest.mark.parametrize("H_q,H_kv,d,n_ctx,length,l_q,kernels", [
     (32, 8, 128, 10, 256, 64, 1), (16, 1, 128, 1, 512, 8, 1), (16, 1, 128, 1, 513, 8, 2),      # one row block of 128 rows: six tiles, seven
     (16, 1, 128, 1, 1200, 1, 1), (16, 1, 128, 1, 1281, 1, 2), (4, 1, 64, 1, 3000, 40, 2),      # of 16 rows: 12 and 13 tiles
