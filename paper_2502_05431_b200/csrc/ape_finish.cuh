@@ -40,7 +40,7 @@ __device__ __forceinline__ void write_row(const RowsOut& p, int64_t out_row, int
     } else {
         *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(r[0], r[1]);
     }
-    if (p.lse_out != nullptr && lane == 0) p.lse_out[out_row * p.H_q + h] = (sum > 0.f) ? (top + fast_log2(sum)) * kLn2 : -INFINITY;
+    if (p.lse_out != nullptr && lane == 0) p.lse_out[out_row * p.H_q + h] = (top > -INFINITY) ? (top + fast_log2(sum)) * kLn2 : -INFINITY;
 }
 
 // Index 0: context, 1: non-context.

@@ -113,6 +113,14 @@ def test_weights_that_are_no_numbers(mode, l_q, d):
         assert torch.isfinite(gpu_attend(b, mode)[0].float()).all() and torch.isfinite(_ordinary(b, mode)[0].float()).all()
 
 
+@pytest.mark.parametrize("mode,l_q", [(libape.APE_DECODE, 1), (libape.APE_PREFILL, 20)])
+def test_scaling_beyond_the_range(mode, l_q):
+    """S so large that the context's log-sum-exp is infinite: row and log-sum-exp are both no number, not one of them."""
+    b = wl.make_batch(H_q=8, H_kv=2, d=64, l_P=40, ctx_lens=[[300]], l_q=l_q, seed=49, T=0.8, S=3e38, name="scale")
+    for out, lse in (gpu_attend(b, mode)[:2], _ordinary(b, mode)):
+        assert torch.isnan(out.float()).all() and torch.isnan(lse).all()
+
+
 @pytest.mark.parametrize("H_q,H_kv,d,n_ctx,length,l_q,kernels", [
     (32, 8, 128, 10, 256, 64, 1), (16, 1, 128, 1, 512, 8, 1), (16, 1, 128, 1, 513, 8, 2),      # one row block of 128 rows: six tiles, seven
     (16, 1, 128, 1, 1200, 1, 1), (16, 1, 128, 1, 1281, 1, 2), (4, 1, 64, 1, 3000, 40, 2),      # of 16 rows: 12 and 13 tiles
