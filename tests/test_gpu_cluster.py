@@ -14,9 +14,11 @@ pytestmark = pytest.mark.gpu
 def _ordinary(b, mode, **kw):
     handle().set_sm_budget(1)
     try:
-        return gpu_attend(b, mode, **kw)[:2]
+        out, lse, n = gpu_attend(b, mode, **kw)
     finally:
         handle().set_sm_budget(0)
+    assert n == 2
+    return out, lse
 
 
 def _kernels(b, mode, **how):
@@ -48,17 +50,19 @@ def test_decode(H_q, H_kv, d, n_req, ctx, l_P, l_k, gap):
             assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
-@pytest.mark.parametrize("n_req,lens,budget", [(1, [3000], 0), (3, [64, 200, 1, 130], 0), (3, [64, 200, 1, 130], 2), (9, [640], 0), (9, [640], 2),
-                                               (33, [100, 700], 2), (70, [129], 0), (70, [129], 3), (2, [], 0)])
-def test_shared_contexts_read_by_every_request_or_once(n_req, lens, budget):
-    """A shared batch whose requests read the (few) contexts themselves, and, under an SM budget, the same batch with one pass over them."""
+@pytest.mark.parametrize("n_req,lens,budget,kernels", [(1, [3000], 0, 1), (3, [64, 200, 1, 130], 0, 1), (3, [64, 200, 1, 130], 2, 3), (9, [640], 0, 1),
+                                                       (9, [640], 2, 3), (33, [100, 700], 2, 3), (70, [129], 0, 3), (70, [129], 3, 3), (2, [], 0, 1)])
+def test_shared_contexts_read_by_every_request_or_once(n_req, lens, budget, kernels):
+    """A shared batch whose requests read the (few) contexts themselves (a cluster each), and, under an SM budget, the same batch with one
+    pass over them."""
     b = wl.share_contexts(wl.make_batch(H_q=32, H_kv=8, d=128, l_P=7, ctx_lens=[lens] * n_req, l_q=1, l_k=3, capacity=90, gap=2, seed=43, T=0.8,
                                         S=0.7, name="shared"))
     handle().set_sm_budget(budget)
     try:
-        out, lse, _ = gpu_attend(b, libape.APE_DECODE, shared=True, kv_extra=70)
+        out, lse, n = gpu_attend(b, libape.APE_DECODE, shared=True, kv_extra=70)
     finally:
         handle().set_sm_budget(0)
+    assert n == kernels
     for r in (0, n_req // 2, n_req - 1):
         ref = oracle_attend(b, r, l_k=73)
         compare(out[r:r + 1], ref.out.float(), f"req {r}")
@@ -83,7 +87,8 @@ def test_shared_contexts_of_short_spans(n_req, n_ctx, length, gap, kernels):
                                                        (1, [900], 128, 33, 33, 0), (1, [129] * 3, 5, 129, 129, 1)])
 def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
     b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=l_P, ctx_lens=[ctx] * n_req, l_q=l_q, l_k=l_k, gap=gap, seed=44, T=0.8, S=0.7, name="short")
-    out, lse, _ = gpu_attend(b, libape.APE_PREFILL)
+    out, lse, n = gpu_attend(b, libape.APE_PREFILL)
+    assert n == 1 or (H_q, ctx) == (4, [900])                  # (33 rows of four heads over nine tiles: the ordinary form)
     ref_o, ref_lse = _ordinary(b, libape.APE_PREFILL)
     compare(out, ref_o.float(), "cluster against ordinary")
     assert (lse - ref_lse).abs().max() < 1e-3

@@ -22,12 +22,14 @@ def test_few_nodes(form, kw):
     b = wl.make_batch(seed=51, T=0.8, S=0.6, name=form, **kw)
     parents = [[-1 if i % 3 == 0 else i - i % 3 for i in range(len(rq.ctx))] for rq in b.requests]
     how = dict(per_context=True) if form == "per_context" else dict(tree=(parents, None))
-    out, lse, _ = gpu_attend(b, libape.APE_PREFILL, **how)
+    out, lse, n = gpu_attend(b, libape.APE_PREFILL, **how)
+    assert n == (4 if 5 in kw["ctx_lens"][0] else 2)           # (seven with tokens: two passes)
     handle().set_sm_budget(1)
     try:
-        two, two_lse, _ = gpu_attend(b, libape.APE_PREFILL, **how)
+        two, two_lse, n = gpu_attend(b, libape.APE_PREFILL, **how)
     finally:
         handle().set_sm_budget(0)
+    assert n == 4
     compare(out, two.float(), "one pass against two")
     assert (lse - two_lse).abs().max() < 1e-3
     for r, rq in enumerate(b.requests):

@@ -92,14 +92,18 @@ def _same_with_and_without_waits(launches, bufs):
     assert handle().get_status() == 0
 
 
-@pytest.mark.parametrize("mode,l_q,n_req,longest", [
-    (libape.APE_DECODE, 1, 4, 256), (libape.APE_PREFILL, 64, 1, 256), (libape.APE_PREFILL, 200, 1, 256),
-    (libape.APE_PREFILL, 200, 1, 18000),       # siblings and 30 tiles a group: the attention kernel is launched in order
+@pytest.mark.parametrize("mode,l_q,n_req,longest,l_P,kernels", [
+    (libape.APE_DECODE, 1, 4, 256, 30, (1, 1)),            # clusters
+    (libape.APE_DECODE, 1, 4, 6000, 30, (2, 3)),           # shared: context pass, rest, merge
+    (libape.APE_DECODE, 1, 24, 700, 30, (2, 3)),           # shared: rest, context pass beside it (alternating halves), merge
+    (libape.APE_DECODE, 1, 40, 300, 30, (2, 3)),           # the same with 160 rows
+    (libape.APE_PREFILL, 64, 1, 256, 30, (1,)), (libape.APE_PREFILL, 200, 1, 700, 900, (2,)),
+    (libape.APE_PREFILL, 200, 1, 18000, 30, (2,)),         # siblings and 30 tiles a group: the attention kernel is launched in order
 ])
-def test_calls_that_feed_each_other(mode, l_q, n_req, longest):
+def test_calls_that_feed_each_other(mode, l_q, n_req, longest, l_P, kernels):
     """The output of a call is the query of the next, all calls share one workspace, and no kernel of another library stands between
     them: what a kernel reads too early is an older query, partial or bias.  All plan kinds, each call over contexts of its own."""
-    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=30, ctx_lens=[[longest, 70, 130, 64] * 12] * n_req, l_q=l_q, l_k=l_q + 5, seed=62, T=0.7, S=0.8,
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=l_P, ctx_lens=[[longest, 70, 130, 64] * 12] * n_req, l_q=l_q, l_k=l_q + 5, seed=62, T=0.7, S=0.8,
                       name="chain", device="cuda:0")
     b.v_pool *= 8                              # (large outputs, a high logit scale: a call's query decides its result)
     bufs = [b.q, torch.zeros_like(b.q)]
@@ -116,6 +120,9 @@ def test_calls_that_feed_each_other(mode, l_q, n_req, longest):
                                           requests=reqs, mode=mode, softmax_scale=0.5, **form))
     ws = torch.empty(max(p.workspace_bytes for p in plans), dtype=torch.uint8, device="cuda:0")
     _same_with_and_without_waits([lambda p=p: p.attend(b.T, b.S, ws) for p in plans], bufs)
+    assert plans[0].last_launches() == kernels[0]          # Eq. 5
+    if mode == libape.APE_DECODE:
+        assert plans[3].last_launches() == kernels[1]      # shared contexts
 
 
 def test_encode_and_prefill_that_feed_each_other():
@@ -143,9 +150,9 @@ def test_budget_leaves_the_other_sms_free(op):
     n = 4000 if op == "encode" else 60000
     b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=64, ctx_lens=[[n], [64]], l_q=1, l_k=9, seed=64, T=0.8, S=0.9, with_encode_q=True,
                       name="budget", device="cuda:0")
-    reqs = b.requests[:1]
+    rq, rq1 = b.requests
+    reqs = [rq] if op != "shared" else [rq, wl.Request(rq1.q_start, 1, rq1.prefix, rq.ctx, rq1.query_kv, rq1.query_kv_capacity)]
     heads = dict(H_q=32, H_kv=8, d=128, k_pool=b.k_pool, v_pool=b.v_pool)
-    rq = reqs[0]
     form = dict(per_context=op == "per_context", shared=op == "shared")
     handle().set_sm_budget(1)
     try:
@@ -166,6 +173,7 @@ def test_budget_leaves_the_other_sms_free(op):
     s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
     run_long(), after.attend(0.8, 0.9, ws[1]), beside.attend(0.8, 0.9, ws[2])       # (first launches load code)
     torch.cuda.synchronize()
+    assert long.last_launches() == {"encode": 1, "shared": 3, "per_context": 4}.get(op, 2)
     with torch.cuda.stream(s1):
         run_long()
         after.attend(0.8, 0.9, ws[1])

@@ -87,16 +87,20 @@ def test_random_trees(seed):
     _check_all(b, out, lse, lambda r: orc.attend_tree(*b.views(r), b.T, b.S, parents[r], None if use_scaled is None else use_scaled[r]))
 
 
-@pytest.mark.parametrize("seed", range(28, 36))
-def test_random_shared_context_batches(seed):
+@pytest.mark.parametrize("seed,times", [(s, 1) for s in range(28, 36)] + [(s, 8) for s in (37, 43, 47, 48, 49, 52, 53, 54, 56, 57, 59)])
+def test_random_shared_context_batches(seed, times):
+    """Contexts of the drawn lengths, which every request reads itself, and of eight times as many tokens, which are read once."""
     rnd, kw = _draw(seed)
     n_req = rnd.choice([1, 2, 7, 16, 33])
-    lens = kw.pop("ctx_lens")[0]
+    lens = [n * times for n in kw.pop("ctx_lens")[0]]
     kw.pop("shuffle_ctx")
     l_k = rnd.choice([1, 9, 70])
-    b = wl.share_contexts(wl.make_batch(ctx_lens=[lens] * n_req, l_q=1, l_k=l_k, capacity=l_k + 4, **kw))
+    if times > 1:
+        n_req = max(n_req, 7)
+    b = wl.share_contexts(wl.make_batch(ctx_lens=[lens] + [[]] * (n_req - 1), l_q=1, l_k=l_k, capacity=l_k + 4, **kw))
     t = rnd.choice([0, 3])
-    out, lse, _ = gpu_attend(b, libape.APE_DECODE, shared=True, kv_extra=t)
+    out, lse, n = gpu_attend(b, libape.APE_DECODE, shared=True, kv_extra=t)
+    assert n == 3 if times > 1 else n < 3
     _check_all(b, out, lse, lambda r: oracle_attend(b, r, l_k=b.requests[r].query_kv[1] + t))
 
 
