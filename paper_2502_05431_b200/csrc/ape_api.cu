@@ -69,8 +69,8 @@ struct ape_plan_s {
     int32_t last_launches = 0;
     int per_context = 0;             // merge form: 0 Eq. 5, 1 Eq. 11-12 (per context), 2 context trees
     DevNode* d_nodes = nullptr;      // tree plans; two-pass plans
-    // Prefill plans of the per-context and tree forms run in two passes (statistics of every node's own tokens, then
-    // the prefill with per-row, per-node biases): their per-node arrays live behind the partials in the workspace.
+    // Prefill plans of the per-context and tree forms, but for those of few nodes, run in two passes (statistics of every node's own tokens,
+    // then the prefill with per-row, per-node biases): their per-node arrays live behind the partials in the workspace.
     bool two_pass = false;
     int32_t* d_req_node0 = nullptr;  // [n_req + 1]
     DevBfsNode* d_bfs = nullptr;
@@ -291,7 +291,7 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int 
     while (static_cast<int>(m.cta_begin.size()) < n_bins + 1) m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
 }
 
-// Tiles of the bin with the most, an item's end counted as item_tiles when the bin has several.
+// Tiles of the bin with the most (what its items' ends cost is not counted: the figures at pick_cluster were measured with this number).
 long long largest_bin(const HostMeta& m) {
     long long most = 0;
     for (size_t b = 0; b + 1 < m.cta_begin.size(); ++b) {
@@ -308,8 +308,7 @@ struct ClusterSplit { int size = 0; long long largest = 0; };
 long long cluster_largest(const std::vector<Run>& runs, int size) {        // tiles of the largest block, 0: more runs than blocks
     long long worst = 0;
     for (size_t i = 0, j; i < runs.size(); i = j) {
-        long long most = 0;
-        for (j = i; j < runs.size() && runs[j].merge0 == runs[i].merge0; ++j) most = std::max<long long>(most, runs[j].t1 - runs[j].t0);
+        for (j = i; j < runs.size() && runs[j].merge0 == runs[i].merge0;) ++j;
         if (static_cast<int>(j - i) > size) return 0;
         for (long long u = std::max(worst, 1ll);; ++u) {
             long long blocks = 0;

@@ -324,7 +324,8 @@ __global__ void __launch_bounds__(256, 4) ape_merge_kernel(const MergeParams p)
     finish_row<VEC>(p, rq.q_row0 + tok, g.kv_head * p.G + row % p.G, lane, M, L, acc);
 }
 
-// Decode plans of the per-context form and of context trees: one warp per output row walks the partials in order.
+// Plans of the per-context form and of context trees that keep a partial per node (decode; prefill of few nodes): one warp per output row
+// walks the partials in order.
 template <int VEC, bool TREE>
 __global__ void __launch_bounds__(256, 2) ape_merge_nodes_kernel(const MergeParams p)
 {
