@@ -31,7 +31,8 @@ __device__ __forceinline__ uint32_t pack_rn(float lo, float hi) {
 // under way before the first store (source and destination could be the same memory as far as the compiler knows, so that turn by turn
 // only two loads were).  The first chunk's table is computed in front of the dependency wait.
 // K, V and Q of 128K tokens (32 / 8 heads) back to back: 517 us with two loads under way and eight blocks per SM asked for, 500 with
-// four loads and four blocks (6.3 TB/s); eight loads and three blocks 517, two loads and six blocks 526.
+// four loads and four blocks (6.3 TB/s; with eight asked for, of which four are resident, 3% less again); eight loads and three blocks 517,
+// two loads and six blocks 526.
 template <int D>
 __global__ void __launch_bounds__(kRopeThreads, kRopeBlocksPerSm)
 ape_rope_kernel(const RopeParams p)

@@ -78,8 +78,9 @@ class _KernelNode(C.Structure):
                 ("kern", C.c_void_p), ("ctx", C.c_void_p)]
 
 
-def kernels_in_order(launch):
-    """The kernels that a call launches, in stream order: the nodes of a graph captured from it, each behind the one before."""
+def kernels_in_order(launch, grids=False):
+    """The kernels that a call launches (grids: and their numbers of blocks), in stream order: the nodes of a graph captured from it, each
+    behind the one before."""
     cu = C.CDLL("libcuda.so.1")
     launch()
     torch.cuda.synchronize()
@@ -101,7 +102,8 @@ def kernels_in_order(launch):
         p, name = _KernelNode(), C.c_char_p()
         assert cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(node), C.byref(p)) == 0
         assert (cu.cuFuncGetName(C.byref(name), C.c_void_p(p.func)) if p.func else cu.cuKernelGetName(C.byref(name), C.c_void_p(p.kern))) == 0
-        out.append(re.search("ape_([a-z_]+)_kernel", name.value.decode()).group(1))
+        kernel = re.search("ape_([a-z_]+)_kernel", name.value.decode()).group(1)
+        out.append((kernel, p.dims[0]) if grids else kernel)
         node = before.get(node)
     assert len(out) == n.value
     return out

@@ -5,7 +5,7 @@ import torch
 
 from oracle import ape_oracle, rope_oracle as ro
 from paper_2502_05431_b200 import libape, workloads as wl
-from tests.gpu_util import handle, compare
+from tests.gpu_util import compare, handle, kernels_in_order
 
 pytestmark = pytest.mark.gpu
 
@@ -163,3 +163,17 @@ def test_rope_chunk_sizes(H, d, n):
     plan.write(x.to("cuda:0"), dst, rotate=False)
     for s0, d0, ln, p0 in runs:
         assert torch.equal(dst[d0:d0 + ln].cpu(), x[s0:s0 + ln])
+
+
+@pytest.mark.parametrize("n_runs,length", [(158, 49), (150, 64), (1, 20000), (3, 70)])
+def test_rope_uses_the_whole_chip(n_runs, length):
+    """A block per chunk up to eight per SM, also where there are a few chunks more than blocks resident at once."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    runs = [(i * length, i * length, length, 7) for i in range(n_runs)]
+    x = torch.randn(n_runs * length, 4, 64).to(torch.bfloat16)
+    dst = torch.zeros_like(x, device="cuda:0")
+    plan, src = libape.RopePlan(handle(), 64, 500000.0, runs), x.to("cuda:0")
+    chunk = next((c for c in (16, 8, 4) if n_runs * length >= 2 * n_sm * c), 2)
+    assert kernels_in_order(lambda: plan.write(src, dst, True), grids=True) == [("rope", min(n_runs * -(-length // chunk), 8 * n_sm))]
+    for s0 in (0, (n_runs - 1) * length):
+        _check_rot(dst[s0:s0 + length].cpu(), ro.rope(x[s0:s0 + length], np.arange(7, 7 + length), 500000.0), float(x.abs().max()))
