@@ -361,7 +361,7 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
 // In us per call, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
 //   1 request   1 x 64 tokens 5.1 / 3.7 (2 / 1)   10 contexts 5.9 / 5.7 (3 / 5)   20: 7.5 / 7.5 (5 / 9: stays ordinary)   40: 9.3 / 11.3 (10 / 18)
 //   2 requests  4 contexts 6.3 / 5.1 (3 / 4)   10: 7.5 / 7.0 (5 / 8)   20: 9.6 / 10.4 (10 / 15)      4 requests  4 contexts 7.4 / 6.2
-constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 12, kFewBlocks = 6;
+constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 13, kPlainTiles64 = 17, kFewBlocks = 6;
 ClusterSplit pick_cluster(const ape_handle_s* h, const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], long long limit, int max_size = kCluster[0]) {
     ClusterSplit best;
     if (h->n_sm < h->n_sm_device) return best;
@@ -960,11 +960,14 @@ int ape_attend_plan_shared(ape_handle_t h, const ape_shape_t* shape, const ape_k
         // 9.5 / 5.1, over 3 x 2,046 tokens (17 tiles per SM against 3) 15.0 / 12.6; 8 requests over 16 x 23 tokens 10.4 / 6.1.
         // Tiles, not tokens: a short span that touches no other is a tile of its own for every request.  16 requests over 300 contexts of 8 tokens
         // with gaps (262 tiles per SM against 16) 38.2 / 136, 2 requests over 500 of 16 (55 against 27) 50.5 / 29.0.
+        // The line, 13 tiles per SM (17 for heads of 64, whose tiles are half as large) and 2.5 for every one of the context pass, is drawn from 220
+        // batches around it: three of those that it sends to the decode step were more than 3% slower there (at most 13%, eight heads of
+        // one query head), 15 of the others would have gained more than 5% (at most 18%).
         long long ctx_tiles64 = 0;
         for (const auto& sp : shared_ctx) ctx_tiles64 += (sp.len + kDecodeTile - 1) / kDecodeTile;
         long long decode_tiles = 0;
         for (const auto& r : runs_b) decode_tiles += r.t1 - r.t0 + ctx_tiles64;
-        if (n_req == 1 || decode_tiles <= static_cast<long long>(kPlainTiles) * h->n_sm + 2ll * (t1 - t0) * H_kv) {
+        if (n_req == 1 || 2 * decode_tiles <= 2ll * (D == 64 ? kPlainTiles64 : kPlainTiles) * h->n_sm + 5ll * (t1 - t0) * H_kv) {
             ape_plan_destroy(p->child_ctx); ape_plan_destroy(p->child_oth);
             p->child_ctx = p->child_oth = nullptr;
             rc = attend_plan_impl(h, shape, pool, q, out, lse, reqs, n_req, APE_DECODE, 0, nullptr, nullptr, &p->child_oth);

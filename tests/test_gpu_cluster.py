@@ -69,7 +69,7 @@ def test_shared_contexts_read_by_every_request_or_once(n_req, lens, budget, kern
         assert (lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
 
 
-@pytest.mark.parametrize("n_req,n_ctx,length,gap,kernels", [(8, 120, 8, 3, 3), (8, 120, 8, 0, 2), (2, 120, 8, 3, 2), (4, 60, 129, 1, 3), (4, 30, 128, 0, 2)])
+@pytest.mark.parametrize("n_req,n_ctx,length,gap,kernels", [(8, 120, 8, 3, 3), (8, 120, 8, 0, 2), (2, 120, 8, 3, 2), (4, 60, 129, 1, 3), (4, 30, 128, 0, 2), (3, 120, 16, 3, 2)])
 def test_shared_contexts_of_short_spans(n_req, n_ctx, length, gap, kernels):
     """Spans that touch are one span; with gaps between them each is a tile of its own, for every request that reads it itself."""
     b = wl.share_contexts(wl.make_batch(H_q=32, H_kv=8, d=128, l_P=7, ctx_lens=[[length] * n_ctx] * n_req, l_q=1, l_k=3, gap=gap, seed=46, T=0.8,

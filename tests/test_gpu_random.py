@@ -87,7 +87,7 @@ def test_random_trees(seed):
     _check_all(b, out, lse, lambda r: orc.attend_tree(*b.views(r), b.T, b.S, parents[r], None if use_scaled is None else use_scaled[r]))
 
 
-@pytest.mark.parametrize("seed,times", [(s, 1) for s in range(28, 36)] + [(s, 8) for s in (37, 43, 47, 48, 49, 52, 53, 54, 56, 57, 59)])
+@pytest.mark.parametrize("seed,times", [(s, 1) for s in range(28, 36)] + [(s, 8) for s in (43, 47, 49, 52, 53, 54, 56, 57)])
 def test_random_shared_context_batches(seed, times):
     """Contexts of the drawn lengths, which every request reads itself, and of eight times as many tokens, which are read once."""
     rnd, kw = _draw(seed)

@@ -24,13 +24,13 @@ def _check(b, once, kv_extra=0, lse_tol=2e-3):
 
 @pytest.mark.parametrize("kw,n_req,once", [
     (dict(**LLAMA, l_P=16, ctx_lens=[64, 200, 1, 130], l_k=5, T=0.9, S=0.9), 3, False),
-    (dict(**LLAMA, l_P=16, ctx_lens=[6000, 200, 1, 1300], l_k=5, T=0.9, S=0.9), 3, True),
+    (dict(**LLAMA, l_P=16, ctx_lens=[9600, 200, 1, 1300], l_k=5, T=0.9, S=0.9), 3, True),
     (dict(**LLAMA, l_P=7, ctx_lens=[300], l_k=66, T=0.6, S=1.2, gap=2), 16, False),
     (dict(**LLAMA, l_P=7, ctx_lens=[1300], l_k=66, T=0.6, S=1.2, gap=2), 16, True),
     (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[100, 100], l_k=9, T=0.9, S=0.5), 5, False),        # G = 1, d = 64
-    (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[2000, 1700], l_k=9, T=0.9, S=0.5), 5, True),
+    (dict(H_q=8, H_kv=8, d=64, l_P=3, ctx_lens=[3300, 2900], l_k=9, T=0.9, S=0.5), 5, True),
     (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 3, l_k=65, T=1.1, S=0.9), 20, False),    # G = 16: two row blocks
-    (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 24, l_k=65, T=1.1, S=0.9), 20, True),
+    (dict(H_q=16, H_kv=1, d=128, l_P=64, ctx_lens=[256] * 28, l_k=65, T=1.1, S=0.9), 20, True),
     (dict(**LLAMA, l_P=4, ctx_lens=[], l_k=3, T=0.9, S=0.9), 2, False),                            # no contexts at all
     (dict(**LLAMA, l_P=900, ctx_lens=[], l_k=3, T=0.9, S=0.9), 16, False),                         # (the rest and the merge alone)
     (dict(**LLAMA, l_P=0, ctx_lens=[129], l_k=1, T=0.8, S=0.7), 70, True),                         # 70 x 4 rows: two row blocks, ragged
@@ -92,7 +92,7 @@ def test_shared_decode_at_the_benchmark_size_sampled_requests():
 @pytest.mark.parametrize("H_q,H_kv,d,n_req,n_ctx,capacity,first", [
     (32, 8, 128, 16, 2000, 64, "attn"), (32, 8, 128, 16, 2000, 65, "decode"),        # alternating halves: 1.73 and 2.6 tiles per SM
     (16, 1, 128, 24, 6000, 320, "attn"), (16, 1, 128, 24, 6000, 321, "decode"),      # 384 rows: 0.97 and 1.14
-    (8, 2, 64, 32, 2048, 400, "attn"),                                               # heads of 64
+    (8, 2, 64, 32, 4096, 400, "attn"),                                               # heads of 64
 ])
 def test_order_of_a_shared_step(H_q, H_kv, d, n_req, n_ctx, capacity, first):
     """The per-request rest goes in front of the context pass where it is long enough to be worth it (148 SMs)."""
