@@ -50,6 +50,20 @@ def test_decode(H_q, H_kv, d, n_req, ctx, l_P, l_k, gap):
             assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("n_req,n_ctx,kernels", [(1, 10, 1), (1, 20, 2), (2, 10, 1), (2, 20, 2)])
+def test_decode_on_both_sides_of_the_line(n_req, n_ctx, kernels):
+    """The largest block of a cluster may have three tiles more than the ordinary form's: 5 against 3 and 9 against 5 tiles for one request (148 SMs)."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the split is that of 148 SMs")
+    b = wl.make_batch(H_q=32, H_kv=8, d=128, l_P=32, ctx_lens=[[256] * n_ctx] * n_req, l_q=1, l_k=65, seed=42, T=0.8, S=0.7, name="line")
+    out, lse, n = gpu_attend(b, libape.APE_DECODE)
+    assert n == kernels
+    for r in range(n_req):
+        ref = oracle_attend(b, r)
+        compare(out[r:r + 1], ref.out.float(), f"req {r}")
+        assert (lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
+
+
 @pytest.mark.parametrize("n_req,lens,budget,kernels", [(1, [3000], 0, 1), (3, [64, 200, 1, 130], 0, 1), (3, [64, 200, 1, 130], 2, 3), (9, [640], 0, 1),
                                                        (9, [640], 2, 3), (33, [100, 700], 2, 3), (70, [129], 0, 3), (70, [129], 3, 3), (2, [], 0, 1)])
 def test_shared_contexts_read_by_every_request_or_once(n_req, lens, budget, kernels):
