@@ -37,6 +37,9 @@ constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kBarBytes = 512;                // barriers, behind the tiles
 constexpr int kStageBytes = 8 * 4096;         // transposition buffers of the softmax warps, behind the barriers
+// Clusters, behind the barriers: a share is 1 / size of at most 128 rows, rounded up; (m, l) of a share from every block and its rows from
+// all but one (sizes 2 ... 10 and 16: at most 135 and 120; a block without a partial of its own has one more sender, but then one is idle)
+constexpr int kRecvMl = 136, kRecvRows = 120;
 constexpr int kSlabBytes = 128 * 128;         // 128 rows x 64 bf16
 constexpr float kRescaleThreshold = 8.0f;     // base-2 units: O is rescaled only when the row maximum grew by more
 
@@ -146,7 +149,9 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint8_t* v_smem = k_smem + kNK * kTileBytes;               // kNV stages
     uint64_t* bars = reinterpret_cast<uint64_t*>(v_smem + kNV * kTileBytes);
     uint8_t* stage_smem = v_smem + kNV * kTileBytes + kBarBytes;   // STAGED: 4 KB per softmax warp
-    float2* recv_ml = reinterpret_cast<float2*>(stage_smem);       // SHORT: (m, l) of the rows this block merges, from every block
+    // SHORT: what the other blocks send of the rows that this block merges: (m, l) from every block, the rows
+    float2* recv_ml = reinterpret_cast<float2*>(stage_smem);
+    uint8_t* recv_rows = stage_smem + kRecvMl * sizeof(float2);
     // barrier map
     const uint32_t bar0 = smem_u32(bars);
     const uint32_t bar_q_full = bar0, bar_q_empty = bar0 + 16;             // [QBUF] each
@@ -158,11 +163,11 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const uint32_t bar_done = bar_o_full + 16;
     const uint32_t bar_tok = bar_done + 8;                     // [2]: turn-taking of the two halves' exponential phases
     const uint32_t bar_o_staged = bar_tok + 16;                // [QBUF][2]: a half's O tile sits in its Q buffer, ready for its bulk store
+    const uint32_t bar_recv = bar_o_staged + 32;               // SHORT: bytes that have arrived in recv_ml and recv_rows
     __shared__ uint32_t tmem_base_smem;
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (SHORT) cluster_arrive();                               // this block's shared memory may be written by the others (they wait below)
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -177,6 +182,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         mbar_init(bar_done, 2);
         mbar_init(bar_tok, 4); mbar_init(bar_tok + 8, 4);          // one arrival per softmax warp of the other half
         for (int b = 0; b < 2 * QBUF; ++b) mbar_init(bar_o_staged + 8 * b, 4);       // one arrival per softmax warp of the half
+        if (SHORT) mbar_init(bar_recv, 1);
         mbar_fence_init();
     }
     if (warp == kMmaWarp) {
@@ -185,6 +191,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     tc_fence_before();
     __syncthreads();
+    if (SHORT) cluster_arrive();                               // this block's shared memory may be written by the others (they wait below)
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_smem;
 
@@ -236,8 +243,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if constexpr (SHORT) {
             __syncwarp();
             named_bar_sync(2, kThreads);
-            cluster_wait(); cluster_arrive();
-            cluster_wait(); cluster_arrive();
+            cluster_wait(); cluster_arrive_relaxed();
             cluster_wait();
         }
     };
@@ -793,21 +799,31 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
         if constexpr (SHORT) {
             // ---- the block's two partials become one, the cluster's blocks merge theirs ------------------------------------------------
-            // Rows are fp32, 16-byte chunk j of row r at j ^ (r mod 8).  K and V stages are free: every product and every copy is done.
+            // Block k merges the k-th share of the row block's rows.  Every block sends the shares of its partial to the blocks that merge
+            // them, a bulk copy each, counted in bytes on a barrier there: a block waits for its own rows only and merges them from its own
+            // shared memory.  Bound by latency and by what the SMs exchange (56 KB in and out per block of a cluster of six, about 2,000
+            // cycles).  Reading the others' rows behind a barrier of the cluster, three blocks at a time, and a second barrier before a block
+            // may leave took 7,600 of the 28,000 cycles of 64 rows over 10 x 256 tokens: 14.4 us, now 13.7; 4 x 64 tokens 6.9, now 6.5.
+            // Rows are fp32, 16-byte chunk j of row r at j ^ (r mod 8).  Q, K and V are free: every product and every copy is done.
             constexpr int kCols = D / 2;                            // columns that a half's threads combine
             constexpr int VEC = D / 8;                              // eight lanes merge a row
             uint8_t* cross = k_smem;                                // [2][128][kCols]: what each half has in the other one's columns
             uint8_t* rows = v_smem;                                 // [128][D]: the block's partial
-            float2* ml = recv_ml + kHalfRows + kMaxCluster;         // [2][128]
+            float2* ml = reinterpret_cast<float2*>(q_smem);         // [2][128]
             const int C = p.cluster, rank = static_cast<int>(cluster_ctarank()), r = r_local;
             const DevMerge merge = p.groups[blockIdx.x / static_cast<unsigned>(C)];
             const DevReq rq = p.reqs[merge.req];
             const int n_rows = min(kHalfRows, (rq.q_len - merge.row_block * TB) * G);       // live rows of the row block
-            const int turn0 = r / C, owner = r - turn0 * C;         // the block that merges row r has its (m, l) at turn0 * C + sender
+            const int n = merge.ctx_n + merge.oth_n;                // blocks 0 .. n - 1 have a partial
+            const int share = (n_rows + C - 1) / C, first = rank * share, mine = min(max(n_rows - first, 0), share);
+            const int owner = r / share;                            // of row r
+            // where block `from` puts its rows for block `to`: a block that has a partial keeps its own rows where they are
+            auto slot = [&](int from, int to) { return from - (to < n && from > to ? 1 : 0); };
             tc_fence_before();
             __syncwarp();
             named_bar_sync(2, kThreads);
             tc_fence_after();
+            if (threadIdx.x == 0) mbar_expect_tx(bar_recv, static_cast<uint32_t>((rank < n ? n - 1 : n) * mine * (D * 4 + 8)));
             ml[w * kHalfRows + r] = (l_end > 0.f) ? make_float2(m_end, l_end) : make_float2(-INFINITY, 0.f);   // empty, as the merge kernel sees it (also: NaN)
             #pragma unroll 1
             for (int c = 0; c < kCols / 32; ++c) {
@@ -824,7 +840,11 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const float M = fmaxf(a.x, b.x);
             const float fa = (a.y > 0.f) ? fast_exp2(a.x - M) : 0.f, fb = (b.y > 0.f) ? fast_exp2(b.x - M) : 0.f;
             cluster_wait();                                         // (of the arrival at the start)
-            if (w == 0) cluster_st2(cluster_map(smem_u32(&recv_ml[turn0 * C + rank]), owner), M, a.y * fa + b.y * fb);
+            if (w == 0 && rank < n && r < n_rows) {
+                float2* at = &recv_ml[rank * share + r - owner * share];
+                if (owner == rank) *at = make_float2(M, a.y * fa + b.y * fb);
+                else cluster_send2(cluster_map(smem_u32(at), owner), M, a.y * fa + b.y * fb, cluster_map(bar_recv, owner));
+            }
             #pragma unroll 1
             for (int c = 0; c < kCols / 32; ++c) {
                 uint32_t o[32];
@@ -841,19 +861,36 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     *reinterpret_cast<float4*>(rows + r * (D * 4) + (((w * (kCols / 4) + c * 8 + j) ^ (r & 7)) << 4)) = y;
                 }
             }
+            fence_proxy_async_smem();
+            named_bar_sync(1, 256);
+            if (warp == 0 && lane < C && lane != rank && rank < n) {
+                const int count = min(n_rows - lane * share, share);
+                if (count > 0)
+                    cluster_copy(cluster_map(smem_u32(recv_rows + slot(rank, lane) * share * (D * 4)), lane), smem_u32(rows + lane * share * (D * 4)),
+                                 static_cast<uint32_t>(count * (D * 4)), cluster_map(bar_recv, lane));
+            }
             __syncwarp();
-            cluster_arrive();
-            cluster_wait();
+            // (all lanes wait: each reads what has arrived)
+            const bool here = __all_sync(0xffffffffu, mbar_wait(bar_recv, 0, &abort_flag, p.status)) != 0;
+            cluster_arrive_relaxed();                               // no block leaves while a copy of its rows is under way
             // eight lanes to a row, so that a block's rows (cluster of 6: 22) are merged side by side
-            for (int turn = warp * 4 + (lane >> 3); rank + C * (turn & ~3) < n_rows; turn += 32) {
-                const int rr = rank + C * turn;
-                if (rr >= n_rows) continue;
+            for (int i = warp * 4 + (lane >> 3); here && (i & ~3) < mine; i += 32) {
+                if (i >= mine) continue;
+                const int rr = first + i;
+                const uint8_t* own = rows + rr * (D * 4);
+                const uint8_t* got = recv_rows + i * (D * 4);
                 float Ms[2], Ls[2], acc[2][VEC];
-                merge_remote<VEC>(&recv_ml[turn * C], smem_u32(rows + rr * (D * 4)), rr & 7, lane & 7, merge.ctx_n, merge.oth_n, Ms, Ls, acc);
+                merge_cluster<VEC>(&recv_ml[i], share, merge.ctx_n, merge.oth_n, [&](int j, float (&x)[VEC]) {
+                    const uint8_t* o = (j == rank ? own : got + slot(j, rank) * share * (D * 4)) + (((lane & 7) ^ (rr & 7)) << 4);
+                    #pragma unroll
+                    for (int v = 0; v < VEC; v += 4) {
+                        const float4 t = *reinterpret_cast<const float4*>(o + v * 32);
+                        x[v] = t.x; x[v + 1] = t.y; x[v + 2] = t.z; x[v + 3] = t.w;
+                    }
+                }, Ms, Ls, acc);
                 finish_row<VEC, 8>(p.fin, rq.q_row0 + merge.row_block * TB + rr / G, merge.kv_head * G + rr % G, lane & 7, Ms, Ls, acc);
             }
             __syncwarp();
-            cluster_arrive();                                       // no block leaves while another one reads its rows
             cluster_wait();
         }
     }
@@ -974,7 +1011,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 size_t attn_smem_bytes(int D, int mode) {
     const size_t tile = static_cast<size_t>(D / 64) * kSlabBytes;
     // Q halves + K stages + V stages
-    if (mode == kAttnShort) return 1024 + (1 + 2 + 2) * tile + kBarBytes + (3 * kHalfRows + kMaxCluster) * sizeof(float2);
+    if (mode == kAttnShort) return 1024 + (1 + 2 + 2) * tile + kBarBytes + kRecvMl * sizeof(float2) + static_cast<size_t>(kRecvRows) * D * 4;
     const int tiles = (mode == kAttnAlt) ? (1 + 3 + 3) : (mode == kAttnEncode) ? (4 + 2 + 1) : (2 + 2 + 2);
     return 1024 + tiles * tile + kBarBytes + (tiles == 6 ? kStageBytes : 0);
 }

@@ -81,15 +81,22 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
+// An arrival that orders no memory: for blocks that only tell each other that they may leave.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_st2(uint32_t addr, float a, float b) {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
 __device__ __forceinline__ void cluster_st4(uint32_t addr, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-
-__device__ __forceinline__ void cluster_ld4(uint32_t addr, float& a, float& b, float& c, float& d) {
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a), "=f"(b), "=f"(c), "=f"(d) : "r"(addr) : "memory");
+// Stores and copies to another block's shared memory, counted in bytes on a barrier there: who waits on it sees them, no barrier of the
+// whole cluster is needed.  addr / dst and bar: addresses of the same block (cluster_map).
+__device__ __forceinline__ void cluster_send2(uint32_t addr, float a, float b, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_copy(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {       // 16-byte pieces
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
 constexpr int kMaxCluster = 16;
@@ -126,52 +133,49 @@ __device__ __forceinline__ void merge_received(const float2* ml, const float* o,
     }
 }
 
-// The same for rows that stay where they were made, with eight lanes to a row of 8 VEC elements: lane l takes the 16-byte chunks l, l + 8,
-// ...; chunk j of a row lies at j ^ swz.  o: the row's address in this block; the other blocks have theirs at the same place.
-template <int VEC>
-__device__ __forceinline__ void merge_remote(const float2* ml, uint32_t o, int swz, int l, int n_ctx, int n_oth, float (&M)[2], float (&L)[2],
-                                             float (&acc)[2][VEC])
+// Merges one row of a cluster whose blocks have each at most one partial of it: those of blocks [0, n_ctx) belong to the context, those
+// of the n_oth behind them do not.  ml[j * ml_stride]: (m, l) of block j's partial; load(j, x): this lane's VEC elements of it.
+// Short loops: the code runs once per launch, and instructions that the SM does not hold yet cost more than the loops' latencies (behind
+// the rows' arrival, 64 rows over 10 x 256 tokens: 3,700 cycles with all sixteen blocks unrolled, 2,700 this way).
+// (An empty partial has m = -inf, l = 0 and a row of zeros.)
+template <int VEC, typename Load>
+__device__ __forceinline__ void merge_cluster(const float2* ml, int ml_stride, int n_ctx, int n_oth, Load load, float (&M)[2], float (&L)[2], float (&acc)[2][VEC])
 {
-    constexpr int kBatch = 3;                              // blocks whose reads are under way at a time
     const int n = n_ctx + n_oth;
-    const uint32_t at = o + static_cast<uint32_t>((l ^ swz) << 4);
-    float x[kBatch][VEC];
-    auto load = [&](int j0) {
-        #pragma unroll
-        for (int u = 0; u < kBatch; ++u)
-            if (j0 + u < n) {
-                const uint32_t a = cluster_map(at, j0 + u);
-                #pragma unroll
-                for (int v = 0; v < VEC; v += 4) cluster_ld4(a + v * 32, x[u][v], x[u][v + 1], x[u][v + 2], x[u][v + 3]);
-            }
-    };
-    load(0);
-    #pragma unroll
-    for (int seg = 0; seg < 2; ++seg) {
-        float top = -INFINITY, sum = 0.f;
-        const int j0 = seg ? n_ctx : 0, j1 = seg ? n : n_ctx;
-        #pragma unroll 4
-        for (int j = j0; j < j1; ++j) top = fmaxf(top, ml[j].x);
-        const float base = (top == -INFINITY) ? 0.f : top;
-        #pragma unroll 4
-        for (int j = j0; j < j1; ++j) sum += ml[j].y * fast_exp2(ml[j].x - base);
-        M[seg] = top; L[seg] = sum;
-        #pragma unroll
-        for (int v = 0; v < VEC; ++v) acc[seg][v] = 0.f;
+    float mc = -INFINITY, mo = -INFINITY;
+    #pragma unroll 2
+    for (int j = 0; j < n; ++j) {
+        const float m = ml[j * ml_stride].x;
+        if (j < n_ctx) mc = fmaxf(mc, m); else mo = fmaxf(mo, m);
     }
-    const float base_c = (M[0] == -INFINITY) ? 0.f : M[0], base_o = (M[1] == -INFINITY) ? 0.f : M[1];
+    M[0] = mc; M[1] = mo; L[0] = L[1] = 0.f;
+    #pragma unroll
+    for (int v = 0; v < VEC; ++v) acc[0][v] = acc[1][v] = 0.f;
     #pragma unroll 1
-    for (int j0 = 0; j0 < n; j0 += kBatch) {
-        if (j0 > 0) load(j0);
+    for (int seg = 0; seg < 2; ++seg) {
+        const int j1 = seg ? n : n_ctx;
+        const float top = seg ? mo : mc, base = (top == -INFINITY) ? 0.f : top;
+        float sum = 0.f, x[VEC], y[VEC];
         #pragma unroll
-        for (int u = 0; u < kBatch; ++u)
-            if (j0 + u < n) {
-                const bool ctx = j0 + u < n_ctx;
-                const float f = fast_exp2(ml[j0 + u].x - (ctx ? base_c : base_o));
-                const float fc = ctx ? f : 0.f, fo = ctx ? 0.f : f;
-                #pragma unroll
-                for (int v = 0; v < VEC; ++v) { acc[0][v] += fc * x[u][v]; acc[1][v] += fo * x[u][v]; }
-            }
+        for (int v = 0; v < VEC; ++v) y[v] = 0.f;
+        #pragma unroll 2
+        for (int j = seg ? n_ctx : 0; j < j1; ++j) {
+            const float2 w = ml[j * ml_stride];
+            load(j, x);
+            const float f = fast_exp2(w.x - base);
+            sum += w.y * f;
+            #pragma unroll
+            for (int v = 0; v < VEC; ++v) y[v] += f * x[v];
+        }
+        if (seg) {
+            L[1] = sum;
+            #pragma unroll
+            for (int v = 0; v < VEC; ++v) acc[1][v] = y[v];
+        } else {
+            L[0] = sum;
+            #pragma unroll
+            for (int v = 0; v < VEC; ++v) acc[0][v] = y[v];
+        }
     }
 }
 

@@ -113,6 +113,23 @@ def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("H_q,H_kv,d", [(4, 1, 128), (16, 2, 64), (8, 8, 128)])
+@pytest.mark.parametrize("n_ctx", [0, 1, 2, 3, 5, 9, 12])
+@pytest.mark.parametrize("l_q", [1, 3, 13, 32])
+def test_prefill_shares_of_rows(H_q, H_kv, d, n_ctx, l_q):
+    """Every block of a cluster merges a share of the rows: rows that do not divide by the blocks, fewer rows than blocks, blocks without a
+    partial, clusters of different sizes.  Against the ordinary form (the same products and sums in another order, rounded to bf16, 2^-9 of
+    the value, on both sides) where the plan takes clusters."""
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=20, ctx_lens=[[130] * n_ctx], l_q=l_q, gap=1, seed=47, T=0.8, S=0.7, name="shares")
+    out, lse, n = gpu_attend(b, libape.APE_PREFILL)
+    ref_o, ref_lse = _ordinary(b, libape.APE_PREFILL)
+    assert (out.float() - ref_o.float()).abs().max() <= 2 ** -7 * max(1.0, ref_o.float().abs().max().item())
+    assert (lse - ref_lse).abs().max() < 1e-4
+    ref = oracle_attend(b, 0)
+    compare(out, ref.out.float(), "shares")
+    assert (lse.double() - ref.lse).abs().max().item() < 2e-3
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("mode,l_q", [(libape.APE_DECODE, 1), (libape.APE_PREFILL, 20)])
 def test_weights_that_are_no_numbers(mode, l_q, d):
