@@ -195,9 +195,11 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_smem;
 
-    const int n_sib = p.n_sib;
+    // (SHORT: block b works on item b.  A range read in front of it is 700 cycles more between two calls, where the second one's clusters
+    // cannot be placed before the first one has left its SMs: 64 rows over 10 x 256 tokens 13.7 us, now 12.95)
+    const int n_sib = SHORT ? 1 : p.n_sib;
     const int group = blockIdx.x / n_sib, sib = blockIdx.x - group * n_sib;
-    const int item_begin = p.cta_item_begin[group], item_end = p.cta_item_begin[group + 1];
+    const int item_begin = SHORT ? group : p.cta_item_begin[group], item_end = SHORT ? group + 1 : p.cta_item_begin[group + 1];
     const int G = p.G;
     constexpr bool alt = ALT;                // both halves read the same 128 rows and take alternate tiles
     const int TB = (alt ? kHalfRows : kAttnRows) / G;            // query tokens per row block
@@ -533,10 +535,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const uint32_t tO = tmem_base + lane_base + (w ? kColO1 : kColO0);
         const uint32_t my_s_full = bar_s_full + 8 * w, my_p_full = bar_p_full + 32 * w, my_o_full = bar_o_full + 8 * w;
         if (item_begin < item_end) prefetch_l1(&p.items[item_begin]);
-        if (SHORT) {                                                // the records of the merge at the end
-            const DevMerge* merge = &p.groups[blockIdx.x / static_cast<unsigned>(p.cluster)];
-            prefetch_l1(&p.reqs[merge->req]);
-        }
+        if (SHORT) prefetch_l1(&p.groups[blockIdx.x / static_cast<unsigned>(p.cluster)]);      // the record of the merge at the end
         wait_for_kernel_before();                                   // in front of the first bias read and the first store
         float m_end = -INFINITY, l_end = 0.f;                       // SHORT: this thread's row at the end of the block's item
         uint32_t scnt = 0, ocnt = 0, q_loads = 0, tcnt = 0;         // tcnt: visible tiles of the CTA so far (either half's)
@@ -812,8 +811,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             float2* ml = reinterpret_cast<float2*>(q_smem);         // [2][128]
             const int C = p.cluster, rank = static_cast<int>(cluster_ctarank()), r = r_local;
             const DevMerge merge = p.groups[blockIdx.x / static_cast<unsigned>(C)];
-            const DevReq rq = p.reqs[merge.req];
-            const int n_rows = min(kHalfRows, (rq.q_len - merge.row_block * TB) * G);       // live rows of the row block
+            const int n_rows = min(kHalfRows, (p.items[item_begin].q_len - merge.row_block * TB) * G);      // live rows of the row block
             const int n = merge.ctx_n + merge.oth_n;                // blocks 0 .. n - 1 have a partial
             const int share = (n_rows + C - 1) / C, first = rank * share, mine = min(max(n_rows - first, 0), share);
             const int owner = r / share;                            // of row r
@@ -888,7 +886,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         x[v] = t.x; x[v + 1] = t.y; x[v + 2] = t.z; x[v + 3] = t.w;
                     }
                 }, Ms, Ls, acc);
-                finish_row<VEC, 8>(p.fin, rq.q_row0 + merge.row_block * TB + rr / G, merge.kv_head * G + rr % G, lane & 7, Ms, Ls, acc);
+                finish_row<VEC, 8>(p.fin, merge.q_row0 + merge.row_block * TB + rr / G, merge.kv_head * G + rr % G, lane & 7, Ms, Ls, acc);
             }
             __syncwarp();
             cluster_wait();

@@ -34,7 +34,7 @@ struct DevItem {
     int32_t tile_end;
     int32_t slot;        // partial slot of sibling 0; sibling s writes slot + s
     int32_t seg;         // SEG_OTHER (prefix + query segment), SEG_CTX, or SEG_FINAL (encode: write O directly)
-    int32_t n_sib;       // live siblings of this item (row blocks that exist)
+    int32_t n_sib;       // live siblings of this item (row blocks that exist); 0: no work (cluster plans: a block without an item)
     // copies of the request geometry and of the first tile record, so that an item is ONE 64-byte load that the
     // tensor-core kernel fetches an item ahead (no dependent loads when it moves to the next item)
     int32_t q_row0;      // first row of Q / O of the request (encode: context start)
@@ -68,6 +68,7 @@ struct DevMerge {
     int32_t ctx_row_off; // added to the row when a context partial is read: shared-context plans keep the context
                          // partials of many requests in one slot, one group of rows per request
     int32_t ctx_stride;  // between consecutive context partials
+    int32_t q_row0;      // first row of Q / O of the request
 };
 
 // One node of a context tree (tree plans): a SEG_CTX item's ctx_id is the index of the node its tiles belong to.
