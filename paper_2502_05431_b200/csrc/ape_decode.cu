@@ -1,6 +1,6 @@
 // Split-KV decode kernel of APE attention: one new query token per request streams the whole cached
 // sequence [prefix | contexts | query segment] once.  HBM-bound: K/V tiles are brought in by the bulk
-// tensor copy engine through a multi-stage shared-memory ring; the small (G rows) x (16 tokens) products run on
+// tensor copy engine through a multi-stage shared-memory ring; the small (G heads) x (16 tokens) products run on
 // warp-level mma so that arithmetic never limits the stream.  Each work item covers tiles of ONE segment
 // (context, or prefix + query segment) and emits one partial (m, l, O~) in base-2 units; the merge kernel
 // applies the hierarchical softmax identity and Eq. 5's S afterwards.
@@ -17,7 +17,6 @@ constexpr int kConsumerWarps = 8;           // two groups of four; group w/4 tak
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
 constexpr int kMaxStages = 8;
 constexpr int kRecvRows = 32;               // (G rows, at most 16, rounded up to a multiple of the cluster's size, at most 16)
-constexpr int kRowPad = 8;                  // floats behind a row of the partials: the rows of a fragment's store fall on different banks
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -39,6 +38,219 @@ __device__ __forceinline__ uint32_t swz(int row, int chunk) {
     return static_cast<uint32_t>((chunk >> 3) * (kTile * 128) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
 }
 
+// 8 x 8 b16 matrix across the warp (lane: two elements of row lane / 4), transposed
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
+
+// The products of a warp with a slice of 16 tokens of a tile, and its running partial (m, l, O~) of the G query heads.  Two forms:
+//
+// HeadsAsColumns, at most eight heads: S^T = K Q^T and O^T = V^T P^T, so the tokens (or the elements of a head) are the 16 rows of an mma
+// and the heads its 8 columns, half the products that 16 rows for the heads take (of which four heads use a quarter).  A step that is not
+// bound by HBM is bound by these chains: 4 requests over 4 x 256 tokens 6.05 -> 5.74 us, 8 over 50 x 256 tokens (two KV heads of 64)
+// 13.4 -> 12.5, 4 over 100 x 256 (eight KV heads of one query head) 69.9 -> 68.2; 16 over 500 x 256, at the HBM rate, as before.
+// HeadsAsRows, 16 heads: O = P V with the heads as the rows.  As columns they are two groups, so as many products, and the maxima over the
+// tokens take three shuffles a head instead of two: 4 requests over 30 x 256 tokens 8.5 us, as columns 8.9.
+template <int D>
+struct HeadsAsColumns {
+    static constexpr int kKSteps = D / 16;
+    static constexpr int kRow = D + 4;      // floats between rows of the partials: a store of 8 elements of every second row falls on 32 banks
+    uint32_t qb[kKSteps][2];        // Q^T (D x 8; columns >= G are zero)
+    float o[D / 16][4];             // O^T: element 16 j + qr (+ 8) of heads 2 qc, + 1; m and l are those heads'
+    float m[2], l[2];
+
+    // Plain loads of Q: this grid exists while the kernel before it, which may be writing Q, still runs, and the read-only path is for data
+    // that nobody writes in a grid's lifetime.
+    __device__ __forceinline__ void begin(const __nv_bfloat16* q, int64_t head_stride, int G) {
+        const int lane = threadIdx.x & 31, qr = lane >> 2, qc = lane & 3;
+        #pragma unroll
+        for (int ks = 0; ks < kKSteps; ++ks) {
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(q + qr * head_stride + ks * 16 + 2 * qc);
+            qb[ks][0] = (qr < G) ? src[0] : 0u;
+            qb[ks][1] = (qr < G) ? src[4] : 0u;
+        }
+        #pragma unroll
+        for (int j = 0; j < D / 16; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
+        m[0] = m[1] = -INFINITY; l[0] = l[1] = 0.f;
+    }
+
+    __device__ __forceinline__ void tile(uint32_t k_s, uint32_t v_s, int tok0, int n_valid, float scale) {
+        const int lane = threadIdx.x & 31, qr = lane >> 2;
+        // (even and odd steps of the head dimension in accumulators of their own: half the chain of dependent products)
+        float sc[4] = {0.f, 0.f, 0.f, 0.f}, sd[4] = {0.f, 0.f, 0.f, 0.f};
+        {
+            const int row = tok0 + (lane & 15), chunk_sel = lane >> 4;
+            #pragma unroll
+            for (int ks = 0; ks < kKSteps; ++ks) {
+                uint32_t a[4];
+                ldmatrix_x4(k_s + swz(row, 2 * ks + chunk_sel), a[0], a[1], a[2], a[3]);
+                mma_bf16_16816((ks & 1) ? sd : sc, a, qb[ks][0], qb[ks][1]);
+            }
+        }
+        // base-2 logits of this lane's two tokens and two heads, validity mask
+        const bool v0 = tok0 + qr < n_valid, v1 = tok0 + qr + 8 < n_valid;
+        float x[4];
+        #pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = (i < 2 ? v0 : v1) ? (sc[i] + sd[i]) * scale : -INFINITY;
+        float mx0 = fmaxf(x[0], x[2]), mx1 = fmaxf(x[1], x[3]);
+        #pragma unroll
+        for (int d = 4; d < 32; d *= 2) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, d));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, d));
+        }
+        const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);       // finite: the slice holds a valid key
+        if (__any_sync(0xffffffffu, (mn0 > m[0]) | (mn1 > m[1]))) {
+            const float f0 = fast_exp2(m[0] - mn0), f1 = fast_exp2(m[1] - mn1);
+            l[0] *= f0; l[1] *= f1;
+            #pragma unroll
+            for (int j = 0; j < D / 16; ++j) { o[j][0] *= f0; o[j][1] *= f1; o[j][2] *= f0; o[j][3] *= f1; }
+            m[0] = mn0; m[1] = mn1;
+        }
+        const float p0 = fast_exp2(x[0] - m[0]), p1 = fast_exp2(x[1] - m[1]), p2 = fast_exp2(x[2] - m[0]), p3 = fast_exp2(x[3] - m[1]);
+        l[0] += p0 + p2;
+        l[1] += p1 + p3;
+        const uint32_t b0 = movmatrix_trans(pack_bf16x2(p0, p1)), b1 = movmatrix_trans(pack_bf16x2(p2, p3));
+        {
+            const int row = tok0 + ((lane >> 4) << 3) + (lane & 7), chunk_sel = (lane >> 3) & 1;
+            #pragma unroll
+            for (int j = 0; j < D / 16; ++j) {
+                uint32_t a[4];
+                ldmatrix_x4_trans(v_s + swz(row, 2 * j + chunk_sel), a[0], a[1], a[2], a[3]);
+                mma_bf16_16816(o[j], a, b0, b1);
+            }
+        }
+    }
+
+    // into shared memory: row g at rows + g * RS, its (m, l) at ms[8 g], ls[8 g]
+    __device__ __forceinline__ void hand_in(float* rows, float* ms, float* ls, int G) {
+        constexpr int RS = kRow;
+        const int lane = threadIdx.x & 31, qr = lane >> 2, qc = lane & 3;
+        #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = 2 * qc + h;
+            #pragma unroll
+            for (int d = 4; d < 32; d *= 2) l[h] += __shfl_xor_sync(0xffffffffu, l[h], d);
+            if (qr == 0) { ms[row * 8] = m[h]; ls[row * 8] = l[h]; }
+            if (row < G) {
+                float* dst = rows + row * RS + qr;
+                #pragma unroll
+                for (int j = 0; j < D / 16; ++j) { dst[16 * j] = o[j][h]; dst[16 * j + 8] = o[j][2 + h]; }
+            }
+        }
+    }
+};
+
+template <int D>
+struct HeadsAsRows {
+    static constexpr int kKSteps = D / 16;
+    static constexpr int kRow = D + 8;      // (pairs of elements of eight rows)
+    uint32_t qa[kKSteps][4];        // Q (16 x D; rows >= G are zero)
+    float o[D / 8][4];              // O: heads qr, qr + 8, elements 8 j + 2 qc, + 1
+    float m_lo, m_hi, l_lo, l_hi;
+
+    __device__ __forceinline__ void begin(const __nv_bfloat16* q, int64_t head_stride, int G) {
+        const int lane = threadIdx.x & 31, qr = lane >> 2, qc = lane & 3;
+        #pragma unroll
+        for (int ks = 0; ks < kKSteps; ++ks) {
+            const uint32_t* r_lo = reinterpret_cast<const uint32_t*>(q + qr * head_stride + ks * 16 + 2 * qc);
+            const uint32_t* r_hi = reinterpret_cast<const uint32_t*>(q + (qr + 8) * head_stride + ks * 16 + 2 * qc);
+            qa[ks][0] = (qr < G) ? *r_lo : 0u;
+            qa[ks][1] = (qr + 8 < G) ? *r_hi : 0u;
+            qa[ks][2] = (qr < G) ? r_lo[4] : 0u;
+            qa[ks][3] = (qr + 8 < G) ? r_hi[4] : 0u;
+        }
+        #pragma unroll
+        for (int j = 0; j < D / 8; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
+        m_lo = m_hi = -INFINITY; l_lo = l_hi = 0.f;
+    }
+
+    __device__ __forceinline__ void tile(uint32_t k_s, uint32_t v_s, int tok0, int n_valid, float scale) {
+        const int lane = threadIdx.x & 31, qc = lane & 3;
+        // S = Q K^T for 16 tokens: two n-tiles of 8 tokens
+        // (even and odd steps of the head dimension in accumulators of their own: half the chain of dependent products)
+        float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        {
+            const int row = tok0 + ((lane >> 4) << 3) + (lane & 7);
+            const int chunk_sel = (lane >> 3) & 1;
+            #pragma unroll
+            for (int ks = 0; ks < kKSteps; ++ks) {
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4(k_s + swz(row, 2 * ks + chunk_sel), b0, b1, b2, b3);
+                mma_bf16_16816((ks & 1) ? sd[0] : sc[0], qa[ks], b0, b1);
+                mma_bf16_16816((ks & 1) ? sd[1] : sc[1], qa[ks], b2, b3);
+            }
+            #pragma unroll
+            for (int i = 0; i < 4; ++i) { sc[0][i] += sd[0][i]; sc[1][i] += sd[1][i]; }
+        }
+        // base-2 logits, validity mask
+        #pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            const int c0 = tok0 + nt * 8 + 2 * qc;
+            const bool v0 = c0 < n_valid, v1 = c0 + 1 < n_valid;
+            sc[nt][0] = v0 ? sc[nt][0] * scale : -INFINITY;
+            sc[nt][1] = v1 ? sc[nt][1] * scale : -INFINITY;
+            sc[nt][2] = v0 ? sc[nt][2] * scale : -INFINITY;
+            sc[nt][3] = v1 ? sc[nt][3] * scale : -INFINITY;
+        }
+        float mx_lo = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1]));
+        float mx_hi = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3]));
+        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
+        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
+        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
+        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
+        const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);   // finite: the slice holds a valid key
+        if (__any_sync(0xffffffffu, (mn_lo > m_lo) | (mn_hi > m_hi))) {
+            const float f_lo = fast_exp2(m_lo - mn_lo), f_hi = fast_exp2(m_hi - mn_hi);
+            l_lo *= f_lo; l_hi *= f_hi;
+            #pragma unroll
+            for (int j = 0; j < D / 8; ++j) { o[j][0] *= f_lo; o[j][1] *= f_lo; o[j][2] *= f_hi; o[j][3] *= f_hi; }
+            m_lo = mn_lo; m_hi = mn_hi;
+        }
+        uint32_t pa[4];
+        {
+            const float p00 = fast_exp2(sc[0][0] - m_lo), p01 = fast_exp2(sc[0][1] - m_lo);
+            const float p02 = fast_exp2(sc[0][2] - m_hi), p03 = fast_exp2(sc[0][3] - m_hi);
+            const float p10 = fast_exp2(sc[1][0] - m_lo), p11 = fast_exp2(sc[1][1] - m_lo);
+            const float p12 = fast_exp2(sc[1][2] - m_hi), p13 = fast_exp2(sc[1][3] - m_hi);
+            l_lo += (p00 + p01) + (p10 + p11);
+            l_hi += (p02 + p03) + (p12 + p13);
+            pa[0] = pack_bf16x2(p00, p01); pa[1] = pack_bf16x2(p02, p03);
+            pa[2] = pack_bf16x2(p10, p11); pa[3] = pack_bf16x2(p12, p13);
+        }
+        // O += P V
+        {
+            const int row = tok0 + (((lane >> 3) & 1) << 3) + (lane & 7);
+            const int chunk_sel = lane >> 4;
+            #pragma unroll
+            for (int j = 0; j < D / 16; ++j) {
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4_trans(v_s + swz(row, 2 * j + chunk_sel), b0, b1, b2, b3);
+                mma_bf16_16816(o[2 * j], pa, b0, b1);
+                mma_bf16_16816(o[2 * j + 1], pa, b2, b3);
+            }
+        }
+    }
+
+    __device__ __forceinline__ void hand_in(float* rows, float* ms, float* ls, int G) {
+        constexpr int RS = kRow;
+        const int lane = threadIdx.x & 31, qr = lane >> 2, qc = lane & 3;
+        l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
+        l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1); l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
+        if (qc == 0) {
+            ms[qr * 8] = m_lo; ms[(qr + 8) * 8] = m_hi;
+            ls[qr * 8] = l_lo; ls[(qr + 8) * 8] = l_hi;
+        }
+        #pragma unroll
+        for (int j = 0; j < D / 8; ++j) {
+            const int e = j * 8 + 2 * qc;
+            if (qr < G) *reinterpret_cast<float2*>(&rows[qr * RS + e]) = make_float2(o[j][0], o[j][1]);
+            if (qr + 8 < G) *reinterpret_cast<float2*>(&rows[(qr + 8) * RS + e]) = make_float2(o[j][2], o[j][3]);
+        }
+    }
+};
+
 }  // namespace
 
 // A long step is bound by HBM (16 requests over 128K tokens: 6.7 TB/s), a short one by a chain of latencies, in cycles for one request
@@ -51,20 +263,19 @@ __device__ __forceinline__ uint32_t swz(int row, int chunk) {
 // cluster), so that a short step is one kernel, no partial goes to memory and no second kernel waits for the last block of the
 // first: 5.8 us for the step above, 3.7 instead of 5.1 for a single context of 64 tokens.  (Sent, not fetched: reading the others'
 // partials behind the barrier cost another 1,600 cycles and a second barrier before a block may leave.)
-template <int D, bool CLUSTER>
+template <int D, bool CLUSTER, typename Products>
 __global__ void __launch_bounds__(kThreads, 1)
 ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                   const __grid_constant__ DecodeParams p)
 {
     constexpr int kSlabs = D / 64;
     constexpr int kStageBytes = 2 * kTile * D * 2;      // K + V
-    constexpr int kKSteps = D / 16;
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int n_stages = p.n_stages;
     uint8_t* stage_base = smem;
-    constexpr int RS = D + kRowPad;
+    constexpr int RS = Products::kRow;
     float* red = reinterpret_cast<float*>(smem + static_cast<size_t>(n_stages) * kStageBytes);  // [8][G][RS], then [16][8] m, [16][8] l
     float* red_m = red + kConsumerWarps * p.G * RS;
     float* red_l = red_m + kConsumerWarps * 16;
@@ -159,7 +370,6 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
         const int grp = warp >> 2;            // which half of the tiles
         const int w4 = warp & 3;              // 16-token slice inside a tile
         const int G = p.G;
-        const int qr = lane >> 2, qc = lane & 3;
         uint32_t cnt = 0;
 
         for (int it = item_begin; it < item_end; ++it) {
@@ -167,28 +377,8 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
             const float scale = (item.seg == SEG_CTX) ? p.scale_ctx_log2 : p.scale_oth_log2;
             const int t_end = live_end(item);
 
-            // Q fragments (A operand, 16 x D, rows >= G are zero).  Plain loads: this grid exists while the kernel before it, which
-            // may be writing Q, still runs, and the read-only path is for data that nobody writes in a grid's lifetime.
-            uint32_t qa[kKSteps][4];
-            {
-                const __nv_bfloat16* qbase = p.q.data + static_cast<int64_t>(item.q_row0) * p.q.token_stride
-                                             + static_cast<int64_t>(item.kv_head) * G * p.q.head_stride;
-                #pragma unroll
-                for (int ks = 0; ks < kKSteps; ++ks) {
-                    const int col = ks * 16 + 2 * qc;
-                    const uint32_t* r_lo = reinterpret_cast<const uint32_t*>(qbase + static_cast<int64_t>(qr) * p.q.head_stride + col);
-                    const uint32_t* r_hi = reinterpret_cast<const uint32_t*>(qbase + static_cast<int64_t>(qr + 8) * p.q.head_stride + col);
-                    qa[ks][0] = (qr < G) ? *r_lo : 0u;
-                    qa[ks][1] = (qr + 8 < G) ? *r_hi : 0u;
-                    qa[ks][2] = (qr < G) ? r_lo[4] : 0u;
-                    qa[ks][3] = (qr + 8 < G) ? r_hi[4] : 0u;
-                }
-            }
-
-            float o[D / 8][4];
-            #pragma unroll
-            for (int j = 0; j < D / 8; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
-            float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
+            Products part;
+            part.begin(p.q.data + static_cast<int64_t>(item.q_row0) * p.q.token_stride + static_cast<int64_t>(item.kv_head) * G * p.q.head_stride, p.q.head_stride, G);
 
             for (int t = item.tile_begin; t < t_end; ++t, ++cnt) {
                 if ((cnt & 1u) != static_cast<uint32_t>(grp)) continue;
@@ -217,87 +407,14 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
                         __syncwarp();
                     }
 
-                    // S = Q K^T for 16 tokens: two n-tiles of 8 tokens
-                    // (even and odd steps of the head dimension in accumulators of their own: half the chain of dependent products)
-                    float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, sd[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-                    {
-                        const int row = tok0 + ((lane >> 4) << 3) + (lane & 7);
-                        const int chunk_sel = (lane >> 3) & 1;
-                        #pragma unroll
-                        for (int ks = 0; ks < kKSteps; ++ks) {
-                            uint32_t b0, b1, b2, b3;
-                            ldmatrix_x4(k_s + swz(row, 2 * ks + chunk_sel), b0, b1, b2, b3);
-                            mma_bf16_16816((ks & 1) ? sd[0] : sc[0], qa[ks], b0, b1);
-                            mma_bf16_16816((ks & 1) ? sd[1] : sc[1], qa[ks], b2, b3);
-                        }
-                        #pragma unroll
-                        for (int i = 0; i < 4; ++i) { sc[0][i] += sd[0][i]; sc[1][i] += sd[1][i]; }
-                    }
-                    // base-2 logits, validity mask
-                    #pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        const int c0 = tok0 + nt * 8 + 2 * qc;
-                        const bool v0 = c0 < n_valid, v1 = c0 + 1 < n_valid;
-                        sc[nt][0] = v0 ? sc[nt][0] * scale : -INFINITY;
-                        sc[nt][1] = v1 ? sc[nt][1] * scale : -INFINITY;
-                        sc[nt][2] = v0 ? sc[nt][2] * scale : -INFINITY;
-                        sc[nt][3] = v1 ? sc[nt][3] * scale : -INFINITY;
-                    }
-                    float mx_lo = fmaxf(fmaxf(sc[0][0], sc[0][1]), fmaxf(sc[1][0], sc[1][1]));
-                    float mx_hi = fmaxf(fmaxf(sc[0][2], sc[0][3]), fmaxf(sc[1][2], sc[1][3]));
-                    mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-                    mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-                    mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-                    mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-                    const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);   // finite: the slice holds a valid key
-                    if (__any_sync(0xffffffffu, (mn_lo > m_lo) | (mn_hi > m_hi))) {
-                        const float f_lo = fast_exp2(m_lo - mn_lo), f_hi = fast_exp2(m_hi - mn_hi);
-                        l_lo *= f_lo; l_hi *= f_hi;
-                        #pragma unroll
-                        for (int j = 0; j < D / 8; ++j) { o[j][0] *= f_lo; o[j][1] *= f_lo; o[j][2] *= f_hi; o[j][3] *= f_hi; }
-                        m_lo = mn_lo; m_hi = mn_hi;
-                    }
-                    uint32_t pa[4];
-                    {
-                        const float p00 = fast_exp2(sc[0][0] - m_lo), p01 = fast_exp2(sc[0][1] - m_lo);
-                        const float p02 = fast_exp2(sc[0][2] - m_hi), p03 = fast_exp2(sc[0][3] - m_hi);
-                        const float p10 = fast_exp2(sc[1][0] - m_lo), p11 = fast_exp2(sc[1][1] - m_lo);
-                        const float p12 = fast_exp2(sc[1][2] - m_hi), p13 = fast_exp2(sc[1][3] - m_hi);
-                        l_lo += (p00 + p01) + (p10 + p11);
-                        l_hi += (p02 + p03) + (p12 + p13);
-                        pa[0] = pack_bf16x2(p00, p01); pa[1] = pack_bf16x2(p02, p03);
-                        pa[2] = pack_bf16x2(p10, p11); pa[3] = pack_bf16x2(p12, p13);
-                    }
-                    // O += P V
-                    {
-                        const int row = tok0 + (((lane >> 3) & 1) << 3) + (lane & 7);
-                        const int chunk_sel = lane >> 4;
-                        #pragma unroll
-                        for (int j = 0; j < D / 16; ++j) {
-                            uint32_t b0, b1, b2, b3;
-                            ldmatrix_x4_trans(v_s + swz(row, 2 * j + chunk_sel), b0, b1, b2, b3);
-                            mma_bf16_16816(o[2 * j], pa, b0, b1);
-                            mma_bf16_16816(o[2 * j + 1], pa, b2, b3);
-                        }
-                    }
+                    part.tile(k_s, v_s, tok0, n_valid, scale);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_empty + 8 * s);
             }
 
             // ---- combine the eight warps' partials of this item and write one (m, l, O~) to the workspace ------------
-            l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-            l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1); l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
-            if (qc == 0) {
-                red_m[qr * 8 + warp] = m_lo; red_m[(qr + 8) * 8 + warp] = m_hi;
-                red_l[qr * 8 + warp] = l_lo; red_l[(qr + 8) * 8 + warp] = l_hi;
-            }
-            #pragma unroll
-            for (int j = 0; j < D / 8; ++j) {
-                const int e = j * 8 + 2 * qc;
-                if (qr < G) *reinterpret_cast<float2*>(&red[(warp * G + qr) * RS + e]) = make_float2(o[j][0], o[j][1]);
-                if (qr + 8 < G) *reinterpret_cast<float2*>(&red[(warp * G + qr + 8) * RS + e]) = make_float2(o[j][2], o[j][3]);
-            }
+            part.hand_in(red + warp * G * RS, red_m + warp, red_l + warp, G);
             // Every consumer warp reaches this barrier, also one that gave up on a wait, so the decision to stop is
             // taken by all of them together.
             named_bar_sync(1, kConsumerWarps * 32);
@@ -361,9 +478,10 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
 }
 
 size_t decode_smem_bytes(int D, int G, int n_stages, int cluster) {
+    const int row = G <= 8 ? HeadsAsColumns<128>::kRow - 128 + D : HeadsAsRows<128>::kRow - 128 + D;
     return 1024 + static_cast<size_t>(n_stages) * (2 * kTile * D * 2)
-           + sizeof(float) * (kConsumerWarps * G * (D + kRowPad) + 2 * kConsumerWarps * 16) + 16 * kMaxStages
-           + (cluster > 0 ? sizeof(float) * (D + kRowPad) * ((G + cluster - 1) / cluster * cluster) : 0);
+           + sizeof(float) * (kConsumerWarps * G * row + 2 * kConsumerWarps * 16) + 16 * kMaxStages
+           + (cluster > 0 ? sizeof(float) * row * ((G + cluster - 1) / cluster * cluster) : 0);
 }
 
 int decode_pick_stages(int D, int G, size_t smem_limit, int cluster) {
@@ -372,25 +490,36 @@ int decode_pick_stages(int D, int G, size_t smem_limit, int cluster) {
     return decode_smem_bytes(D, G, n, cluster) <= smem_limit ? n : 0;
 }
 
+using DecodeKernel = void(CUtensorMap, CUtensorMap, DecodeParams);
+template <int D>
+static DecodeKernel* decode_kernel(bool cluster, int G) {
+    if (G <= 8) return cluster ? ape_decode_kernel<D, true, HeadsAsColumns<D>> : ape_decode_kernel<D, false, HeadsAsColumns<D>>;
+    return cluster ? ape_decode_kernel<D, true, HeadsAsRows<D>> : ape_decode_kernel<D, false, HeadsAsRows<D>>;
+}
+static DecodeKernel* decode_kernel(int D, bool cluster, int G) { return D == 128 ? decode_kernel<128>(cluster, G) : decode_kernel<64>(cluster, G); }
+
 cudaError_t launch_decode(int D, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const DecodeParams& p,
                           int n_cta, size_t smem_bytes, bool early, cudaStream_t stream)
 {
-    if (p.cluster > 0)
-        return launch_cluster(p.cluster, early, D == 128 ? ape_decode_kernel<128, true> : ape_decode_kernel<64, true>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
-    return launch_kernel(early, D == 128 ? ape_decode_kernel<128, false> : ape_decode_kernel<64, false>, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
+    const bool c = p.cluster > 0;
+    auto* kernel = decode_kernel(D, c, p.G);
+    return c ? launch_cluster(p.cluster, early, kernel, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p)
+             : launch_kernel(early, kernel, n_cta, kThreads, smem_bytes, stream, tm_k, tm_v, p);
 }
 
 cudaError_t decode_set_smem_attr(int D, size_t smem_limit) {
-    const int n = static_cast<int>(smem_limit);
-    cudaError_t e = cudaFuncSetAttribute(D == 128 ? ape_decode_kernel<128, false> : ape_decode_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    if (e != cudaSuccess) return e;
-    auto* kernel = D == 128 ? ape_decode_kernel<128, true> : ape_decode_kernel<64, true>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int g : {8, 16})
+        for (bool c : {false, true}) {
+            auto* kernel = decode_kernel(D, c, g);
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_limit));
+            if (e == cudaSuccess && c) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 int decode_max_clusters(int D, int cluster, size_t smem_limit) {
-    return max_clusters(cluster, D == 128 ? ape_decode_kernel<128, true> : ape_decode_kernel<64, true>, kThreads, smem_limit);
+    return max_clusters(cluster, decode_kernel(D, true, 8), kThreads, smem_limit);
 }
 
 }  // namespace ape
