@@ -53,7 +53,7 @@ struct ape_plan_s {
     int32_t* d_cta_begin = nullptr;
     DevReq* d_reqs = nullptr;
     DevMerge* d_merge = nullptr;
-    int n_items = 0, n_cta = 0, n_merge = 0, n_sib = 1, n_slots = 0;
+    int n_items = 0, n_cta = 0, n_merge = 0, n_sib = 1, n_slots = 0, max_partials = 0;
     int n_stages = 0;
     size_t smem_bytes = 0;
     size_t ws_bytes = 0;
@@ -431,6 +431,12 @@ void finish_items(HostMeta& m) {
     for (auto& g : m.merge) g.q_row0 = m.reqs[g.req].q_row0;
 }
 
+int most_partials(const HostMeta& m) {       // of a segment of a row
+    int most = 0;
+    for (const auto& g : m.merge) most = std::max({most, g.ctx_n, g.oth_n});
+    return most;
+}
+
 int upload(ape_plan_t p, const HostMeta& m) {
     auto rnd = [](size_t x) { return (x + 255) & ~size_t(255); };
     const size_t b_tiles = rnd(m.tiles.size() * sizeof(DevTile) + 16), b_items = rnd(m.items.size() * sizeof(DevItem) + 16),
@@ -464,6 +470,7 @@ int upload(ape_plan_t p, const HostMeta& m) {
     p->d_levels = reinterpret_cast<int32_t*>(b + o_lv);
     p->n_items = static_cast<int>(m.items.size());
     p->n_merge = static_cast<int>(m.merge.size());
+    p->max_partials = most_partials(m);
     return APE_OK;
 }
 
@@ -1351,7 +1358,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = nullptr; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = p->n_merge;
         mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = b_o; mp.ws_ml = b_ml;
         mp.ws_o_ctx = a_o; mp.ws_ml_ctx = a_ml; mp.rows_per_slot_ctx = a->alt_halves ? kAttnRows / 2 : kAttnRows;
-        static_cast<RowsOut&>(mp) = rows_out; mp.G = G; mp.D = D; mp.n_sm = p->h->n_sm_device;
+        static_cast<RowsOut&>(mp) = rows_out; mp.G = G; mp.D = D; mp.n_sm = p->h->n_sm_device; mp.max_partials = p->max_partials;
         if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
         p->last_launches++;
         return APE_OK;
@@ -1410,7 +1417,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
     mp.groups = p->d_merge; mp.reqs = p->d_reqs; mp.items = p->d_items; mp.per_context = p->two_pass ? 0 : p->per_context; mp.nodes = p->d_nodes; mp.n_groups = p->n_merge; mp.rows_per_slot = rows_per_slot;
     mp.tokens_per_block = rows_per_slot / G; mp.ws_o = ws_o; mp.ws_ml = ws_ml;
     mp.ws_o_ctx = ws_o; mp.ws_ml_ctx = ws_ml; mp.rows_per_slot_ctx = rows_per_slot;
-    static_cast<RowsOut&>(mp) = rows_out; mp.G = G; mp.D = D; mp.n_sm = p->h->n_sm_device;
+    static_cast<RowsOut&>(mp) = rows_out; mp.G = G; mp.D = D; mp.n_sm = p->h->n_sm_device; mp.max_partials = p->max_partials;
     if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
     p->last_launches++;
     return APE_OK;
@@ -1701,6 +1708,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     if (!reqs || n_req <= 0 || out->n_rows < q->n_rows) return APE_ERR_INVALID_ARG;
     if (!(T > 0.f) || !(S > 0.f) || !std::isfinite(T) || !std::isfinite(S)) return APE_ERR_RANGE;
     int64_t max_extra = INT64_MAX, total_tiles = 0;
+    int max_partials = 0;
     try {
         for (int r = 0; r < n_req; ++r) {
             const ape_request_t& rq = reqs[r];
@@ -1761,6 +1769,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
         }
         assign_stream(runs, n_cta, 1, kDecodeItemTiles, m);
         finish_items(m);
+        max_partials = most_partials(m);
         auto rnd = [](size_t x) { return (x + 255) & ~size_t(255); };
         o_tiles = 256;                                                     // after the status word
         o_items = o_tiles + rnd(m.tiles.size() * sizeof(DevTile));
@@ -1817,7 +1826,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = ws_o; mp.ws_ml = ws_ml; mp.out = rows_desc(*out); mp.lse_out = lse;
     mp.ws_o_ctx = ws_o; mp.ws_ml_ctx = ws_ml; mp.rows_per_slot_ctx = G;
     mp.part_o_ctx = nullptr; mp.part_lse_ctx = nullptr; mp.part_o_oth = nullptr; mp.part_lse_oth = nullptr;
-    mp.S = S; mp.G = G; mp.H_q = shape->n_q_heads; mp.D = D; mp.n_sm = dv->h.n_sm;
+    mp.S = S; mp.G = G; mp.H_q = shape->n_q_heads; mp.D = D; mp.n_sm = dv->h.n_sm; mp.max_partials = max_partials;
     if (launch_merge(mp, stream) != cudaSuccess) return APE_ERR_CUDA;
     if (device_status != nullptr) {
         // the caller asked for the status word: this makes the call synchronous; a word that was set is cleared once read

@@ -128,6 +128,7 @@ struct MergeParams : RowsOut {
     int32_t G;
     int32_t D;
     int32_t n_sm;                    // SMs of the device (an SM budget does not limit the merge)
+    int32_t max_partials;            // of a segment of a row
 };
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
 

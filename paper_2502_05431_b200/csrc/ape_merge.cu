@@ -324,6 +324,76 @@ __global__ void __launch_bounds__(256, 4) ape_merge_kernel(const MergeParams p)
     finish_row<VEC>(p, rq.q_row0 + tok, g.kv_head * p.G + row % p.G, lane, M, L, acc);
 }
 
+// Eq. 5 form for rows of few partials (at most kRowPartials a segment): eight lanes to a row, so that a warp has the loads of four rows
+// under way, and every lane reads a row's (m, l) itself instead of twenty shuffles a row.  Bound by the latency of the loads.
+constexpr int kRowPartials = 8;
+template <int VEC>
+__global__ void __launch_bounds__(128, 4) ape_merge_rows_kernel(const MergeParams p)
+{
+    constexpr int kBatch = 3;
+    constexpr int D = VEC * 8;
+    const int lane = threadIdx.x & 7;
+    const int row_global = blockIdx.x * (blockDim.x / 8) + threadIdx.x / 8;
+    const int group = row_global / p.rows_per_slot;
+    const int row = row_global - group * p.rows_per_slot;
+    bool live = group < p.n_groups;
+    DevMerge g{};
+    DevReq rq{};
+    if (live) { g = p.groups[group]; rq = p.reqs[g.req]; }
+    const int tok = g.row_block * p.tokens_per_block + row / p.G;     // query row inside the request
+    live = live && tok < rq.q_len;
+    pdl_wait();
+    pdl_trigger();
+    if (!live) return;
+    float M[2], L[2], acc[2][VEC];                                    // context, other
+    #pragma unroll
+    for (int seg = 0; seg < 2; ++seg) {
+        const int n = seg ? g.oth_n : g.ctx_n, per_slot = seg ? p.rows_per_slot : p.rows_per_slot_ctx;
+        const size_t row0 = static_cast<size_t>(seg ? g.oth_slot0 : g.ctx_slot0) * per_slot + row + (seg ? 0 : g.ctx_row_off);
+        const size_t step = static_cast<size_t>(seg ? g.slot_stride : g.ctx_stride) * per_slot;        // rows between consecutive partials
+        const float2* ml_at = reinterpret_cast<const float2*>(seg ? p.ws_ml : p.ws_ml_ctx) + row0;
+        const float* src = (seg ? p.ws_o : p.ws_o_ctx) + row0 * D + lane * 4;
+        float2 ml[kRowPartials];
+        #pragma unroll
+        for (int j = 0; j < kRowPartials; ++j) ml[j] = (j < n) ? ml_at[j * step] : make_float2(-INFINITY, 0.f);
+        float x[kBatch][VEC];
+        // The row of an empty partial was never written, but it lies inside the workspace, and the fold never looks at what was read from it.
+        auto load = [&](int j0) {
+            #pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                if (j0 + u < n) {
+                    #pragma unroll
+                    for (int v = 0; v < VEC; v += 4) {
+                        const float4 t = *reinterpret_cast<const float4*>(src + (j0 + u) * step * D + v * 8);
+                        x[u][v] = t.x; x[u][v + 1] = t.y; x[u][v + 2] = t.z; x[u][v + 3] = t.w;
+                    }
+                }
+        };
+        load(0);
+        float top = -INFINITY, sum = 0.f;
+        #pragma unroll
+        for (int j = 0; j < kRowPartials; ++j) top = fmaxf(top, (ml[j].y > 0.f) ? ml[j].x : -INFINITY);       // (empty partial: no positive sum)
+        const float base = (top == -INFINITY) ? 0.f : top;
+        #pragma unroll
+        for (int v = 0; v < VEC; ++v) acc[seg][v] = 0.f;
+        #pragma unroll
+        for (int j0 = 0; j0 < kRowPartials; j0 += kBatch) {
+            if (j0 >= n) break;
+            if (j0 > 0) load(j0);
+            #pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                if (j0 + u < kRowPartials && j0 + u < n && ml[j0 + u].y > 0.f) {
+                    const float f = fast_exp2(ml[j0 + u].x - base);
+                    sum += ml[j0 + u].y * f;
+                    #pragma unroll
+                    for (int v = 0; v < VEC; ++v) acc[seg][v] += x[u][v] * f;
+                }
+        }
+        M[seg] = top; L[seg] = sum;
+    }
+    finish_row<VEC, 8>(p, rq.q_row0 + tok, g.kv_head * p.G + row % p.G, lane, M, L, acc);
+}
+
 // Plans of the per-context form and of context trees that keep a partial per node (decode; prefill of few nodes): one warp per output row
 // walks the partials in order.
 template <int VEC, bool TREE>
@@ -555,7 +625,13 @@ cudaError_t launch_merge_vec(const MergeParams& p, long long rows, cudaStream_t 
     // 60.5 with eight; 16 requests over shared 128K tokens: 129.0 and 124.4).  With more rows the warps of other rows hide it,
     // and sharing a row only adds the meeting in shared memory (64 rows over 10 x 256 tokens, 2048 rows to merge: 19.4 us with
     // one, 24.4 with eight; 4 x 128 rows over 20K tokens: 212 and 254).
-    if (rows <= 4ll * p.n_sm) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
+    // Of those with more rows, the ones with few partials a segment (most prefills: the runs of a head span few blocks) take eight lanes to a
+    // row: 4 x 128 rows over 20 documents each, five partials, 203 us per call with a warp per row, 198 this way; 2 x 256 rows over 20 x 256
+    // tokens 69.3 and 64.1.  (Few rows: 4 requests' decode step over 20 documents 55.9 with eight warps per row, 57.1-57.9 this way.)
+    const bool few = rows <= 4ll * p.n_sm;
+    if (!few && p.max_partials <= kRowPartials)
+        return launch_pdl(ape_merge_rows_kernel<VEC * 4>, static_cast<unsigned>((rows + 15) / 16), 128, 0, stream, p);
+    if (few) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
     return launch_pdl(ape_merge_kernel<VEC, 1>, static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
 }
 }  // namespace

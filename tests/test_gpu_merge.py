@@ -33,6 +33,18 @@ def test_partials_per_row(n_sm, mode, d, l_q):
         handle().set_sm_budget(0)
 
 
+@pytest.mark.parametrize("n_sm", [1, 7, 8, 9, 10, 16, 0])
+@pytest.mark.parametrize("d,G,l_q", [(64, 4, 151), (128, 1, 601), (64, 16, 41), (128, 4, 149)])
+def test_many_rows_with_few_and_with_more_partials(n_sm, d, G, l_q):
+    """More rows than the eight-warp form takes: up to eight partials a segment eight lanes share a row, with more a warp has it."""
+    b = wl.make_batch(H_q=G, H_kv=1, d=d, l_P=70, ctx_lens=[[2000]], l_q=l_q, l_k=l_q + 40, seed=34, T=0.8, S=0.9, name=f"merge_rows_sm{n_sm}")
+    handle().set_sm_budget(n_sm)
+    try:
+        _check(b, libape.APE_PREFILL)
+    finally:
+        handle().set_sm_budget(0)
+
+
 def test_more_partials_than_one_round_of_lanes():
     """One KV head and a shared-context batch of at most 128 rows, two tiles per thread block: two partials per block, 296 per row on
     148 SMs, of which the eight warps of a row take 256 in one round."""
