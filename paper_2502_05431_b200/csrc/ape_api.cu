@@ -233,7 +233,7 @@ struct HostMeta {
 
 // What the end of an item costs, in tiles: 0.8 us against 0.6 per tile (decode kernel), 5,000 to 8,000 cycles against 3,500 (attention
 // kernel).
-constexpr int kDecodeItemTiles = 1, kAttnItemTiles = 2;
+constexpr int kDecodeItemTiles = 1, kAttnItemTiles = 2, kLongRun = 32;
 
 // The decode kernel's static shared memory, which counts against the same limit (1,024 bytes, and as much to spare).
 constexpr size_t kDecodeStaticSmem = 2048;
@@ -251,7 +251,13 @@ struct Run {   // a run of tiles of one segment for one (request, kv head, row-b
 // can be cut into bins of its own without the largest bin growing by more than that, no bin gets two items.
 // (One request over 10 x 256 tokens, eight heads x (40 + 3) tiles on 148 blocks: 9.25 us per step with blocks of 3 tiles of
 // which some held two items, 8.02 this way; 16 requests over shared 128K tokens: 121.6 and 119.2.)
-void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int item_tiles, HostMeta& m, bool align_nodes = false) {
+// Otherwise the bins get equal shares of tiles and items' ends together, so that no bin is the last one for its many items.  Equal shares
+// of tiles alone / this way, us: prefill, 4 x 128 rows over 20 documents 199 / 191, 256 rows over 500 x 256 tokens 533 / 525, 2 x 229 rows
+// over 71 contexts of 158 to 474 tokens (8 KV heads) 73.8 / 63.2, 4 x 125 rows over 181 short ones 42.7 / 36.1; decode, 3 requests over 7
+// contexts of 206 to 618 tokens 10.4 / 9.5, per-context form, 5 over 45 of 154 to 463 21.5 / 20.3.  Of 27 such drawn calls one was slower
+// (15.9 / 16.2).  Not in decode plans whose runs have more than kLongRun tiles on average: there an end is hidden behind the stream of the other
+// blocks and only the bytes count (4 requests over 61 contexts of 126 tokens, 65 tiles a run, 24.6 / 25.1).
+void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int item_tiles, HostMeta& m, bool align_nodes = false, bool weigh_ends = true) {
     long long total = 0;
     for (const auto& r : runs) total += r.t1 - r.t0;
     const long long chunk = std::max<long long>(1, (total + n_bins - 1) / n_bins);
@@ -261,14 +267,35 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int 
         for (const auto& r : runs) bins += (r.t1 - r.t0 + u - 1) / u;
         if (bins <= n_bins) own = u;
     }
+    const bool hidden = item_tiles == kDecodeItemTiles && total > kLongRun * static_cast<long long>(runs.size());
+    const long long end = (own || align_nodes || hidden || !weigh_ends) ? 0 : item_tiles;
+    long long share = chunk;
+    if (end > 0) {
+        auto bins_for = [&](long long u) {
+            long long bins = 1, room = u;
+            for (const auto& r : runs)
+                for (long long left = r.t1 - r.t0; left > 0;) {
+                    if (room <= end) { ++bins; room = u; }
+                    const long long take = std::min(left, room - end);
+                    left -= take; room -= take + end;
+                }
+            return bins;
+        };
+        long long lo = std::max((total + end * static_cast<long long>(runs.size()) - 1) / n_bins, end), step = 1;      // below the mean: too small
+        while (bins_for(lo + step) > n_bins) { lo += step; step *= 2; }
+        long long hi = lo + step;
+        while (hi - lo > 1) { const long long mid = (lo + hi) / 2; (bins_for(mid) <= n_bins ? hi : lo) = mid; }
+        share = hi;
+    }
     m.cta_begin.assign(1, 0);
-    long long room = chunk;
+    long long room = share;
     for (const auto& r : runs) {
         int t = r.t0;
         long long left = own ? (r.t1 - r.t0 + own - 1) / own : 0;      // bins this run still gets
         while (t < r.t1) {
             if (own) { room = (r.t1 - t + left - 1) / left; --left; }
-            int take = static_cast<int>(std::min<long long>(room, r.t1 - t));
+            if (room <= end && end > 0) { m.cta_begin.push_back(static_cast<int32_t>(m.items.size())); room = share; }
+            int take = static_cast<int>(std::min<long long>(room - end, r.t1 - t));
             if (align_nodes && r.seg == SEG_CTX)
                 while (t + take < r.t1 && !(m.tiles[t + take - 1].flags & TILE_CTX_END)) ++take;
             DevItem it;
@@ -284,8 +311,8 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int 
                 else { if (g.oth_n == 0) g.oth_slot0 = it.slot + s; g.oth_n++; }
             }
             m.items.push_back(it);
-            t += take; room -= take;
-            if (room <= 0) { m.cta_begin.push_back(static_cast<int32_t>(m.items.size())); room = chunk; }
+            t += take; room -= take + end;
+            if (room <= 0 && end == 0) { m.cta_begin.push_back(static_cast<int32_t>(m.items.size())); room = chunk; }
         }
     }
     while (static_cast<int>(m.cta_begin.size()) < n_bins + 1) m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
@@ -1767,7 +1794,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
                 for (const auto& cr : ctx_ranges) runs.push_back(Run{r, hh, 0, 1, SEG_CTX, cr.t0, cr.t1, mi});
             }
         }
-        assign_stream(runs, n_cta, 1, kDecodeItemTiles, m);
+        assign_stream(runs, n_cta, 1, kDecodeItemTiles, m, false, false);      // (the fixed scratch takes what it always took)
         finish_items(m);
         max_partials = most_partials(m);
         auto rnd = [](size_t x) { return (x + 255) & ~size_t(255); };

@@ -625,13 +625,13 @@ cudaError_t launch_merge_vec(const MergeParams& p, long long rows, cudaStream_t 
     // 60.5 with eight; 16 requests over shared 128K tokens: 129.0 and 124.4).  With more rows the warps of other rows hide it,
     // and sharing a row only adds the meeting in shared memory (64 rows over 10 x 256 tokens, 2048 rows to merge: 19.4 us with
     // one, 24.4 with eight; 4 x 128 rows over 20K tokens: 212 and 254).
-    // Of those with more rows, the ones with few partials a segment (most prefills: the runs of a head span few blocks) take eight lanes to a
-    // row: 4 x 128 rows over 20 documents each, five partials, 203 us per call with a warp per row, 198 this way; 2 x 256 rows over 20 x 256
-    // tokens 69.3 and 64.1.  (Few rows: 4 requests' decode step over 20 documents 55.9 with eight warps per row, 57.1-57.9 this way.)
-    const bool few = rows <= 4ll * p.n_sm;
-    if (!few && p.max_partials <= kRowPartials)
+    // With more rows than fit on the device at once that way (four blocks of eight to an SM) and few partials a segment (most prefills: the
+    // runs of a head span few blocks), eight lanes take a row.  64 rows over 30 x 256 tokens, 2 / 3 / 4 requests (4,096 / 6,144 / 8,192
+    // rows to merge): 28.9 / 42.6 / 52.6 us per call with a warp per row, 29.5 / 40.3 / 49.3 this way; 4 x 128 rows over 20 documents 203
+    // and 198; a tree's 3,072 rows 54.8 and 55.8.
+    if (rows > 32ll * p.n_sm && p.max_partials <= kRowPartials)
         return launch_pdl(ape_merge_rows_kernel<VEC * 4>, static_cast<unsigned>((rows + 15) / 16), 128, 0, stream, p);
-    if (few) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
+    if (rows <= 4ll * p.n_sm) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
     return launch_pdl(ape_merge_kernel<VEC, 1>, static_cast<unsigned>((rows + 7) / 8), 256, 0, stream, p);
 }
 }  // namespace

@@ -33,11 +33,12 @@ def test_partials_per_row(n_sm, mode, d, l_q):
         handle().set_sm_budget(0)
 
 
-@pytest.mark.parametrize("n_sm", [1, 7, 8, 9, 10, 16, 0])
-@pytest.mark.parametrize("d,G,l_q", [(64, 4, 151), (128, 1, 601), (64, 16, 41), (128, 4, 149)])
-def test_many_rows_with_few_and_with_more_partials(n_sm, d, G, l_q):
-    """More rows than the eight-warp form takes: up to eight partials a segment eight lanes share a row, with more a warp has it."""
-    b = wl.make_batch(H_q=G, H_kv=1, d=d, l_P=70, ctx_lens=[[2000]], l_q=l_q, l_k=l_q + 40, seed=34, T=0.8, S=0.9, name=f"merge_rows_sm{n_sm}")
+@pytest.mark.parametrize("n_sm", [3, 24, 60, 100, 146])
+@pytest.mark.parametrize("d,H_q,H_kv,n_req,l_q", [(64, 8, 8, 3, 3), (128, 32, 8, 3, 20), (128, 16, 4, 5, 9), (64, 32, 2, 10, 17)])
+def test_more_rows_than_warps(n_sm, d, H_q, H_kv, n_req, l_q):
+    """5,120 or 6,144 slot rows, more than there are places for a warp per row: eight lanes share a row, up to eight partials a segment."""
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=70, ctx_lens=[[900 - 100 * r] for r in range(n_req)] if n_req < 9 else [[500]] * n_req, l_q=l_q,
+                      l_k=l_q + 40, seed=34, T=0.8, S=0.9, name=f"merge_rows_sm{n_sm}")
     handle().set_sm_budget(n_sm)
     try:
         _check(b, libape.APE_PREFILL)
