@@ -826,15 +826,15 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             p->smem_bytes = attn_smem_bytes(D, kAttnPrefill);
             if (per_context == 0) {
                 // The cluster form: row blocks of 128 rows, whose two halves take alternate tiles, so that a block may have twice the tiles of
-                // the ordinary form's largest in about the same time, a little less for long ones (16 tiles against 31: 38.3 / 40.4 us).
-                // Ordinary / cluster, us per call: 4 x 64 tokens 8.2 / 6.9, 64 rows over 10 contexts of 256 16.5 / 14.4, 2 x 16 rows over
-                // 10 contexts 16.5 / 13.1, 4 x 5 rows over 24 contexts of 284 44.5 / 34.1, 128 rows over 10 contexts 17.6 / 17.6.
-                // A row's merge reads the partials of all blocks, three at a time, and with few row blocks the ordinary form has few rows to merge and
-                // leaves more of the chip to the tiles.  So clusters of more than six blocks only where the partials and the rows of a row block
-                // stay below a line that rises with the number of row blocks; else at most six blocks, all of one tile when there are fewer than
-                // four row blocks.  One KV head, one row block, ordinary / cluster: 128 rows, 10 tiles 9.9 / 11.0, 20 tiles 9.9 / 12.1, 16 rows, 10 tiles
-                // 9.1 / 8.3; eight heads of 40 rows, 20 tiles 14.8 / 11.1.  Of 329 calls with such clusters, 226 pass the line: six of
-                // them are more than 1.5% slower (one 7%), and 14 of the others would be more than 5% faster (none 10%).
+                // the ordinary form's largest in about the same time, a little less for long ones (16 tiles against 31: 38.3 / 32.0 us).
+                // Ordinary / cluster, us per call: 4 x 64 tokens 8.0 / 6.4, 64 rows over 10 contexts of 256 16.6 / 13.0, 2 x 16 rows over
+                // 10 contexts 16.5 / 11.7, 4 x 5 rows over 24 contexts of 284 38.3 / 32.1.
+                // With few row blocks the ordinary form has few rows to merge and leaves more of the chip to the tiles.  So clusters of more than
+                // six blocks only where the partials and the rows of a row block stay below a line that rises with the number of row blocks;
+                // else at most six blocks, all of one tile when there are fewer than four row blocks.  The line was drawn when the merge read the other
+                // blocks' rows; since they are sent it errs to the ordinary form: of 40 calls that it decides, 33 would be faster in clusters (one KV
+                // head, 3 x 2 rows over 33 contexts 15.8 / 11.6; 8 / 2 heads of 64, 3 x 24 rows over 38 contexts 15.3 / 10.7), one slower
+                // (10.1 / 10.6).  What it gives the cluster form is faster there: of 149 calls three were slower, by at most 3%.
                 const int TS = kAttnRows / 2 / G;
                 std::vector<Run> runs_s;
                 HostMeta ms;
