@@ -65,10 +65,10 @@ def decode_bytes(n_req: int, tokens_per_req: int) -> float:
 # cached tokens).  Valid only for the kernel sources the counters were taken with: the figure is dropped (null) as
 # soon as the hash of those sources changes.
 NCU_TRAFFIC = {
-    "prefill": {"bytes": 2 * (267.21e6 + 10.27e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "e537f8ccb34598b7"},
-    "encode": {"bytes": 2 * (791.07e6 + 484.68e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "e537f8ccb34598b7"},
-    "decode": {"bytes": (1.05517e9 + 3.91e6) * (8409907200.0 / 1053835264.0), "sources": ["ape_decode.cu", "ape_common.cuh", "ape_finish.cuh"], "sha": "d767962b3ebe39ad"},
-    "rope": {"bytes": 2 * ((131.29e6 + 84.12e6) + (131.31e6 + 77.99e6) + (524.91e6 + 475.75e6)), "sources": ["ape_rope.cu", "ape_common.cuh"], "sha": "88933f860f77de7c"},
+    "prefill": {"bytes": 2 * (266.90e6 + 10.46e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "40056cbcae4a4560"},
+    "encode": {"bytes": 2 * (790.78e6 + 484.33e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "40056cbcae4a4560"},
+    "decode": {"bytes": (1.05511e9 + 3.41e6) * (8409907200.0 / 1053835264.0), "sources": ["ape_decode.cu", "ape_common.cuh", "ape_finish.cuh"], "sha": "d858d51375fd8e0f"},
+    "rope": {"bytes": 2 * ((131.28e6 + 84.20e6) + (131.28e6 + 78.17e6) + (524.91e6 + 476.13e6)), "sources": ["ape_rope.cu", "ape_common.cuh"], "sha": "50dd0f0ff777a3a3"},
 }
 
 
