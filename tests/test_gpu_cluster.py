@@ -50,6 +50,23 @@ def test_decode(H_q, H_kv, d, n_req, ctx, l_P, l_k, gap):
             assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("H_q,H_kv", [(3, 3), (4, 2), (8, 2), (16, 2), (32, 2)])
+@pytest.mark.parametrize("lens", [[15, 17, 64], [128, 1, 79]])
+def test_decode_query_heads_per_kv_head(H_q, H_kv, d, lens):
+    """1, 2, 4, 8 query heads to a KV head are the columns of the products (8: all of them), 16 their rows; slices of 16 tokens that end
+    inside, at the edge and before; both forms of the step."""
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=33, ctx_lens=[lens, lens[:1]], l_q=1, l_k=5, capacity=70, gap=1, seed=51, T=0.8, S=0.7, name="heads")
+    for extra in (0, 11, 12, 65):
+        out, lse, n = gpu_attend(b, libape.APE_DECODE, kv_extra=extra)
+        assert n == 1
+        for got, got_lse in ((out, lse), _ordinary(b, libape.APE_DECODE, kv_extra=extra)):
+            for r in range(2):
+                ref = oracle_attend(b, r, l_k=5 + extra)
+                compare(got[r:r + 1], ref.out.float(), f"req {r} extra {extra}")
+                assert (got_lse[r:r + 1].double() - ref.lse).abs().max().item() < 2e-3
+
+
 @pytest.mark.parametrize("n_req,n_ctx,kernels", [(1, 10, 1), (1, 20, 2), (2, 10, 1), (2, 20, 2)])
 def test_decode_on_both_sides_of_the_line(n_req, n_ctx, kernels):
     """The largest block of a cluster may have three tiles more than the ordinary form's: 5 against 3 and 9 against 5 tiles for one request (148 SMs)."""
