@@ -13,9 +13,14 @@ namespace ape {
 namespace {
 
 constexpr int kTile = kDecodeTile;          // tokens per stage
-constexpr int kConsumerWarps = 8;           // two groups of four; group w/4 takes every other tile
+constexpr int kGroups = 2;                  // of four warps; warp w belongs to group w / 4, which takes every other tile
+constexpr int kConsumerWarps = 4 * kGroups;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
+// Tile n is group n % kGroups's and lies in stage n % depth, and the depth is a multiple of kGroups, so that a stage always belongs to the
+// same group.  A wait tells the phases of a barrier apart by their parity only: a group that saw every other use of a stage could take a
+// phase that has not ended for the one before it, and read a tile that is still landing.
 constexpr int kMaxStages = 8;
+static_assert(kMaxStages % kGroups == 0);
 constexpr int kRecvRows = 32;               // (G rows, at most 16, rounded up to a multiple of the cluster's size, at most 16)
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -367,7 +372,7 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
         }
     } else {
         // ---------------- consumers ----------------------------------------------------------------------------------
-        const int grp = warp >> 2;            // which half of the tiles
+        const int grp = warp >> 2;
         const int w4 = warp & 3;              // 16-token slice inside a tile
         const int G = p.G;
         uint32_t cnt = 0;
@@ -381,7 +386,7 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
             part.begin(p.q.data + static_cast<int64_t>(item.q_row0) * p.q.token_stride + static_cast<int64_t>(item.kv_head) * G * p.q.head_stride, p.q.head_stride, G);
 
             for (int t = item.tile_begin; t < t_end; ++t, ++cnt) {
-                if ((cnt & 1u) != static_cast<uint32_t>(grp)) continue;
+                if (cnt % kGroups != static_cast<uint32_t>(grp)) continue;
                 const int s = cnt % n_stages;
                 const uint32_t use = cnt / n_stages;
                 if (!mbar_wait(bar_full + 8 * s, use & 1, &abort_flag, p.status)) break;
@@ -486,7 +491,7 @@ size_t decode_smem_bytes(int D, int G, int n_stages, int cluster) {
 
 int decode_pick_stages(int D, int G, size_t smem_limit, int cluster) {
     int n = kMaxStages;
-    while (n > 2 && decode_smem_bytes(D, G, n, cluster) > smem_limit) --n;
+    while (n > kGroups && decode_smem_bytes(D, G, n, cluster) > smem_limit) n -= kGroups;
     return decode_smem_bytes(D, G, n, cluster) <= smem_limit ? n : 0;
 }
 
