@@ -1708,7 +1708,7 @@ constexpr size_t kNoAllocMetaBytes = 4u << 20;    // [0, 256): status word; then
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 struct NoAllocDevice {
-    bool ready = false;
+    bool ready = false, loaded = false;
     unsigned char* scratch = nullptr;             // DEVICE address of g_noalloc_scratch on this device
     ape_handle_s h;                               // host-side record only (no device allocation behind it)
 };
@@ -1740,6 +1740,15 @@ int noalloc_setup(int device, NoAllocDevice** out) {
         d.ready = true;
     }
     *out = &d;
+    return APE_OK;
+}
+
+// Once per device, in the first step: every kernel that any step may take, for all head sizes.  Loading one may allocate; no later call does.
+int noalloc_load(NoAllocDevice* d) {
+    std::lock_guard<std::mutex> lock(g_noalloc_mutex);
+    for (int D : {64, 128})
+        if (!d->loaded && (decode_set_smem_attr(D, d->h.smem_optin - kDecodeStaticSmem) != cudaSuccess || merge_load(D) != cudaSuccess)) return APE_ERR_CUDA;
+    d->loaded = true;
     return APE_OK;
 }
 
@@ -1795,6 +1804,7 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
         if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) return APE_ERR_CUDA;
         if (cap != cudaStreamCaptureStatusNone) return APE_ERR_MODE;
     }
+    rc = noalloc_load(dv);                            if (rc) return rc;
     const int D = shape->head_dim, H_kv = shape->n_kv_heads, tile = kDecodeTile;
     const int n_cta = dv->h.n_sm;
 

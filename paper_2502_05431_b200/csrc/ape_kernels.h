@@ -131,6 +131,9 @@ struct MergeParams : RowsOut {
     int32_t max_partials;            // of a segment of a row
 };
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
+// Loads the kernels of the Eq. 5 form for this head size.  (The runtime loads a kernel, and may allocate memory for its code, when it is
+// first asked for.)
+cudaError_t merge_load(int D);
 
 // Between the two passes of a plan with separately scaled context nodes (per-context form: every context a marked
 // top-level node; context trees): from the (maximum, sum) of every node's own tokens to the bias of its tokens' logits.

@@ -660,4 +660,15 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream)
     return p.D == 128 ? launch_merge_vec<4>(p, rows, stream) : launch_merge_vec<2>(p, rows, stream);
 }
 
+template <int VEC>
+static cudaError_t merge_load_vec() {
+    cudaFuncAttributes attr;
+    for (auto* kernel : {ape_merge_kernel<VEC, 8>, ape_merge_kernel<VEC, 1>, ape_merge_rows_kernel<VEC * 4>}) {
+        const cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+cudaError_t merge_load(int D) { return D == 128 ? merge_load_vec<4>() : merge_load_vec<2>(); }
+
 }  // namespace ape

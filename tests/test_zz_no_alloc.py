@@ -3,6 +3,10 @@ server whose own pool owns the whole GPU, a latency-critical loop, a sandboxed p
 a fixed device array inside the library, shared by all calls, so the test runs it twice in a row on different inputs
 and compares each result with the plan-based entry point (ape_attend_plan + ape_attend), which uses caller-provided
 scratch.  This file is collected last on purpose."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -62,6 +66,15 @@ def test_noalloc_decode_matches_planned_decode_twice_in_a_row():
         o_ref, o_new, l_ref, l_new = _both(b, kv_extra=extra)
         _close(o_ref, o_new)
         assert (l_ref - l_new).abs().max().item() < 2e-3
+
+
+def test_noalloc_allocates_nothing_in_a_process_that_has_loaded_little():
+    """A kernel is loaded, which may allocate, when it is first asked for, so the set-up asks for all that any later step may take.  The test
+    above in a process of its own, where no other test has loaded them."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-m", "pytest", "-q", "-m", "gpu", "-p", "no:cacheprovider",
+                        f"{__file__}::test_noalloc_decode_matches_planned_decode_twice_in_a_row"], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "1 passed" in r.stdout, r.stdout[-2000:]
 
 
 def test_noalloc_decode_asynchronous_form_and_limits():
