@@ -126,16 +126,29 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// The same for a barrier that other blocks of the cluster complete: what they have written is visible behind it.  (The wait above acquires
+// at the scope of the block.)
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 
 // Every wait in the library is bounded: after about a second (2^31 SM cycles) the waiter raises the CTA's
 // abort flag and the device status word, and every role of the CTA leaves its loop.  Returns false on abort.
 constexpr long long kWaitCycles = 1ll << 31;
 
+template <bool CLUSTER = false>           // CLUSTER: mbar_try_wait_cluster
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto done = [&] { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (done()) return true;
     long long t0 = 0;
     for (uint32_t spin = 1;; ++spin) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (done()) return true;
         if ((spin & 63u) == 0u) {
             if (*abort_flag) return false;
             const long long now = clock64();
