@@ -869,8 +869,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
             __syncwarp();
             // (all lanes wait: each reads what has arrived)
-            const bool here = __all_sync(0xffffffffu, mbar_wait<true>(bar_recv, 0, &abort_flag, p.status)) != 0;
-            cluster_arrive_relaxed();                               // no block leaves while a copy of its rows is under way
+            const bool here = __all_sync(0xffffffffu, mbar_wait_received(bar_recv, &abort_flag, p.status)) != 0;
+            cluster_arrive_relaxed();                               // no block leaves while a copy of its rows or to its memory is under way
             // eight lanes to a row, so that a block's rows (cluster of 6: 22) are merged side by side
             for (int i = warp * 4 + (lane >> 3); here && (i & ~3) < mine; i += 32) {
                 if (i >= mine) continue;

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ape_wait.h"
+
 namespace ape {
 
 // ---- plan metadata (host-built, device-resident) ---------------------------------------------------------------
@@ -138,17 +140,12 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
     return ok != 0;
 }
 
-// Every wait in the library is bounded: after about a second (2^31 SM cycles) the waiter raises the CTA's
-// abort flag and the device status word, and every role of the CTA leaves its loop.  Returns false on abort.
-constexpr long long kWaitCycles = 1ll << 31;
-
-template <bool CLUSTER = false>           // CLUSTER: mbar_try_wait_cluster
+// A bounded wait (ape_wait.h).  Returns false on abort.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-    auto done = [&] { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
-    if (done()) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     long long t0 = 0;
     for (uint32_t spin = 1;; ++spin) {
-        if (done()) return true;
+        if (mbar_try_wait(bar, parity)) return true;
         if ((spin & 63u) == 0u) {
             if (*abort_flag) return false;
             const long long now = clock64();
@@ -160,6 +157,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             }
         }
     }
+}
+
+// The wait for what other blocks of the cluster send to this one (first phase of `bar`).
+__device__ __forceinline__ bool mbar_wait_received(uint32_t bar, volatile int* abort_flag, int* status) {
+    return wait_received([&] { return mbar_try_wait_cluster(bar, 0); }, [] { return clock64(); },
+                         [&] { *abort_flag = 1; atomicExch(status, kStatusTimeout); });
 }
 
 __device__ __forceinline__ void fence_proxy_async_smem() {

@@ -89,8 +89,8 @@ __device__ __forceinline__ void cluster_st2(uint32_t addr, float a, float b) {
 __device__ __forceinline__ void cluster_st4(uint32_t addr, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-// Stores and copies to another block's shared memory, counted in bytes on a barrier there: who waits on it sees them, no barrier of the
-// whole cluster is needed.  addr / dst and bar: addresses of the same block (cluster_map).
+// Stores and copies to another block's shared memory, counted in bytes on a barrier there: who waits on it (mbar_wait_received) sees them, no barrier
+// of the whole cluster is needed.  addr / dst and bar: addresses of the same block (cluster_map).
 __device__ __forceinline__ void cluster_send2(uint32_t addr, float a, float b, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
