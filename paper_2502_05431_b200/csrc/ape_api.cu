@@ -401,7 +401,8 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
                 (seg == SEG_CTX ? g.ctx_n : g.oth_n) += blocks;
                 used += blocks;
             }
-        for (; used < cs.size; ++used) {                   // every block has a record, so that block b reads the b-th one without a range in front
+        // every block has a record: block b reads the b-th one without a range in front, and the request's rows from it
+        for (; used < cs.size; ++used) {
             DevItem none{};
             none.req = runs[i].req; none.kv_head = runs[i].kv_head; none.row_block = runs[i].row_block;
             m.items.push_back(none);
@@ -480,7 +481,6 @@ void finish_items(HostMeta& m) {
         if (it.tile_begin < static_cast<int32_t>(m.tiles.size())) it.first_tile = m.tiles[it.tile_begin];
         else it.first_tile = DevTile{0, 0, 0, 0};
     }
-    for (auto& g : m.merge) g.q_row0 = m.reqs[g.req].q_row0;
 }
 
 int most_partials(const HostMeta& m) {       // of a segment of a row

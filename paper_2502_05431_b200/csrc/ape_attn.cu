@@ -811,7 +811,9 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             float2* ml = reinterpret_cast<float2*>(q_smem);         // [2][128]
             const int C = p.cluster, rank = static_cast<int>(cluster_ctarank()), r = r_local;
             const DevMerge merge = p.groups[blockIdx.x / static_cast<unsigned>(C)];
-            const int n_rows = min(kHalfRows, (p.items[item_begin].q_len - merge.row_block * TB) * G);      // live rows of the row block
+            const DevItem& item = p.items[item_begin];
+            const int q_row0 = item.q_row0 + merge.row_block * TB;
+            const int n_rows = min(kHalfRows, (item.q_len - merge.row_block * TB) * G);      // live rows of the row block
             const int n = merge.ctx_n + merge.oth_n;                // blocks 0 .. n - 1 have a partial
             const int share = (n_rows + C - 1) / C, first = rank * share, mine = min(max(n_rows - first, 0), share);
             const int owner = r / share;                            // of row r
@@ -886,7 +888,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         x[v] = t.x; x[v + 1] = t.y; x[v + 2] = t.z; x[v + 3] = t.w;
                     }
                 }, Ms, Ls, acc);
-                finish_row<VEC, 8>(p.fin, merge.q_row0 + merge.row_block * TB + rr / G, merge.kv_head * G + rr % G, lane & 7, Ms, Ls, acc);
+                finish_row<VEC, 8>(p.fin, q_row0 + rr / G, merge.kv_head * G + rr % G, lane & 7, Ms, Ls, acc);
             }
             __syncwarp();
             cluster_wait();

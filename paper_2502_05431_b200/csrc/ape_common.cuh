@@ -70,7 +70,6 @@ struct DevMerge {
     int32_t ctx_row_off; // added to the row when a context partial is read: shared-context plans keep the context
                          // partials of many requests in one slot, one group of rows per request
     int32_t ctx_stride;  // between consecutive context partials
-    int32_t q_row0;      // first row of Q / O of the request
 };
 
 // One node of a context tree (tree plans): a SEG_CTX item's ctx_id is the index of the node its tiles belong to.

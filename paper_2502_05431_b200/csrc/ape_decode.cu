@@ -477,7 +477,7 @@ ape_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constan
             const int at = turn * C;
             float M[2], L[2], acc[2][VEC];
             merge_received<VEC>(&recv_ml[at], recv + at * RS + lane * VEC, RS, group.ctx_n, group.oth_n, M, L, acc);
-            finish_row<VEC>(p.fin, group.q_row0, group.kv_head * p.G + row, lane, M, L, acc);
+            finish_row<VEC>(p.fin, first.q_row0, group.kv_head * p.G + row, lane, M, L, acc);
         }
     }
 }

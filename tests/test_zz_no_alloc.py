@@ -12,7 +12,7 @@ import torch
 
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
-from tests.gpu_util import MAX_ABS, MEAN_ABS, handle
+from tests.gpu_util import MAX_ABS, MEAN_ABS, compare, handle, oracle_attend
 
 pytestmark = pytest.mark.gpu
 LLAMA = dict(H_q=32, H_kv=8, d=128)
@@ -159,6 +159,48 @@ def test_noalloc_size_gate_counts_fused_spans():
     assert libape.decode_noalloc(out=out_a, requests=[many], want_status=True, **kw) == 0
     assert libape.decode_noalloc(out=out_b, requests=b.requests, want_status=True, **kw) == 0
     assert torch.equal(out_a, out_b) and not torch.isnan(out_a.float()).any()
+
+
+def test_noalloc_accepts_a_batch_whose_records_just_fit():
+    """The tile lists, items, requests and merge records of a step share 4 MiB of the fixed array (behind 256 bytes for the status word; each list
+    rounded up to 256).  A batch that fills them to the last 256 bytes is taken, one of sixteen tiles more is refused.  64 requests of 8 KV
+    heads, so that four bytes more for a merge record would refuse the first, too."""
+    n_req, H_kv, n_cta, limit = 64, 8, torch.cuda.get_device_properties(0).multi_processor_count, 4 << 20
+    rnd = lambda x: (x + 255) // 256 * 256  # noqa: E731
+
+    def records(n_ctx):                                     # bytes, for n_ctx[r] contexts of one token in request r
+        runs = [t for n in n_ctx for _ in range(H_kv) for t in (2, n)]            # prefix and query segment: a tile each
+        chunk, room, items = -(-sum(runs) // n_cta), 0, 0
+        for t in runs:
+            while t > 0:
+                room = room or chunk
+                take = min(t, room)
+                t, room, items = t - take, room - take, items + 1
+        return 256 + rnd(16 * (sum(n_ctx) + 2 * n_req)) + rnd(64 * items) + rnd(4 * (n_cta + 1)) + rnd(16 * n_req) + rnd(40 * n_req * H_kv)
+
+    n_ctx = [3000] * n_req
+    while records(n_ctx) < limit:                           # the last tiles of the last requests, sixteen at a time
+        more = max(16, (limit - records(n_ctx)) // 32 // 16 * 16)
+        n_ctx[n_ctx.index(min(n_ctx))] += min(more, 1000)
+    while records(n_ctx) > limit:
+        n_ctx[-1] -= 16
+    assert limit - 1024 < records(n_ctx) <= limit
+    b = wl.make_batch(H_q=H_kv, H_kv=H_kv, d=64, l_P=8, ctx_lens=[[1] * max(n_ctx)] + [[]] * (n_req - 1), l_q=1, l_k=4, gap=1, seed=28, T=0.9, S=0.9)
+    spans = b.requests[0].ctx
+    for r, n in zip(b.requests, n_ctx):
+        r.ctx = spans[:n]
+    g = b.to("cuda:0")
+    out = torch.full_like(g.q, float("nan"))
+    kw = dict(H_q=H_kv, H_kv=H_kv, d=64, k_pool=g.k_pool, v_pool=g.v_pool, q=g.q, out=out, requests=b.requests, T=b.T, S=b.S)
+    assert libape.decode_noalloc(want_status=True, **kw) == 0
+    for r in (0, n_req - 1):
+        ref = oracle_attend(b, r)
+        compare(out[r:r + 1].cpu(), ref.out.float(), f"req {r}")
+    n_ctx[-1] += 1024 // 16
+    b.requests[-1].ctx = (spans + spans)[:n_ctx[-1]]
+    with pytest.raises(libape.ApeError) as e:
+        libape.decode_noalloc(want_status=True, **kw)
+    assert e.value.code == -6
 
 
 def test_noalloc_calls_of_different_batches_back_to_back():
