@@ -343,7 +343,7 @@ void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int 
     while (static_cast<int>(m.cta_begin.size()) < n_bins + 1) m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
 }
 
-// Tiles of the bin with the most (what its items' ends cost is not counted: the figures at pick_cluster were measured with this number).
+// Tiles of the bin with the most (what its items' ends cost is not counted).
 long long largest_bin(const HostMeta& m) {
     long long most = 0;
     for (size_t b = 0; b + 1 < m.cta_begin.size(); ++b) {
@@ -416,9 +416,13 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
 // the smallest; and that block may have kClusterTiles tiles more than the largest of the ordinary form, whose merge kernel costs about
 // as much.  Never under an SM budget: the budget leaves SMs to a kernel that runs beside, which takes some of every part, and a
 // cluster waits until it finds as many free SMs in one part as it has blocks; single blocks take the SMs that are left.
-// In us per call, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
-//   1 request   1 x 64 tokens 5.1 / 3.7 (2 / 1)   10 contexts 5.9 / 5.7 (3 / 5)   20: 7.5 / 7.5 (5 / 9: stays ordinary)   40: 9.3 / 11.3 (10 / 18)
-//   2 requests  4 contexts 6.3 / 5.1 (3 / 4)   10: 7.5 / 7.0 (5 / 8)   20: 9.6 / 10.4 (10 / 15)      4 requests  4 contexts 7.4 / 6.2
+// In us per call in a graph of calls, 32 / 8 heads, contexts of 256 tokens, ordinary / cluster (tiles of the largest):
+//   1 request   1 x 64 tokens 4.7 / 3.6 (2 / 1)   10 contexts 6.0 / 5.4 (3 / 5)   20: 7.4 / 7.0 (5 / 9: stays ordinary)   40: 8.8 / 10.5 (10 / 18)
+//   2 requests  4 contexts 5.8 / 4.9 (3 / 4)   10: 6.9 / 6.5 (5 / 8)   20: 8.6 / 9.6 (10 / 15)      4 requests  4 contexts 6.8 / 5.7
+// and on inputs that change from call to call, as a program has them, 10 contexts 6.5 / 5.9, 20: 7.6 / 8.0; 2 requests 10: 7.4 / 7.2, 20: 11.6 / 12.4.
+// The ordinary form's largest block is that of a split in which items' ends count (assign_stream), and may have a tile more than equal shares
+// would leave it.  Of 40 decode steps that this tile decides, 32 are faster in clusters (by up to 19%, all 40 together by 7%), two more than 3%
+// slower (11 requests of 4 heads over 1,782 tokens 8.6 / 10.3, 45 of 16 / 1 heads over 1,974 tokens 13.4 / 14.6).
 constexpr int kClusterTiles = 3, kOnePassNodes = 6, kPlainTiles = 13, kPlainTiles64 = 17, kFewBlocks = 6;
 ClusterSplit pick_cluster(const ape_handle_s* h, const std::vector<Run>& runs, int n_groups, const int (&resident)[kClusterSizes], long long limit, int max_size = kCluster[0]) {
     ClusterSplit best;
