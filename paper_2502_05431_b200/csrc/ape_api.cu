@@ -21,10 +21,6 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Cluster sizes that a plan may choose, largest first (above 8 not every device's limit allows them; the device is asked).
-constexpr int kClusterSizes = 9;
-constexpr int kCluster[kClusterSizes] = {16, 10, 9, 8, 6, 5, 4, 3, 2};
-
 }  // namespace
 
 struct ape_handle_s {

@@ -38,8 +38,14 @@ constexpr int kMmaWarp = 9;
 constexpr int kBarBytes = 512;                // barriers, behind the tiles
 constexpr int kStageBytes = 8 * 4096;         // transposition buffers of the softmax warps, behind the barriers
 // Clusters, behind the barriers: a share is 1 / size of at most 128 rows, rounded up; (m, l) of a share from every block and its rows from
-// all but one (sizes 2 ... 10 and 16: at most 135 and 120; a block without a partial of its own has one more sender, but then one is idle)
+// all but one (a block without a partial of its own has one more sender, but then one is idle).  Sizes of 9 and 16 fill the rows to the last.
 constexpr int kRecvMl = 136, kRecvRows = 120;
+constexpr bool shares_fit() {
+    for (int c : kCluster)
+        if (const int share = (kHalfRows + c - 1) / c; share * c > kRecvMl || share * (c - 1) > kRecvRows) return false;
+    return true;
+}
+static_assert(shares_fit(), "a block's share of the rows does not fit");
 constexpr int kSlabBytes = 128 * 128;         // 128 rows x 64 bf16
 constexpr float kRescaleThreshold = 8.0f;     // base-2 units: O is rescaled only when the row maximum grew by more
 

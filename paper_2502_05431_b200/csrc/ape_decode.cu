@@ -21,7 +21,14 @@ constexpr int kThreads = (kConsumerWarps + 1) * 32;
 // phase that has not ended for the one before it, and read a tile that is still landing.
 constexpr int kMaxStages = 8;
 static_assert(kMaxStages % kGroups == 0);
-constexpr int kRecvRows = 32;               // (G rows, at most 16, rounded up to a multiple of the cluster's size, at most 16)
+constexpr int kRecvRows = 32;               // (m, l) of a block's share of the rows, from every block: G, at most 16, rounded up to a multiple of the size
+constexpr bool shares_fit() {
+    for (int c : kCluster)
+        for (int G = 1; G <= 16; ++G)
+            if ((G + c - 1) / c * c > kRecvRows) return false;
+    return true;
+}
+static_assert(shares_fit(), "a block's share of the rows does not fit");
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"

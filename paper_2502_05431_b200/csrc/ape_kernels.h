@@ -7,6 +7,10 @@ namespace ape {
 
 constexpr int kDecodeTile = 64;     // tokens per pipeline stage of the decode kernel
 constexpr int kAttnTileN = 128;     // keys per tile of the tensor-core (prefill / encode) kernel
+// Cluster sizes that a plan may choose, largest first (above 8 not every device's limit allows them; the device is asked).  What the kernels keep
+// for rows from other blocks is checked against them.
+constexpr int kClusterSizes = 9;
+constexpr int kCluster[kClusterSizes] = {16, 10, 9, 8, 6, 5, 4, 3, 2};
 constexpr int kAttnRows = 256;      // packed (token, head-in-group) rows per row block of that kernel (two 128-row halves)
 
 // Where the finished rows of an attend call go, and the scaling factor of Eq. 5.

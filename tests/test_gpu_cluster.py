@@ -6,7 +6,7 @@ import torch
 
 from paper_2502_05431_b200 import libape
 from paper_2502_05431_b200 import workloads as wl
-from tests.gpu_util import compare, gpu_attend, handle, oracle_attend
+from tests.gpu_util import compare, gpu_attend, handle, kernels_in_order, oracle_attend
 
 pytestmark = pytest.mark.gpu
 
@@ -130,21 +130,55 @@ def test_prefill(H_q, H_kv, d, n_req, ctx, l_P, l_q, l_k, gap):
         assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
+# (query heads, contexts, rows) that the line between the forms sends to the ordinary one on 148 SMs
+_ORDINARY_SHARES = {(4, 3, 32), (4, 5, 13), (4, 5, 32), (4, 9, 32), (4, 12, 1), (4, 12, 3), (4, 12, 13), (4, 12, 32), (16, 5, 13), (16, 9, 13),
+                    (16, 12, 3), (16, 12, 13), (16, 12, 32)}
+
+
 @pytest.mark.parametrize("H_q,H_kv,d", [(4, 1, 128), (16, 2, 64), (8, 8, 128)])
 @pytest.mark.parametrize("n_ctx", [0, 1, 2, 3, 5, 9, 12])
 @pytest.mark.parametrize("l_q", [1, 3, 13, 32])
 def test_prefill_shares_of_rows(H_q, H_kv, d, n_ctx, l_q):
     """Every block of a cluster merges a share of the rows: rows that do not divide by the blocks, fewer rows than blocks, blocks without a
-    partial, clusters of different sizes.  Against the ordinary form (the same products and sums in another order, rounded to bf16, 2^-9 of
-    the value, on both sides) where the plan takes clusters."""
+    partial, clusters of two to sixteen.  Against the ordinary form (the same products and sums in another order, rounded to bf16, 2^-9 of
+    the value, on both sides) and the oracle; 13 of the 84 calls take the ordinary form themselves."""
     b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=20, ctx_lens=[[130] * n_ctx], l_q=l_q, gap=1, seed=47, T=0.8, S=0.7, name="shares")
     out, lse, n = gpu_attend(b, libape.APE_PREFILL)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert n == (2 if (H_q, n_ctx, l_q) in _ORDINARY_SHARES else 1)
     ref_o, ref_lse = _ordinary(b, libape.APE_PREFILL)
     assert (out.float() - ref_o.float()).abs().max() <= 2 ** -7 * max(1.0, ref_o.float().abs().max().item())
     assert (lse - ref_lse).abs().max() < 1e-4
     ref = oracle_attend(b, 0)
     compare(out, ref.out.float(), "shares")
     assert (lse.double() - ref.lse).abs().max().item() < 2e-3
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("H_q,H_kv,l_q,lens,size", [
+    (16, 4, 32, [[130] * 4, [130] * 4], 10),               # 128 rows, ten blocks of a tile: shares of 13 rows, the last of 11
+    (16, 4, 32, [[130, 130, 130, 60], [130]], 9),          # nine blocks: shares of 15, rows from eight others fill what there is; four blocks, five idle
+    (16, 4, 32, [[130] * 3, []], 8),                       # eight blocks, and two and six idle ones
+    (32, 8, 32, [[130] * 4], 10), (28, 7, 20, [[130] * 7], 16)])       # (sixteen: 80 rows at most)
+def test_prefill_full_row_blocks_in_large_clusters(H_q, H_kv, l_q, lens, size, d):
+    """As many rows as a row block has in the clusters whose shares of them fill the space for rows from other blocks."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the split is that of 148 SMs")
+    b = wl.make_batch(H_q=H_q, H_kv=H_kv, d=d, l_P=20, ctx_lens=lens, l_q=l_q, gap=1, seed=47, T=0.8, S=0.7, name="full")
+    dev = b.to("cuda:0")
+    plan = handle().attend_plan(H_q=H_q, H_kv=H_kv, d=d, k_pool=dev.k_pool, v_pool=dev.v_pool, q=dev.q, out=torch.zeros_like(dev.q),
+                                requests=b.requests, mode=libape.APE_PREFILL)
+    ws = plan.alloc_workspace()
+    assert kernels_in_order(lambda: plan.attend(b.T, b.S, ws), grids=True) == [("attn", size * H_kv * len(lens))]
+    out, lse, _ = gpu_attend(b, libape.APE_PREFILL)
+    ref_o, ref_lse = _ordinary(b, libape.APE_PREFILL)
+    assert (out.float() - ref_o.float()).abs().max() <= 2 ** -7 * max(1.0, ref_o.float().abs().max().item())
+    assert (lse - ref_lse).abs().max() < 1e-4
+    for r, rq in enumerate(b.requests):
+        ref = oracle_attend(b, r)
+        sl = slice(rq.q_start, rq.q_start + rq.q_len)
+        compare(out[sl], ref.out.float(), f"req {r}")
+        assert (lse[sl].double() - ref.lse).abs().max().item() < 2e-3
 
 
 @pytest.mark.parametrize("d", [64, 128])
