@@ -376,7 +376,7 @@ long long cluster_partials(const std::vector<Run>& runs, const ClusterSplit& cs)
     return most;
 }
 void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostMeta& m) {
-    m.cta_begin.assign(1, 0);
+    m.cta_begin.clear();                                   // block b's item is the b-th one
     for (size_t i = 0, j; i < runs.size(); i = j) {
         for (j = i; j < runs.size() && runs[j].merge0 == runs[i].merge0;) ++j;
         DevMerge& g = m.merge[runs[i].merge0];
@@ -392,7 +392,6 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
                     it.req = r.req; it.kv_head = r.kv_head; it.row_block = r.row_block; it.seg = r.seg; it.n_sib = r.n_sib; it.ctx_id = r.ctx_id;
                     it.tile_begin = r.t0 + static_cast<int>(n * b / blocks); it.tile_end = r.t0 + static_cast<int>(n * (b + 1) / blocks);
                     m.items.push_back(it);
-                    m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
                 }
                 (seg == SEG_CTX ? g.ctx_n : g.oth_n) += blocks;
                 used += blocks;
@@ -402,7 +401,6 @@ void assign_clusters(const std::vector<Run>& runs, const ClusterSplit& cs, HostM
             DevItem none{};
             none.req = runs[i].req; none.kv_head = runs[i].kv_head; none.row_block = runs[i].row_block;
             m.items.push_back(none);
-            m.cta_begin.push_back(static_cast<int32_t>(m.items.size()));
         }
     }
 }
@@ -1383,7 +1381,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         float* b_ml = reinterpret_cast<float*>(base + a->ws_bytes + rnd(rows_b * D * 4));
         p->last_launches = 0;
         DecodeParams dp{};
-        dp.tiles = b->d_tiles; dp.items = b->d_items; dp.cta_item_begin = b->d_cta_begin; dp.reqs = b->d_reqs;
+        dp.tiles = b->d_tiles; dp.items = b->d_items; dp.cta_item_begin = b->d_cta_begin;
         dp.q = rows_desc(p->q); dp.ws_o = b_o; dp.ws_ml = b_ml;
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = b->n_stages; dp.status = p->h->d_status;
@@ -1396,10 +1394,10 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         if (p->rest_first && !launch_rest()) return APE_ERR_CUDA;
         if (a->n_items > 0) {
             AttnParams ap{};
-            ap.tiles = a->d_tiles; ap.items = a->d_items; ap.cta_item_begin = a->d_cta_begin; ap.reqs = a->d_reqs;
+            ap.tiles = a->d_tiles; ap.items = a->d_items; ap.cta_item_begin = a->d_cta_begin;
             ap.out = rows_desc(p->out); ap.lse_out = nullptr; ap.ws_o = a_o; ap.ws_ml = a_ml;
             ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
-            ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = a->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
+            ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = a->n_sib; ap.mode = kAttnPrefill; ap.status = p->h->d_status;
             ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1; if (a->alt_halves) ap.mode = kAttnAlt;
             ap.wait_late = (p->rest_first && a->early) ? 1 : 0;    // beside the kernel in front of it, where it is placed early at all
             if (launch_attn(D, a->tm_q, a->tm_k, a->tm_v, a->tm_q, a->tm_split, ap, a->n_cta, a->smem_bytes, a->early, stream) != cudaSuccess) return APE_ERR_CUDA;
@@ -1423,7 +1421,7 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
 
     if (p->kind == PLAN_DECODE) {
         DecodeParams dp{};
-        dp.tiles = p->d_tiles; dp.items = p->d_items; dp.cta_item_begin = p->d_cta_begin; dp.reqs = p->d_reqs;
+        dp.tiles = p->d_tiles; dp.items = p->d_items; dp.cta_item_begin = p->d_cta_begin;
         dp.q = rows_desc(p->q); dp.ws_o = ws_o; dp.ws_ml = ws_ml;
         dp.scale_oth_log2 = p->c * kLog2e; dp.scale_ctx_log2 = p->c / T * kLog2e;
         dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = p->n_stages; dp.status = p->h->d_status;
@@ -1437,10 +1435,10 @@ static int attend_impl(ape_plan_t p, float T, float S, int64_t kv_extra, void* w
         if (launch_decode(D, p->tm_k, p->tm_v, dp, p->n_cta, p->smem_bytes, true, stream) != cudaSuccess) return APE_ERR_CUDA;
     } else {
         AttnParams ap{};
-        ap.tiles = p->d_tiles; ap.items = p->d_items; ap.cta_item_begin = p->d_cta_begin; ap.reqs = p->d_reqs;
+        ap.tiles = p->d_tiles; ap.items = p->d_items; ap.cta_item_begin = p->d_cta_begin;
         ap.out = rows_desc(p->out); ap.lse_out = nullptr; ap.ws_o = ws_o; ap.ws_ml = ws_ml;
         ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c / T * kLog2e;
-        ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = p->n_sib; ap.mode = kAttnPrefill; ap.q_rows_are_pool = 0; ap.status = p->h->d_status;
+        ap.G = G; ap.H_q = p->shape.n_q_heads; ap.n_sib = p->n_sib; ap.mode = kAttnPrefill; ap.status = p->h->d_status;
         ap.o_via_tma = 0; ap.split_r = 0; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1;
         if (p->two_pass) {
             // per-context form / context trees: (1) every node's own (maximum, sum) per row, (2) per-row, per-node biases
@@ -1531,10 +1529,10 @@ int ape_encode_contexts(ape_plan_t p, void* workspace, size_t ws_bytes, void* st
     if (p->n_items == 0) return APE_OK;
     constexpr float kLog2e = 1.4426950408889634f;
     AttnParams ap{};
-    ap.tiles = p->d_tiles; ap.items = p->d_items; ap.cta_item_begin = p->d_cta_begin; ap.reqs = p->d_reqs;
+    ap.tiles = p->d_tiles; ap.items = p->d_items; ap.cta_item_begin = p->d_cta_begin;
     ap.out = rows_desc(p->out); ap.lse_out = p->lse; ap.ws_o = nullptr; ap.ws_ml = nullptr;
     ap.scale_oth_log2 = p->c * kLog2e; ap.scale_ctx_log2 = p->c * kLog2e;
-    ap.G = p->G; ap.H_q = p->shape.n_q_heads; ap.n_sib = 1; ap.mode = kAttnEncode; ap.q_rows_are_pool = 1; ap.status = p->h->d_status;
+    ap.G = p->G; ap.H_q = p->shape.n_q_heads; ap.n_sib = 1; ap.mode = kAttnEncode; ap.status = p->h->d_status;
     ap.o_via_tma = p->o_via_tma ? 1 : 0; ap.split_r = p->split_r; ap.stats = nullptr; ap.bias = nullptr; ap.stat_rows = 0; ap.let_next_in = p->budget ? 0 : 1;
     if (launch_attn(p->shape.head_dim, p->tm_q, p->tm_k, p->tm_v, p->tm_o, p->tm_split, ap, p->n_cta, p->smem_bytes, p->early,
                     static_cast<cudaStream_t>(stream_v)) != cudaSuccess) return APE_ERR_CUDA;
@@ -1877,14 +1875,14 @@ int ape_decode_noalloc(const ape_shape_t* shape, const ape_kv_pool_t* pool, cons
     float* ws_ml = reinterpret_cast<float*>(base + kNoAllocMetaBytes + ((rows * D * 4 + 255) & ~size_t(255)));
     DecodeParams dp{};
     dp.tiles = reinterpret_cast<const DevTile*>(base + o_tiles); dp.items = reinterpret_cast<const DevItem*>(base + o_items);
-    dp.cta_item_begin = reinterpret_cast<const int32_t*>(base + o_cta); dp.reqs = reinterpret_cast<const DevReq*>(base + o_reqs);
+    dp.cta_item_begin = reinterpret_cast<const int32_t*>(base + o_cta);
     dp.q = rows_desc(*q); dp.ws_o = ws_o; dp.ws_ml = ws_ml;
     dp.scale_oth_log2 = c * kLog2e; dp.scale_ctx_log2 = c / T * kLog2e;
     dp.kv_extra = static_cast<int32_t>(kv_extra); dp.G = G; dp.n_stages = n_stages; dp.status = reinterpret_cast<int*>(base); dp.let_next_in = 1;
     // Not early: the records that the kernel reads in front of its dependency wait are those of the copy above, on this stream.
     if (launch_decode(D, tm_k, tm_v, dp, n_cta, smem_bytes, false, stream) != cudaSuccess) return APE_ERR_CUDA;
     MergeParams mp;
-    mp.groups = reinterpret_cast<const DevMerge*>(base + o_merge); mp.reqs = dp.reqs; mp.items = dp.items; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = static_cast<int32_t>(m.merge.size());
+    mp.groups = reinterpret_cast<const DevMerge*>(base + o_merge); mp.reqs = reinterpret_cast<const DevReq*>(base + o_reqs); mp.items = dp.items; mp.per_context = 0; mp.nodes = nullptr; mp.n_groups = static_cast<int32_t>(m.merge.size());
     mp.rows_per_slot = G; mp.tokens_per_block = 1; mp.ws_o = ws_o; mp.ws_ml = ws_ml; mp.out = rows_desc(*out); mp.lse_out = lse;
     mp.ws_o_ctx = ws_o; mp.ws_ml_ctx = ws_ml; mp.rows_per_slot_ctx = G;
     mp.part_o_ctx = nullptr; mp.part_lse_ctx = nullptr; mp.part_o_oth = nullptr; mp.part_lse_oth = nullptr;

@@ -99,8 +99,6 @@ __device__ __forceinline__ void cluster_copy(uint32_t dst, uint32_t src, uint32_
                  ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-constexpr int kMaxCluster = 16;
-
 // One warp merges one row of a cluster whose blocks have each sent at most one partial of it to this block: those of blocks
 // [0, n_ctx) belong to the context, those of the n_oth behind them do not.  ml[j]: (m, l) of block j's partial; o + j * stride: this
 // lane's VEC elements of it.

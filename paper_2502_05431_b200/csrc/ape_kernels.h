@@ -31,8 +31,7 @@ struct RowsOut {
 struct DecodeParams {
     const DevTile* tiles;
     const DevItem* items;
-    const int32_t* cta_item_begin;   // [n_cta + 1]
-    const DevReq* reqs;
+    const int32_t* cta_item_begin;   // [n_cta + 1] (cluster form: block b works on item b)
     RowsDesc q;
     float* ws_o;                     // [n_slots][G][D]  unnormalised partial outputs
     float* ws_ml;                    // [n_slots][G][2]  running maximum (base-2 logits) and sum
@@ -73,8 +72,7 @@ enum : int32_t {
 struct AttnParams {
     const DevTile* tiles;
     const DevItem* items;
-    const int32_t* cta_item_begin;   // [n_groups + 1]; CTA b serves group b / n_sib as sibling b % n_sib
-    const DevReq* reqs;
+    const int32_t* cta_item_begin;   // [n_groups + 1]; CTA b serves group b / n_sib as sibling b % n_sib (kAttnShort: works on item b)
     RowsDesc out;                    // SEG_FINAL items write here
     float* lse_out;                  // nullable, [rows, H_q] natural-log LSE for SEG_FINAL items
     float* ws_o;                     // [n_slots][kAttnRows][D]
@@ -84,7 +82,6 @@ struct AttnParams {
     int32_t G;
     int32_t H_q;
     int32_t n_sib;                   // sibling CTAs per group (row blocks that stream the same tiles together)
-    int32_t q_rows_are_pool;         // encode: Q / O rows are pool tokens (row = context start + i)
     int32_t split_r;                 // rows of a TILE_SPLIT tile that come from the prefix (a multiple of 8; 0: no such tiles)
     int32_t o_via_tma;               // two-buffer plans whose items all have their own Q: full halves of O leave through shared
                                      // memory (the item's Q buffer) and a bulk tensor store described by tm_o
