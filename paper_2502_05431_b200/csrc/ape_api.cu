@@ -249,10 +249,11 @@ struct Run {   // a run of tiles of one segment for one (request, kv head, row-b
 // (One request over 10 x 256 tokens, eight heads x (40 + 3) tiles on 148 blocks: 9.25 us per step with blocks of 3 tiles of
 // which some held two items, 8.02 this way; 16 requests over shared 128K tokens: 121.6 and 119.2.)
 // Otherwise the bins get equal shares of tiles and items' ends together, so that no bin is the last one for its many items.  Equal shares
-// of tiles alone / this way, us: prefill, 4 x 128 rows over 20 documents 199 / 191, 256 rows over 500 x 256 tokens 533 / 525, 2 x 229 rows
-// over 71 contexts of 158 to 474 tokens (8 KV heads) 73.8 / 63.2, 4 x 125 rows over 181 short ones 42.7 / 36.1; decode, 3 requests over 7
-// contexts of 206 to 618 tokens 10.4 / 9.5, per-context form, 5 over 45 of 154 to 463 21.5 / 20.3.  Of 27 such drawn calls one was slower
-// (15.9 / 16.2).  Not in decode plans whose runs have more than kLongRun tiles on average: there an end is hidden behind the stream of the other
+// of tiles alone / this way, us per call, 32 / 8 heads: prefill, 4 x 128 rows over 20 documents of 512 to 1,536 tokens 199.6 / 196.6, 2 x 229 rows
+// over 71 contexts of 158 to 474 212.4 / 207.7, 4 x 125 rows over 181 of 16 to 48 75.6 / 72.5; two passes, 64 rows over a tree of 85 x 84 tokens
+// 58.3 / 50.9; per-context decode step of 5 requests over 45 contexts of 154 to 463 73.0 / 72.4.  256 rows over 500 x 256 tokens, Eq. 5 and per
+// context: no difference (542 / 540, 914 / 912).  Of 27 drawn calls in a graph of calls, 0.85 to 1.02 times as long, one was slower (15.9 / 16.2).
+// Not in decode plans whose runs have more than kLongRun tiles on average: there an end is hidden behind the stream of the other
 // blocks and only the bytes count (4 requests over 61 contexts of 126 tokens, 65 tiles a run, 24.6 / 25.1).
 void assign_stream(const std::vector<Run>& runs, int n_bins, int slot_mult, int item_tiles, HostMeta& m, bool align_nodes = false, bool weigh_ends = true) {
     long long total = 0;
@@ -824,13 +825,13 @@ static int attend_plan_impl(ape_handle_t h, const ape_shape_t* shape, const ape_
             p->smem_bytes = attn_smem_bytes(D, kAttnPrefill);
             if (per_context == 0) {
                 // The cluster form: row blocks of 128 rows, whose two halves take alternate tiles, so that a block may have twice the tiles of
-                // the ordinary form's largest in about the same time, a little less for long ones (16 tiles against 31: 38.3 / 32.0 us).
-                // Ordinary / cluster, us per call: 4 x 64 tokens 8.0 / 6.4, 64 rows over 10 contexts of 256 16.6 / 13.0, 2 x 16 rows over
-                // 10 contexts 16.5 / 11.7, 4 x 5 rows over 24 contexts of 284 38.3 / 32.1.
+                // the ordinary form's largest in about the same time, a little less for long ones (16 tiles against 31: 40.0 / 33.4 us).
+                // Ordinary / cluster, us per call: 4 x 64 tokens 8.4 / 6.5, 64 rows over 10 contexts of 256 17.2 / 13.7, 2 x 16 rows over
+                // 10 contexts 17.2 / 12.5, 4 x 5 rows over 24 contexts of 284 40.0 / 33.4.  (In a graph of calls on the same inputs 0.2 to 2 less.)
                 // With few row blocks the ordinary form has few rows to merge and leaves more of the chip to the tiles.  So clusters of more than
                 // six blocks only where the partials and the rows of a row block stay below a line that rises with the number of row blocks;
                 // else at most six blocks, all of one tile when there are fewer than four row blocks.  The line was drawn when the merge read the other
-                // blocks' rows; since they are sent it errs to the ordinary form: of 40 calls that it decides, 33 would be faster in clusters (one KV
+                // blocks' rows; since they are sent it errs to the ordinary form: of 40 calls that it decides, 33 would be faster in clusters (in a graph of calls, one KV
                 // head, 3 x 2 rows over 33 contexts 15.8 / 11.6; 8 / 2 heads of 64, 3 x 24 rows over 38 contexts 15.3 / 10.7), one slower
                 // (10.1 / 10.6).  What it gives the cluster form is faster there: of 149 calls three were slower, by at most 3%.
                 const int TS = kAttnRows / 2 / G;

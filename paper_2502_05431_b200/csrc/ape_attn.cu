@@ -202,7 +202,7 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const uint32_t tmem_base = tmem_base_smem;
 
     // (SHORT: block b works on item b.  A range read in front of it is 700 cycles more between two calls, where the second one's clusters
-    // cannot be placed before the first one has left its SMs: 64 rows over 10 x 256 tokens 13.7 us, now 12.95)
+    // cannot be placed before the first one has left its SMs: 64 rows over 10 x 256 tokens 14.3 us per call, 13.7 without it)
     const int n_sib = SHORT ? 1 : p.n_sib;
     const int group = blockIdx.x / n_sib, sib = blockIdx.x - group * n_sib;
     const int item_begin = SHORT ? group : p.cta_item_begin[group], item_end = SHORT ? group + 1 : p.cta_item_begin[group + 1];
@@ -808,7 +808,8 @@ ape_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // them, a bulk copy each, counted in bytes on a barrier there: a block waits for its own rows only and merges them from its own
             // shared memory.  Bound by latency and by what the SMs exchange (56 KB in and out per block of a cluster of six, about 2,000
             // cycles).  Reading the others' rows behind a barrier of the cluster, three blocks at a time, and a second barrier before a block
-            // may leave took 7,600 of the 28,000 cycles of 64 rows over 10 x 256 tokens: 14.4 us, now 13.7; 4 x 64 tokens 6.9, now 6.5.
+            // may leave took 7,600 of the 28,000 cycles of 64 rows over 10 x 256 tokens.  Per call, both before the records were found by the
+            // block's index: 15.1 us that way, 14.3 with rows that are sent; 4 x 64 tokens 7.2 and 6.6.
             // Rows are fp32, 16-byte chunk j of row r at j ^ (r mod 8).  Q, K and V are free: every product and every copy is done.
             constexpr int kCols = D / 2;                            // columns that a half's threads combine
             constexpr int VEC = D / 8;                              // eight lanes merge a row

@@ -268,12 +268,12 @@ struct HeadsAsRows {
 // A long step is bound by HBM (16 requests over 128K tokens: 6.7 TB/s), a short one by a chain of latencies, in cycles for one request
 // over 10 x 256 tokens: wait for the kernel before -> first tile 1,500 (2,200 when the records and the copy engine's descriptors
 // are fetched behind that wait), 950 per tile of a warp, 750 for the partials of the eight warps (1,430 with a row's (m, l) read one by
-// one and rows 128 floats apart), then the merge.  All of them together: 7.4 us per call, now 6.3 in two kernels.
+// one and rows 128 floats apart), then the merge.  All of them together, in two kernels: 7.4 us per call, then 6.3 to 6.5.
 //
 // CLUSTER: the blocks of a thread-block cluster share the tiles of one (request, KV head), one item each, and merge their partials
 // themselves: each block sends the rows of its partial to the blocks that merge them (distributed shared memory, one barrier of the
 // cluster), so that a short step is one kernel, no partial goes to memory and no second kernel waits for the last block of the
-// first: 5.8 us for the step above, 3.7 instead of 5.1 for a single context of 64 tokens.  (Sent, not fetched: reading the others'
+// first: 5.9 us for the step above, and in a graph of calls 3.6 instead of 4.7 for a single context of 64 tokens.  (Sent, not fetched: reading the others'
 // partials behind the barrier cost another 1,600 cycles and a second barrier before a block may leave.)
 template <int D, bool CLUSTER, typename Products>
 __global__ void __launch_bounds__(kThreads, 1)

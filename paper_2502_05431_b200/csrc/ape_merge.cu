@@ -4,7 +4,7 @@
 //      LSE = logsumexp_s(m_s + log2 l_s),  O = sum_s 2^(LSE_s - LSE) O_s;
 //   2. the context log-sum-exp is multiplied by the scaling factor S and the two segments are merged by a
 //      softmax over [S * LSE_C, LSE_other] (Eq. 5; appendix "Efficient Implementation").
-// One or eight warps per output row (query token, query head); lanes cover the head dimension.
+// An output row (query token, query head) belongs to one warp, to eight or to eight lanes of one; lanes cover the head dimension.
 #include "ape_common.cuh"
 #include "ape_finish.cuh"
 #include "ape_kernels.h"
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256, 4) ape_merge_kernel(const MergeParams p)
             const size_t step = static_cast<size_t>(stride) * per_slot;        // rows between consecutive partials
             if (W > 1 && n <= W) {
                 // at most a partial per warp: it is the warp's result as it is, without the shuffles of two segments (2 requests' decode step
-                // over 20 x 256 tokens 9.3 us, now 8.6)
+                // over 20 x 256 tokens 13.2 us per call, 12.6 this way; on inputs that stay in L2 9.3 and 8.6)
                 if (part < n) {
                     const float2 ml = *reinterpret_cast<const float2*>(ws_ml + (row0 + part * step) * 2);
                     const float* a = ws_o + (row0 + part * step) * D + lane * VEC;
@@ -643,9 +643,9 @@ cudaError_t launch_merge_vec(const MergeParams& p, long long rows, cudaStream_t 
     // and sharing a row only adds the meeting in shared memory (64 rows over 10 x 256 tokens, 2048 rows to merge: 19.4 us with
     // one, 24.4 with eight; 4 x 128 rows over 20K tokens: 212 and 254).
     // With more rows than fit on the device at once that way (four blocks of eight to an SM) and few partials a segment (most prefills: the
-    // runs of a head span few blocks), eight lanes take a row.  64 rows over 30 x 256 tokens, 2 / 3 / 4 requests (4,096 / 6,144 / 8,192
-    // rows to merge): 28.9 / 42.6 / 52.6 us per call with a warp per row, 29.5 / 40.3 / 49.3 this way; 4 x 128 rows over 20 documents 203
-    // and 198; a tree's 3,072 rows 54.8 and 55.8.
+    // runs of a head span few blocks), eight lanes take a row.  64 rows over 30 x 256 tokens, 3 / 4 requests (6,144 / 8,192 rows to merge):
+    // 43.2 / 53.5 us per call with a warp per row, 41.2 / 50.9 this way; 2 x 256 rows over 20 x 256 tokens 68.3 and 64.2; 4 x 128 rows over 20
+    // documents 200.7 and 196.7.  Below the line, 2 requests (4,096 rows) 28.9 and 29.5, a tree's 3,072 rows 54.8 and 55.8.
     if (rows > 32ll * p.n_sm && p.max_partials <= kRowPartials)
         return launch_pdl(ape_merge_rows_kernel<VEC * 4>, static_cast<unsigned>((rows + 15) / 16), 128, 0, stream, p);
     if (rows <= 4ll * p.n_sm) return launch_pdl(ape_merge_kernel<VEC, 8>, static_cast<unsigned>(rows), 256, 0, stream, p);
