@@ -65,10 +65,10 @@ def decode_bytes(n_req: int, tokens_per_req: int) -> float:
 # cached tokens).  Valid only for the kernel sources the counters were taken with: the figure is dropped (null) as
 # soon as the hash of those sources changes.
 NCU_TRAFFIC = {
-    "prefill": {"bytes": 2 * (266.90e6 + 10.46e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "40056cbcae4a4560"},
-    "encode": {"bytes": 2 * (790.78e6 + 484.33e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_finish.cuh"], "sha": "40056cbcae4a4560"},
-    "decode": {"bytes": (1.05511e9 + 3.41e6) * (8409907200.0 / 1053835264.0), "sources": ["ape_decode.cu", "ape_common.cuh", "ape_finish.cuh"], "sha": "d858d51375fd8e0f"},
-    "rope": {"bytes": 2 * ((131.28e6 + 84.20e6) + (131.28e6 + 78.17e6) + (524.91e6 + 476.13e6)), "sources": ["ape_rope.cu", "ape_common.cuh"], "sha": "50dd0f0ff777a3a3"},
+    "prefill": {"bytes": 2 * (266.90e6 + 12.76e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_wait.h", "ape_finish.cuh"], "sha": "4755f83f46918caf"},
+    "encode": {"bytes": 2 * (789.41e6 + 484.03e6), "sources": ["ape_attn.cu", "ape_tcgen05.cuh", "ape_common.cuh", "ape_wait.h", "ape_finish.cuh"], "sha": "4755f83f46918caf"},
+    "decode": {"bytes": (1.05505e9 + 4.18e6) * (8409907200.0 / 1053835264.0), "sources": ["ape_decode.cu", "ape_common.cuh", "ape_wait.h", "ape_finish.cuh"], "sha": "04f3f5831626f80d"},
+    "rope": {"bytes": 2 * ((131.28e6 + 83.92e6) + (131.29e6 + 78.45e6) + (524.94e6 + 475.41e6)), "sources": ["ape_rope.cu", "ape_common.cuh", "ape_wait.h"], "sha": "43851ffa15e32695"},
 }
 
 

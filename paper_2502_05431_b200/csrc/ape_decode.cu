@@ -61,7 +61,7 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
 //
 // HeadsAsColumns, at most eight heads: S^T = K Q^T and O^T = V^T P^T, so the tokens (or the elements of a head) are the 16 rows of an mma
 // and the heads its 8 columns, half the products that 16 rows for the heads take (of which four heads use a quarter).  A step that is not
-// bound by HBM is bound by these chains: 4 requests over 4 x 256 tokens 6.05 -> 5.74 us, 8 over 50 x 256 tokens (two KV heads of 64)
+// bound by HBM is bound by these chains, in a graph of calls: 4 requests over 4 x 256 tokens 6.05 -> 5.74 us, 8 over 50 x 256 tokens (two KV heads of 64)
 // 13.4 -> 12.5, 4 over 100 x 256 (eight KV heads of one query head) 69.9 -> 68.2; 16 over 500 x 256, at the HBM rate, as before.
 // HeadsAsRows, 16 heads: O = P V with the heads as the rows.  As columns they are two groups, so as many products, and the maxima over the
 // tokens take three shuffles a head instead of two: 4 requests over 30 x 256 tokens 8.5 us, as columns 8.9.

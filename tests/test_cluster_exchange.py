@@ -48,8 +48,8 @@ int main() {
 
 
 def test_no_block_leaves_before_what_is_sent_to_it_has_landed(tmp_path):
-    """Also a block whose waits have run out is sent its rows, by blocks that come to it later: it waits for them, longer than any of their own waits
-    can last, and for ever only in no case.  And its sends depend on nothing that an abort changes: the others count on them."""
+    """A block whose waits have run out is sent its rows, too, perhaps by blocks that come to it later: it waits for them longer than any of their own
+    waits can last, but not for ever.  And its sends depend on nothing that an abort changes: the others count on them."""
     src = tmp_path / "two_blocks.cpp"
     src.write_text(_TWO_BLOCKS)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(tmp_path / "two_blocks")], check=True)
